@@ -21,9 +21,9 @@
  * Streams: `stream` is a cudaStream_t (NULL = the legacy default stream).  All
  * of a call's device work is issued on that stream, after the work the caller
  * queued on it before the call.  A call returns once its results are written:
- * the Borůvka round loop and the Filter-Borůvka recursion are steered by
- * counts (list lengths, active components) that the host reads back on that
- * stream, so a solve is stream-ordered but not asynchronous to the host.  A
+ * the Filter-Borůvka recursion is planned from a count that the host reads
+ * back on that stream, and the final status is read back, so a solve is
+ * stream-ordered but not asynchronous to the host.  A
  * handle must not be used by two host threads at once; different handles may
  * solve at the same time from different threads (each on its own stream): a
  * solve grows its buffers in stream order and never waits for the whole
@@ -78,12 +78,12 @@ typedef struct {
                                   edges (<= 6144) fit one block's shared memory, finish its rounds in
                                   one launch (the role of the paper's base case, Section 4.4); 0: run
                                   every round globally */
-  int graph_rounds;            /* 1 (default): from the second round of a Borůvka call on, run the
-                                  rounds as one CUDA graph launch whose conditional loop the device
-                                  ends (no host round trip per round); 0: one host readback per round */
-  int graph_jump_launches;     /* pointer-jumping launches per round inside the graph, 1..8, of up to
-                                  256 parent steps each (default 2: chains up to 256^2); a round that
-                                  needs more hands the state back to the host, which finishes the jump */
+  int graph_rounds;            /* 1 (default): the rounds of a Borůvka call run in one cooperative launch
+                                  that the device ends (no host round trip per round; not with hash or
+                                  sort dedupe, nor for n >= 2^31); 0: one host readback per round */
+  int graph_jump_launches;     /* 1..8 (default 2); kept for callers that set it, without effect: the
+                                  one-launch rounds repeat their jump passes of 256 parent steps on the
+                                  device until every vertex has its root */
   int filter_carry;            /* Filter-Borůvka: 1 hands a level's filtered heavy edges, when at most
                                   n/8, back to the level above instead of solving them there (Section
                                   6.3); 0 (default, measured faster on GB300): every level solves its own */
@@ -111,16 +111,16 @@ typedef struct {
                                   block handles block_threads x items_per_thread per tile.  Both are
                                   autotuner choices; every shape computes the same forest */
   int filter_plan;             /* Filter-Borůvka (Alg. 2) with the default filter options (no carry, one
-                                  filter pass, CUDA-graph rounds, no dedupe, no local contraction):
+                                  filter pass, one-launch rounds, no dedupe, no local contraction):
                                   1 (default): after the top-level partition, the host plans the
                                   remaining recursion levels and list capacities from its light count
                                   and queues every level without reading counts back (lengths stay in
-                                  device memory; Borůvka rounds run as device-ended graph loops); the
-                                  call reads back twice.  If a list outgrows its planned capacity or a
-                                  round needs the host, the call starts over on the host-driven path
-                                  (same result).  0: the host reads every level's counts */
-  uint32_t relabel_block_threads;    /* threads per block of the relabel compaction, which runs in every
-                                        Borůvka round, mostly on short lists: 128, 256 or 512; both
+                                  device memory; each Borůvka call's rounds run in one launch); the
+                                  call reads back twice.  If a list outgrows its planned capacity, the
+                                  call starts over on the host-driven path (same result).  0: the host
+                                  reads every level's counts */
+  uint32_t relabel_block_threads;    /* threads per block of the relabel compaction of host-driven rounds
+                                        (the one-launch rounds have their own): 128, 256 or 512; both
                                         relabel fields 0: 128 x 4, measured fastest on GB300 (more,
                                         smaller tiles spread a short list over more SMs) */
   uint32_t relabel_items_per_thread; /* edges per thread of the relabel compaction: 4, 8 or 16 */
@@ -245,7 +245,7 @@ enum {
   MST_K_FINALIZE,       /* bitmap -> ascending ids + weight */
   MST_K_TILE,           /* tile-local contraction (count, bucket, contract) */
   MST_K_BASE,           /* single-block base case (the last rounds of a Borůvka call) */
-  MST_K_GRAPH,          /* Borůvka rounds run as one CUDA graph launch (time only; bytes not counted) */
+  MST_K_GRAPH,          /* Borůvka rounds run as one launch (time only; bytes not counted) */
   MST_K_COUNT
 };
 typedef struct {

@@ -1,0 +1,81 @@
+// Device helpers shared by the kernel files: memory-order loads and stores, the
+// edge and relaxation keys, the block-wide scan and the weight counters.
+#pragma once
+#include "internal.h"
+
+namespace mstgpu {
+
+__device__ __forceinline__ u64 ld_relaxed(const u64 *p) {
+  u64 v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_relaxed(u64 *p, u64 v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+__device__ __forceinline__ u64 edge_key(uint32_t w, uint32_t id) { return ((u64)w << 32) | (u64)id; }
+
+// Relaxation key of an edge as seen from one end (see KeyLayout).
+__device__ __forceinline__ u64 relax_key(const KeyLayout &kl, uint32_t w, uint32_t id, uint32_t other) {
+  return kl.packed ? (((u64)w << (kl.idbits + kl.vbits)) | ((u64)id << kl.vbits) | (u64)other) : edge_key(w, id);
+}
+__device__ __forceinline__ uint32_t key_edge_id(const KeyLayout &kl, u64 key) {
+  return kl.packed ? (uint32_t)((key >> kl.vbits) & ((1ULL << kl.idbits) - 1)) : (uint32_t)key;
+}
+// The layout with `packed` decided on the device: where the largest weight
+// *max_w leaves room for the id and the far end (max_w == nullptr: kl as is).
+__device__ __forceinline__ KeyLayout resolve_layout(KeyLayout kl, const uint32_t *max_w) {
+  if (max_w) {
+    const uint32_t mw = __ldcg(max_w);
+    kl.packed = (mw ? 32 - __clz(mw) : 0) + kl.idbits + kl.vbits <= 63;
+  }
+  return kl;
+}
+// Do two keys name the same edge (the 2-cycle test)?
+__device__ __forceinline__ bool same_edge(const KeyLayout &kl, u64 a, u64 b) {
+  return kl.packed ? (a >> kl.vbits) == (b >> kl.vbits) : a == b;
+}
+
+// Exclusive block-wide scan of one uint32 per thread (B threads; s_warp holds
+// B / 32 + 1 words).
+template <int B = 256>
+__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t &total, uint32_t *s_warp) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t incl = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) s_warp[wid] = incl;
+  __syncthreads();
+  if (wid == 0) {
+    const uint32_t wv = lane < B / 32 ? s_warp[lane] : 0u;
+    uint32_t wi = wv;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
+      if (lane >= o) wi += y;
+    }
+    if (lane < B / 32) s_warp[lane] = wi - wv;
+    if (lane == B / 32 - 1) s_warp[B / 32] = wi;
+  }
+  __syncthreads();
+  total = s_warp[B / 32];
+  return s_warp[wid] + incl - x;
+}
+
+// Adds this thread's sum of chosen weights into a spread counter: one atomic
+// per warp (all 32 lanes call together).
+__device__ __forceinline__ void wsum_add(u64 *wsum, u64 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (wsum && (threadIdx.x & 31) == 0 && v)
+    atomicAdd(reinterpret_cast<unsigned long long *>(wsum) +
+                  ((blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) & (WSUM_SLOTS - 1)),
+              (unsigned long long)v);
+}
+
+}  // namespace mstgpu

@@ -18,7 +18,6 @@ enum : uint32_t {
   ERR_TMA = 16u,      // a bulk copy never completed (bounded mbarrier wait ran out); tiles were skipped
   ERR_TABLE = 32u,    // a batched size table is inconsistent (offsets not starting at 0 or decreasing)
   ERR_OVERFLOW = 64u, // a compaction's survivors exceeded its output capacity (nothing past it was written)
-  ERR_HANDBACK = 128u,  // device-driven rounds met a case that needs the host (long jump chain, round bound)
 };
 
 // Small per-handle device state.
@@ -165,8 +164,9 @@ constexpr int WSUM_SLOTS = 256;
 // ---- launchers (kernels.cu); all asynchronous on `s` ----
 int max_scan_tiles(uint64_t count);
 void launch_compact(CompactMode mode, const CompactArgs &a, uint64_t max_count, cudaStream_t s);
+// max_w: as in RoundsArgs.
 void launch_min_edges(EdgeList in, uint64_t m, uint32_t n, int validate, KeyLayout kl, u64 *best, uint32_t *err,
-                      int sms, cudaStream_t s);
+                      int sms, cudaStream_t s, const uint32_t *max_w = nullptr);
 void launch_max_weight(const uint32_t *w, uint64_t m, uint32_t *out, int sms, cudaStream_t s);
 void launch_hook(const HookArgs &a, uint64_t max_cand, cudaStream_t s);
 // max_steps: parent steps per thread and launch (0: the default of 64).
@@ -234,29 +234,45 @@ size_t min_edges_sort_scratch_bytes(uint64_t m, int sms);
 bool launch_min_edges_sort(EdgeList E, uint64_t m, uint32_t n, int validate, KeyLayout kl, u64 *best, uint32_t *err,
                            void *scratch, int sms, cudaStream_t s);
 
-// Borůvka rounds as a CUDA graph (device-driven loop): state in device memory.
-enum : uint32_t { ROUNDS_RUNNING = 0xff, ROUNDS_DONE = 0, ROUNDS_BASE = 1, ROUNDS_JUMP = 2, ROUNDS_BOUND = 3 };
-struct GraphRounds {
-  u64 ce[2];      // edges in the list of slot 0 / 1
-  u64 ca[2];      // active vertices of slot 0 / 1
-  u64 saved_ce, saved_ca;  // counts of the slot handed back to the host
-  uint32_t jflag; // the round's last jump launch left a vertex short of its root
-  uint32_t jdummy;  // flag word of the earlier jump launches (not read)
-  uint32_t iter;  // body executions (two rounds each)
-  uint32_t reason, slot;
+// The rounds of a Borůvka call in one cooperative launch (rounds.cu).
+constexpr int ROUNDS_MAX = 72;  // rounds of a call at most (components at least halve: 2 * (32 + 2) for 32-bit ids)
+struct RoundsState {            // zero before the launch
+  uint32_t bar;                 // grid barrier
+  uint32_t jflag[4];            // a jump pass left a vertex short of its root (rotating)
+  uint32_t levels;              // rounds run
+  u64 ca;                       // vertices of the call (with at least one edge)
+  u64 ce[ROUNDS_MAX], cv[ROUNDS_MAX];  // edges left after round r; components left with a root in round r
+  u64 off[ROUNDS_MAX + 1];      // offset of each round's part of link and rep
 };
-void launch_round_init(GraphRounds *g, uint64_t m, uint64_t n_act, cudaStream_t s);
-// The same from a device count of edges (at most cap); the active count is
-// zeroed for the hooking launch of the call's first round to fill.
-void launch_round_init_dev(GraphRounds *g, const u64 *m_dev, uint64_t cap, cudaStream_t s);
-// The graph's first node: enter the loop only with active vertices and edges
-// and a finished jump (else end it; a jump left short is ERR_HANDBACK in
-// *err_handback when that is given, the device-driven mode).
-void launch_round_pre(GraphRounds *g, cudaGraphConditionalHandle h, u64 *out_counts, uint32_t *err_handback,
-                      cudaStream_t s);
-void launch_round_check(GraphRounds *g, int base_ok, uint32_t *err_handback, cudaStream_t s);
-void launch_round_cond(GraphRounds *g, cudaGraphConditionalHandle h, int base_ok, uint32_t max_iter, u64 *out_counts,
-                       uint32_t *err_handback, cudaStream_t s);
+struct RoundsArgs {
+  EdgeList in;          // the call's list; ends are current representatives (plain ids < n)
+  uint64_t m;           // its length, or with m_dev its capacity
+  const u64 *m_dev;     // length in device memory (read as min(*m_dev, m)), or nullptr
+  EdgeOut list[2];      // ping-pong lists of the rounds, each with room for the whole list
+  int first_slot;       // the first round's output (in may be the other one)
+  int best_ready;       // best[] already holds the list's minEdges
+  int validate;         // check u, v < n in the first pass (without best_ready)
+  KeyLayout kl;         // with max_w only its bit widths count
+  const uint32_t *max_w;  // largest weight in device memory: packs the keys when they fit; or nullptr
+  u64 *best;            // [n] all KEY_INF but for a ready first round; all KEY_INF again afterwards
+  uint32_t *parent;     // [n] representatives; the call's vertices are updated if want_parent
+  uint32_t *link;       // [n] links of the rounds after the first
+  uint32_t *rep;        // [n] representatives of their components (want_parent)
+  uint32_t *act;        // [n] the call's vertices
+  int want_parent;
+  const uint32_t *src, *dst;  // ends by id of a list whose ends nothing recorded
+  uint32_t *cur_u, *cur_v;    // ends by id as last written (unpacked keys)
+  int ends_rec;         // cur_u, cur_v hold the list's ends
+  int record_first;     // record them in the first pass (a list with ids whose ends nothing recorded)
+  uint32_t *chosen_bits;
+  u64 *wsum;
+  uint32_t n, max_rounds;
+  RoundsState *st;
+  uint32_t *err;
+};
+// max_edges: bound on the list's length.  False if the launch was refused
+// (nothing ran).
+bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, int sms, cudaStream_t s);
 
 // single-block base case: the last rounds of a Borůvka call in one launch
 constexpr uint32_t BASE_MAX_N = 4096;  // live components (16-bit local ends; shared-memory vertex arrays)

@@ -19,6 +19,7 @@
 
 #include <cooperative_groups.h>
 
+#include "device.cuh"
 #include "internal.h"
 
 namespace mstgpu {
@@ -30,16 +31,6 @@ constexpr uint32_t JUMP_STEPS = 64;        // pointer steps per jump launch
 constexpr u64 PAIR_EMPTY = ~0ULL;
 
 // ------------------------------------------------------------------ helpers
-
-__device__ __forceinline__ u64 ld_relaxed(const u64 *p) {
-  u64 v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void st_relaxed(u64 *p, u64 v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
 
 // Striped item layout inside a tile of B * I items (B threads, I items each, I
 // a multiple of 4): item k of thread t sits at tile offset
@@ -76,20 +67,6 @@ __device__ __forceinline__ uint32_t local_pos(uint32_t keep, int k, uint32_t exc
   return (total_p & 0xffffu) + (excl_p >> 16) + (uint32_t)__popc((keep >> 4) & ((1u << (k - 4)) - 1u));
 }
 
-__device__ __forceinline__ u64 edge_key(uint32_t w, uint32_t id) { return ((u64)w << 32) | (u64)id; }
-
-// Relaxation key of an edge as seen from one end (see KeyLayout).
-__device__ __forceinline__ u64 relax_key(const KeyLayout &kl, uint32_t w, uint32_t id, uint32_t other) {
-  return kl.packed ? (((u64)w << (kl.idbits + kl.vbits)) | ((u64)id << kl.vbits) | (u64)other) : edge_key(w, id);
-}
-__device__ __forceinline__ uint32_t key_edge_id(const KeyLayout &kl, u64 key) {
-  return kl.packed ? (uint32_t)((key >> kl.vbits) & ((1ULL << kl.idbits) - 1)) : (uint32_t)key;
-}
-// Do two keys name the same edge (the 2-cycle test)?
-__device__ __forceinline__ bool same_edge(const KeyLayout &kl, u64 a, u64 b) {
-  return kl.packed ? (a >> kl.vbits) == (b >> kl.vbits) : a == b;
-}
-
 __device__ __forceinline__ bool aligned16_dev(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 __device__ __forceinline__ u64 pair_of(uint32_t a, uint32_t b) {
@@ -106,35 +83,6 @@ __device__ __forceinline__ u64 mix64(u64 z) {  // splitmix64 finaliser
 // (Steele, Lea, Flood, OOPSLA 2014).
 __device__ __forceinline__ u64 splitmix64_at(u64 state, u64 i) {
   return mix64(state + (i + 1ULL) * 0x9e3779b97f4a7c15ULL);
-}
-
-// Exclusive block-wide scan of one uint32 per thread (B threads; s_warp holds
-// B / 32 + 1 words).
-template <int B = BLOCK>
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t &total, uint32_t *s_warp) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t incl = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) s_warp[wid] = incl;
-  __syncthreads();
-  if (wid == 0) {
-    const uint32_t wv = lane < B / 32 ? s_warp[lane] : 0u;
-    uint32_t wi = wv;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += y;
-    }
-    if (lane < B / 32) s_warp[lane] = wi - wv;
-    if (lane == B / 32 - 1) s_warp[B / 32] = wi;
-  }
-  __syncthreads();
-  total = s_warp[B / 32];
-  return s_warp[wid] + incl - x;
 }
 
 // Decoupled look-back by the whole block.  Publishes the tile's aggregate,
@@ -1015,7 +963,9 @@ __global__ void __launch_bounds__(WS::threads, WS::minb) stream_warp_kernel(Comp
 // built by partition/filter): best[c] = min slot key over incident edges.
 template <bool VEC>
 __global__ void __launch_bounds__(BLOCK) min_edges_kernel(EdgeList in, uint64_t m, uint32_t n, int validate,
-                                                          KeyLayout kl, u64 *best, uint32_t *err) {
+                                                          KeyLayout kl, const uint32_t *max_w, u64 *best,
+                                                          uint32_t *err) {
+  kl = resolve_layout(kl, max_w);
   const uint64_t ntiles = (m + TILE - 1) / TILE;
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const uint64_t tb = tile * TILE;
@@ -1056,17 +1006,6 @@ __global__ void __launch_bounds__(BLOCK) min_edges_kernel(EdgeList in, uint64_t 
     }
     relax_pairs(best, eu, ev, key, keyb, mask);
   }
-}
-
-// Adds this thread's sum of chosen weights into a spread counter: one atomic
-// per warp (all 32 lanes call together).
-__device__ __forceinline__ void wsum_add(u64 *wsum, u64 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (wsum && (threadIdx.x & 31) == 0 && v)
-    atomicAdd(reinterpret_cast<unsigned long long *>(wsum) +
-                  ((blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) & (WSUM_SLOTS - 1)),
-              (unsigned long long)v);
 }
 
 // -------------------------------------------------------------------- hook
@@ -2388,128 +2327,6 @@ bool launch_min_edges_sort(EdgeList E, uint64_t m, uint32_t n, int validate, Key
   return true;
 }
 
-// ------------------------------------------------- device-driven round loop
-
-// State of the Borůvka rounds run as a CUDA graph: a conditional WHILE node
-// repeats a body of two rounds (lists and active lists alternate between slot
-// 0 and slot 1) while round_cond_kernel sets its condition.  Counts live here,
-// so no round waits for the host.
-__global__ void round_init_kernel(GraphRounds *g, uint64_t m, uint64_t n_act) {
-  g->ce[0] = m;
-  g->ca[0] = n_act;
-  g->ce[1] = g->ca[1] = 0;  // outputs of the first round
-  g->jflag = 0;
-  g->iter = 0;
-  g->reason = ROUNDS_RUNNING;
-  g->slot = 0;
-  g->saved_ce = g->saved_ca = 0;
-}
-
-// The same from a device count of edges; the active count is filled by the
-// hooking launch of the call's first round, which runs before the graph.
-__global__ void round_init_dev_kernel(GraphRounds *g, const u64 *m_dev, uint64_t cap) {
-  g->ce[0] = min((uint64_t)*m_dev, cap);
-  g->ca[0] = 0;
-  g->ce[1] = g->ca[1] = 0;
-  g->jflag = 0;
-  g->iter = 0;
-  g->reason = ROUNDS_RUNNING;
-  g->slot = 0;
-  g->saved_ce = g->saved_ca = 0;
-}
-
-// The graph's first node: run the loop only if there are active vertices and
-// edges and the jump before the graph reached the roots.  Otherwise end here
-// and publish the outcome as round_cond_kernel does.
-__global__ void round_pre_kernel(GraphRounds *g, cudaGraphConditionalHandle h, u64 *out_counts, uint32_t *err_handback) {
-  unsigned int go = 0;
-  if (g->jflag) {
-    g->reason = ROUNDS_JUMP;
-    if (err_handback) atomicOr(err_handback, ERR_HANDBACK);
-  } else if (g->ca[0] == 0 || g->ce[0] == 0) {
-    g->reason = ROUNDS_DONE;
-  } else {
-    go = 1;
-  }
-  if (!go) {
-    g->slot = 0;
-    g->saved_ce = g->ce[0];
-    g->saved_ca = g->ca[0];
-    out_counts[0] = g->saved_ce;
-    out_counts[1] = g->saved_ca;
-    out_counts[2] = (u64)g->reason;
-  }
-  g->jflag = 0;
-  cudaGraphSetConditional(h, go);
-}
-
-// After the first round of the body (slot 0 -> 1): stop early (the second
-// round then sees zero counts and does nothing) when the jump did not reach
-// the roots or the base case fits.
-__global__ void round_check_kernel(GraphRounds *g, int base_ok, uint32_t *err_handback) {
-  if (g->jflag || (base_ok && g->ca[1] > 0 && g->ca[1] <= BASE_MAX_N && g->ce[1] > 0 && g->ce[1] <= BASE_MAX_M)) {
-    if (g->jflag && err_handback) atomicOr(err_handback, ERR_HANDBACK);
-    g->reason = g->jflag ? ROUNDS_JUMP : ROUNDS_BASE;
-    g->slot = 1;
-    g->saved_ce = g->ce[1];
-    g->saved_ca = g->ca[1];
-    g->ce[1] = g->ca[1] = 0;
-  }
-  g->ce[0] = g->ca[0] = 0;  // outputs of the second round
-  g->jflag = 0;
-}
-
-// After the second round (slot 1 -> 0): decide whether the body runs again,
-// and publish the outcome in the solver's counters (edges, active, info).
-__global__ void round_cond_kernel(GraphRounds *g, cudaGraphConditionalHandle h, int base_ok, uint32_t max_iter,
-                                  u64 *out_counts, uint32_t *err_handback) {
-  const uint32_t it = ++g->iter;
-  unsigned int go = 0;
-  if (g->reason == ROUNDS_RUNNING) {
-    if (g->jflag) {
-      g->reason = ROUNDS_JUMP;
-    } else if (g->ca[0] == 0 || g->ce[0] == 0) {
-      g->reason = ROUNDS_DONE;
-    } else if (base_ok && g->ca[0] <= BASE_MAX_N && g->ce[0] <= BASE_MAX_M) {
-      g->reason = ROUNDS_BASE;
-    } else if (it >= max_iter) {
-      g->reason = ROUNDS_BOUND;
-    } else {
-      go = 1;
-    }
-    if (!go) {
-      g->slot = 0;
-      g->saved_ce = g->ce[0];
-      g->saved_ca = g->ca[0];
-      if (err_handback && (g->reason == ROUNDS_JUMP || g->reason == ROUNDS_BOUND)) atomicOr(err_handback, ERR_HANDBACK);
-    }
-  }
-  out_counts[0] = g->saved_ce;
-  out_counts[1] = g->saved_ca;
-  out_counts[2] = (u64)g->reason | ((u64)g->slot << 8) | ((u64)it << 16);
-  g->ce[1] = g->ca[1] = 0;  // outputs of the next body's first round
-  g->jflag = 0;
-  cudaGraphSetConditional(h, go);
-}
-
-void launch_round_init(GraphRounds *g, uint64_t m, uint64_t n_act, cudaStream_t s) {
-  round_init_kernel<<<1, 1, 0, s>>>(g, m, n_act);
-}
-void launch_round_init_dev(GraphRounds *g, const u64 *m_dev, uint64_t cap, cudaStream_t s) {
-  round_init_dev_kernel<<<1, 1, 0, s>>>(g, m_dev, cap);
-}
-void launch_round_pre(GraphRounds *g, cudaGraphConditionalHandle h, u64 *out_counts, uint32_t *err_handback,
-                      cudaStream_t s) {
-  round_pre_kernel<<<1, 1, 0, s>>>(g, h, out_counts, err_handback);
-}
-void launch_round_check(GraphRounds *g, int base_ok, uint32_t *err_handback, cudaStream_t s) {
-  round_check_kernel<<<1, 1, 0, s>>>(g, base_ok, err_handback);
-}
-void launch_round_cond(GraphRounds *g, cudaGraphConditionalHandle h, int base_ok, uint32_t max_iter, u64 *out_counts,
-                       uint32_t *err_handback, cudaStream_t s) {
-  round_cond_kernel<<<1, 1, 0, s>>>(g, h, base_ok, max_iter, out_counts, err_handback);
-}
-
 // ---------------------------------------------------- single-block base case
 
 // Once the live components and edges of a Borůvka call fit in one block's
@@ -2867,13 +2684,13 @@ void launch_compact(CompactMode mode, const CompactArgs &a, uint64_t max_count, 
 }
 
 void launch_min_edges(EdgeList in, uint64_t m, uint32_t n, int validate, KeyLayout kl, u64 *best, uint32_t *err,
-                      int sms, cudaStream_t s) {
+                      int sms, cudaStream_t s, const uint32_t *max_w) {
   if (m == 0) return;
   const unsigned grid = grid_for((m + (uint64_t)TILE - 1) / TILE, sms, 8);
   if (aligned16(in.u) && aligned16(in.v) && aligned16(in.w) && (!in.id || aligned16(in.id)))
-    min_edges_kernel<true><<<grid, BLOCK, 0, s>>>(in, m, n, validate, kl, best, err);
+    min_edges_kernel<true><<<grid, BLOCK, 0, s>>>(in, m, n, validate, kl, max_w, best, err);
   else
-    min_edges_kernel<false><<<grid, BLOCK, 0, s>>>(in, m, n, validate, kl, best, err);
+    min_edges_kernel<false><<<grid, BLOCK, 0, s>>>(in, m, n, validate, kl, max_w, best, err);
 }
 
 void launch_max_weight(const uint32_t *w, uint64_t m, uint32_t *out, int sms, cudaStream_t s) {

@@ -1,0 +1,583 @@
+// The Borůvka rounds of one call in a single persistent kernel.
+//
+// Every round (Section 2.3) is a few short passes over lists that shrink
+// quickly, so a round loop driven by the host, or by a CUDA graph's
+// conditional node, mostly waits between launches: on GB300 a graph iteration
+// of two rounds cost about 25 us before its first kernel, and a call about
+// 50 us more to enter the loop, against 5-30 us of work in a late round.  Here
+// all blocks of one cooperative launch stay resident and pass from phase to
+// phase through a grid barrier (about 1.5 us); once a list fits one block, the
+// other blocks leave and the last rounds run behind block barriers.
+//
+// Components are renumbered densely in every round: the roots that hooking
+// leaves get the ids 0..k-1 of the next round, so that later rounds read and
+// write compact, coalesced vertex arrays (no list of active vertices), and a
+// few components' minima fit a shared-memory table.
+#include <algorithm>
+#include <cstdint>
+
+#include "device.cuh"
+#include "internal.h"
+
+namespace mstgpu {
+
+namespace {
+
+constexpr int RB = 512;            // threads per block; two blocks per SM (64 registers)
+constexpr int RI = 4;              // edges per thread and tile of a long list
+constexpr int RT = RB * RI;        // edges per tile of a long list
+constexpr int RW = RB / 32;
+constexpr int HI = 16;             // vertices per thread and tile of a long hooking pass
+constexpr uint32_t ROOT = 0x80000000u;  // link entry: a root with its next-round id, or a resolved vertex
+constexpr uint32_t FIN = 0xffffffffu;   // link entry: component without edges left
+constexpr uint32_t RSTEPS = 256;        // parent steps per jump pass
+constexpr uint32_t RPASSES = 256;       // jump passes per round (each multiplies the reach)
+// Components up to which a round's minima are first collected in shared memory
+// per block.  With few components and many edges every block would send its
+// minima to the same few words: a GNM round (n=2^16, m=2^20) with 300
+// components left took 46 us, most of it those atomics queueing; 12 us with
+// the table.
+constexpr uint32_t STAB = 4096;
+// A call's last rounds run in one block from this size on.
+constexpr uint64_t SOLO_EDGES = 4096, SOLO_VERTS = 4096;
+constexpr uint32_t BAR_SPINS = 1u << 24;  // polls of the grid barrier before giving up
+
+struct Smem {
+  uint32_t out[4][RT];  // a tile's survivors (hooking: its vertices)
+  u64 tab[STAB];        // per-block minima of a round with few components
+};
+
+// All blocks of the launch are resident (cooperative launch), so a wait for
+// the others ends; it is bounded all the same.
+struct GridSync {
+  uint32_t nb, bid;  // blocks that take part, this block's number
+  uint32_t *bar, *err;
+  uint32_t target;
+  bool solo;
+  // False when the wait ran out (the error is latched; the kernel ends).
+  __device__ __forceinline__ bool sync() {
+    if (solo) {
+      __syncthreads();
+      return true;
+    }
+    int bad = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      target += nb;
+      __threadfence();
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+      uint32_t spins = 0;
+      for (;;) {
+        uint32_t v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+        if ((int32_t)(v - target) >= 0) break;
+        if (++spins >= BAR_SPINS) {
+          atomicOr(err, ERR_JUMP);
+          bad = 1;
+          break;
+        }
+      }
+      __threadfence();
+    }
+    return !__syncthreads_or(bad);
+  }
+};
+
+__device__ __forceinline__ bool aligned16_list(const EdgeList &l) {
+  return ((((uintptr_t)l.u | (uintptr_t)l.v | (uintptr_t)l.w | (uintptr_t)l.id) & 15u) == 0);
+}
+
+// best[x] = min(best[x], key): the current value first (it only falls, so a
+// stale copy costs an extra atomic at most).
+__device__ __forceinline__ void relax(u64 *best, uint32_t x, u64 key, u64 cur) {
+  if (key < cur) atomicMin(best + x, key);
+}
+
+// minEdges over the call's first list: vertex check, best[] of both ends, and
+// the ends by id where the hook will look them up and nothing recorded them.
+__device__ __forceinline__ void min_edges_phase(const RoundsArgs &a, KeyLayout kl, uint64_t m, uint32_t nb, uint32_t bid) {
+  const bool vec = aligned16_list(a.in);
+  const bool record = a.record_first && !kl.packed;
+  for (uint64_t tb = (uint64_t)bid * RT; tb < m; tb += (uint64_t)nb * RT) {
+    const uint64_t j0 = tb + 4 * threadIdx.x;
+    uint32_t eu[RI], ev[RI], ew[RI], ei[RI];
+    if (vec && tb + RT <= m) {
+      const uint4 x = __ldg(reinterpret_cast<const uint4 *>(a.in.u + j0));
+      const uint4 y = __ldg(reinterpret_cast<const uint4 *>(a.in.v + j0));
+      const uint4 z = __ldg(reinterpret_cast<const uint4 *>(a.in.w + j0));
+      eu[0] = x.x, eu[1] = x.y, eu[2] = x.z, eu[3] = x.w;
+      ev[0] = y.x, ev[1] = y.y, ev[2] = y.z, ev[3] = y.w;
+      ew[0] = z.x, ew[1] = z.y, ew[2] = z.z, ew[3] = z.w;
+      if (a.in.id) {
+        const uint4 t = __ldg(reinterpret_cast<const uint4 *>(a.in.id + j0));
+        ei[0] = t.x, ei[1] = t.y, ei[2] = t.z, ei[3] = t.w;
+      } else {
+#pragma unroll
+        for (int k = 0; k < RI; ++k) ei[k] = (uint32_t)(j0 + k);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < RI; ++k) {
+        const uint64_t j = j0 + k;
+        const bool in = j < m;
+        eu[k] = in ? a.in.u[j] : 0u;
+        ev[k] = in ? a.in.v[j] : 0u;
+        ew[k] = in ? a.in.w[j] : 0u;
+        ei[k] = in ? (a.in.id ? a.in.id[j] : (uint32_t)j) : 0u;
+      }
+    }
+    u64 cu[RI], cv[RI];
+    uint32_t ok = 0;
+#pragma unroll
+    for (int k = 0; k < RI; ++k) {
+      bool v = eu[k] != ev[k] && j0 + k < m;
+      if (a.validate && j0 + k < m && (eu[k] >= a.n || ev[k] >= a.n)) {
+        atomicOr(a.err, ERR_VERTEX);
+        v = false;
+      }
+      ok |= (v ? 1u : 0u) << k;
+      cu[k] = v ? __ldca(a.best + eu[k]) : 0ULL;
+      cv[k] = v ? __ldca(a.best + ev[k]) : 0ULL;
+    }
+#pragma unroll
+    for (int k = 0; k < RI; ++k) {
+      relax(a.best, eu[k], relax_key(kl, ew[k], ei[k], ev[k]), cu[k]);
+      relax(a.best, ev[k], relax_key(kl, ew[k], ei[k], eu[k]), cv[k]);
+      if (record && (ok >> k & 1)) {
+        a.cur_u[ei[k]] = eu[k];
+        a.cur_v[ei[k]] = ev[k];
+      }
+    }
+  }
+}
+
+// Hooking over the round's vertices 0..nc-1 (round 0: all vertices of the
+// call): a vertex with a minimum edge links to the edge's other end; of a
+// 2-cycle the smaller id stays root and takes the next free id of the next
+// round.  `link` gets the other end, or ROOT | next id; a component without
+// edges gets FIN (in round 0 its entry, a plain representative, is kept).
+// A tile of 512 * I vertices is first reduced to those with an edge, so that
+// the dependent gathers behind them run with full warps however sparse the
+// call is (a light list of RMAT n=2^24 touches 6% of the vertices).  Vertices
+// and the roots' new ids keep their order inside a tile: neighbouring ids of a
+// geometric graph stay neighbours in every round (ids out of order there made
+// the RGG2D n=2^22 first relabel 263 us instead of 213).
+template <int I>
+__device__ __forceinline__ void hook_phase(const RoundsArgs &a, const KeyLayout &kl, int r, uint64_t nc, uint64_t off,
+                                           bool rec, uint32_t nb, uint32_t bid, Smem &sm, uint32_t *s_warp,
+                                           uint32_t *s_base) {
+  static_assert(I * RB <= 4 * RT, "a tile's vertices fit the output stage");
+  uint32_t *link = r == 0 ? a.parent : a.link + off;
+  const uint32_t *rep = a.rep + off;
+  uint32_t *rep_next = a.rep + (r == 0 ? 0 : off + nc);
+  const uint32_t *eu = rec ? a.cur_u : a.src, *ev = rec ? a.cur_v : a.dst;
+  uint32_t *s_c = &sm.out[0][0];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t below = (1u << lane) - 1u;
+  u64 wacc = 0;
+  constexpr uint64_t T = (uint64_t)RB * I;
+  constexpr int C = I >= 4 ? 4 : I;  // vertices with an edge in flight per thread
+  const int wshift = kl.packed ? kl.idbits + kl.vbits : 32;
+  for (uint64_t tb = (uint64_t)bid * T; tb < nc; tb += (uint64_t)nb * T) {
+    // warp w reduces the tile's vertices [w * 32 I, (w + 1) * 32 I)
+    const uint64_t c0 = tb + (uint64_t)wid * (32 * I) + lane;
+    uint32_t act = 0, cnt = 0;
+#pragma unroll
+    for (int q = 0; q < I; ++q) act |= (c0 + 32 * q < nc && a.best[c0 + 32 * q] != KEY_INF ? 1u : 0u) << q;
+#pragma unroll
+    for (int q = 0; q < I; ++q) cnt += __popc(__ballot_sync(0xffffffffu, act >> q & 1));
+    uint32_t total;
+    uint32_t p = block_exclusive_scan<RB>(lane == 0 ? cnt : 0u, total, s_warp);
+    p = __shfl_sync(0xffffffffu, p, 0);
+    if (r == 0 && threadIdx.x == 0 && total) s_base[1] = (uint32_t)atomicAdd(&a.st->ca, (u64)total);
+#pragma unroll
+    for (int q = 0; q < I; ++q) {
+      const uint32_t b = __ballot_sync(0xffffffffu, act >> q & 1);
+      if (act >> q & 1)
+        s_c[p + __popc(b & below)] = (uint32_t)(c0 + 32 * q);
+      else if (r > 0 && c0 + 32 * q < nc)
+        link[c0 + 32 * q] = FIN;
+      p += __popc(b);
+    }
+    __syncthreads();
+    // warp w hooks the entries [w * per, (w + 1) * per) of the reduced tile
+    const uint32_t per = ((total + RW - 1) / RW + 31u) & ~31u;  // at most 32 I
+    const uint32_t lo = wid * per + lane, hi = min(total, (wid + 1) * per);
+    uint32_t roots = 0;
+#pragma unroll
+    for (int q = 0; q < I / C; ++q) {
+      if ((uint32_t)q * (32 * C) >= per) break;
+      uint32_t c[C], oth[C];
+      u64 kk[C];
+#pragma unroll
+      for (int k = 0; k < C; ++k) {
+        const uint32_t i = lo + (q * C + k) * 32;
+        c[k] = i < hi ? s_c[i] : 0u;
+        kk[k] = i < hi ? a.best[c[k]] : KEY_INF;
+        if (r == 0 && i < hi) a.act[s_base[1] + i] = c[k];
+      }
+#pragma unroll
+      for (int k = 0; k < C; ++k) {
+        oth[k] = 0;
+        if (kk[k] == KEY_INF) continue;
+        if (kl.packed) {
+          oth[k] = (uint32_t)(kk[k] & ((1ULL << kl.vbits) - 1));
+        } else {
+          const uint32_t e = (uint32_t)kk[k];
+          oth[k] = __ldca(eu + e) ^ __ldca(ev + e) ^ c[k];
+        }
+      }
+      u64 ob[C];
+#pragma unroll
+      for (int k = 0; k < C; ++k) ob[k] = kk[k] != KEY_INF ? a.best[oth[k]] : 0ULL;
+#pragma unroll
+      for (int k = 0; k < C; ++k) {
+        if (kk[k] == KEY_INF) continue;
+        if (same_edge(kl, ob[k], kk[k]) && c[k] < oth[k]) {
+          roots |= 1u << (q * C + k);
+        } else {
+          link[c[k]] = oth[k];
+          const uint32_t e = key_edge_id(kl, kk[k]);
+          atomicOr(a.chosen_bits + (e >> 5), 1u << (e & 31));
+          wacc += kk[k] >> wshift;
+        }
+      }
+    }
+    cnt = 0;
+#pragma unroll
+    for (int b = 0; b < I; ++b) cnt += __popc(__ballot_sync(0xffffffffu, roots >> b & 1));
+    uint32_t did = block_exclusive_scan<RB>(lane == 0 ? cnt : 0u, total, s_warp);
+    if (threadIdx.x == 0 && total) s_base[0] = (uint32_t)atomicAdd(&a.st->cv[r], (u64)total);
+    __syncthreads();
+    did = s_base[0] + __shfl_sync(0xffffffffu, did, 0);
+#pragma unroll
+    for (int b = 0; b < I; ++b) {
+      const uint32_t m = __ballot_sync(0xffffffffu, roots >> b & 1);
+      if (roots >> b & 1) {
+        const uint32_t c = s_c[lo + b * 32], d = did + __popc(m & below);
+        link[c] = ROOT | d;
+        if (a.want_parent) rep_next[d] = r == 0 ? c : rep[c];
+      }
+      did += __popc(m);
+    }
+    __syncthreads();  // s_c, s_warp and s_base are reused by the next tile
+  }
+  wsum_add(a.wsum, wacc);
+}
+
+// Pointer jumping (Section 4.2): every vertex that is not a root follows the
+// links to its root and takes the root's next-round id; best[] goes back to
+// INF.  Other threads' progress may be read on the way (an entry is either a
+// vertex nearer the root or the final id).  At most RSTEPS steps per pass.
+__device__ __forceinline__ void jump_phase(const RoundsArgs &a, int r, uint64_t cnt, uint64_t off, bool reset,
+                                        uint32_t *flag, uint32_t nb, uint32_t bid) {
+  uint32_t *link = r == 0 ? a.parent : a.link + off;
+  const uint64_t stride = (uint64_t)nb * RB;
+  bool left = false;
+  for (uint64_t i0 = (uint64_t)bid * RB + threadIdx.x; i0 < cnt; i0 += 4 * stride) {
+    uint32_t c[4], q[4], pend = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint64_t i = i0 + k * stride;
+      const bool in = i < cnt;
+      c[k] = in ? (r == 0 ? __ldca(a.act + i) : (uint32_t)i) : 0u;
+      q[k] = in ? __ldca(link + c[k]) : ROOT;
+      if (reset && in) a.best[c[k]] = KEY_INF;
+      pend |= (q[k] & ROOT ? 0u : 1u) << k;
+    }
+    const uint32_t moved = pend;
+    for (uint32_t s = 0; pend && s < RSTEPS; ++s) {
+      uint32_t t[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) t[k] = (pend >> k & 1) ? __ldca(link + q[k]) : 0u;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (pend >> k & 1) {
+          q[k] = t[k];
+          if (t[k] & ROOT) pend &= ~(1u << k);
+        }
+    }
+    left |= pend != 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (moved >> k & 1) __stcg(link + c[k], q[k]);
+  }
+  if (left) atomicOr(flag, 1u);
+}
+
+// Relabel, self-loop removal and compaction of the round's list, with the next
+// round's minEdges on the survivors (Section 4.3).  Tiles of 512 * I edges.
+// Survivors are staged in shared memory for coalesced stores; the minima are
+// relaxed from there, so that a warp's gathers have no idle lanes.  `tab`:
+// collect the minima in shared memory first.  A long list's tiles are bound by
+// the label and best[] gathers (four per edge, one L1 line each), so shared
+// memory is kept small for L1's sake: with the next tile copied ahead into a
+// shared-memory stage (160 KB per SM instead of 128) RMAT n=2^22 m=2^26 took
+// 4.36 ms per plain solve instead of 4.18; 192 KB: 4.53, 224 KB: 5.96.  One
+// block of 1024 threads per SM, or four of 256: 4.45, 4.58.
+template <int I>
+__device__ __forceinline__ void relabel_phase(const RoundsArgs &a, KeyLayout kl, int r, uint64_t m, uint64_t off,
+                                           bool tab, uint32_t nb, uint32_t bid, Smem &sm, uint32_t *s_warp,
+                                           uint32_t *s_base) {
+  const uint32_t *link = r == 0 ? a.parent : a.link + off;
+  const EdgeOut out = a.list[(a.first_slot + r) & 1], prev = a.list[(a.first_slot + r + 1) & 1];
+  const EdgeList in = r == 0 ? a.in : EdgeList{prev.u, prev.v, prev.w, prev.id};
+  u64 *counter = &a.st->ce[r];
+  constexpr uint64_t T = (uint64_t)RB * I;
+  const uint64_t nfull = I == RI && aligned16_list(in) ? m / T : 0;
+  for (uint64_t tile = bid; tile * T < m; tile += nb) {
+    const uint64_t j0 = tile * T + (uint64_t)I * threadIdx.x;
+    uint32_t eu[I], ev[I], ew[I], ei[I];
+    uint32_t valid = 0;
+    bool whole = false;
+    if constexpr (I == RI) {
+      if (tile < nfull) {
+        whole = true;
+        const uint4 x = __ldcg(reinterpret_cast<const uint4 *>(in.u + j0));
+        const uint4 y = __ldcg(reinterpret_cast<const uint4 *>(in.v + j0));
+        const uint4 z = __ldcg(reinterpret_cast<const uint4 *>(in.w + j0));
+        eu[0] = x.x, eu[1] = x.y, eu[2] = x.z, eu[3] = x.w;
+        ev[0] = y.x, ev[1] = y.y, ev[2] = y.z, ev[3] = y.w;
+        ew[0] = z.x, ew[1] = z.y, ew[2] = z.z, ew[3] = z.w;
+        if (in.id) {
+          const uint4 t = __ldcg(reinterpret_cast<const uint4 *>(in.id + j0));
+          ei[0] = t.x, ei[1] = t.y, ei[2] = t.z, ei[3] = t.w;
+        } else {
+#pragma unroll
+          for (int k = 0; k < I; ++k) ei[k] = (uint32_t)(j0 + k);
+        }
+        valid = (1u << I) - 1u;
+      }
+    }
+    if (!whole) {
+#pragma unroll
+      for (int k = 0; k < I; ++k) {
+        const bool ok = j0 + k < m;
+        eu[k] = ok ? __ldca(in.u + j0 + k) : 0u;
+        ev[k] = ok ? __ldca(in.v + j0 + k) : 0u;
+        ew[k] = ok ? __ldca(in.w + j0 + k) : 0u;
+        ei[k] = ok ? (in.id ? __ldca(in.id + j0 + k) : (uint32_t)(j0 + k)) : 0u;
+        valid |= (ok ? 1u : 0u) << k;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+      eu[k] = (valid >> k & 1) ? __ldca(link + eu[k]) & ~ROOT : 0u;
+      ev[k] = (valid >> k & 1) ? __ldca(link + ev[k]) & ~ROOT : 0u;
+    }
+    uint32_t keep = 0;
+#pragma unroll
+    for (int k = 0; k < I; ++k) keep |= (eu[k] != ev[k] ? 1u : 0u) << k;
+    uint32_t total;
+    uint32_t p = block_exclusive_scan<RB>((uint32_t)__popc(keep), total, s_warp);
+    if (threadIdx.x == 0) s_base[0] = total ? (uint32_t)atomicAdd(counter, (u64)total) : 0u;
+#pragma unroll
+    for (int k = 0; k < I; ++k)
+      if (keep >> k & 1) {
+        sm.out[0][p] = eu[k];
+        sm.out[1][p] = ev[k];
+        sm.out[2][p] = ew[k];
+        sm.out[3][p] = ei[k];
+        ++p;
+      }
+    __syncthreads();
+    const uint64_t ob = s_base[0];
+    constexpr int E = I > 2 ? 2 : I;  // survivors in flight per thread
+    for (uint32_t i0 = 0; i0 < total; i0 += E * RB) {
+      uint32_t x[E], y[E], id[E];
+      u64 kx[E], ky[E], cx[E], cy[E];
+#pragma unroll
+      for (int k = 0; k < E; ++k) {
+        const uint32_t i = i0 + k * RB + threadIdx.x;
+        kx[k] = ky[k] = KEY_INF;
+        cx[k] = cy[k] = 0;
+        x[k] = y[k] = id[k] = 0;
+        if (i < total) {
+          x[k] = sm.out[0][i], y[k] = sm.out[1][i], id[k] = sm.out[3][i];
+          const uint32_t w = sm.out[2][i];
+          kx[k] = relax_key(kl, w, id[k], y[k]);
+          ky[k] = relax_key(kl, w, id[k], x[k]);
+          cx[k] = tab ? sm.tab[x[k]] : __ldca(a.best + x[k]);
+          cy[k] = tab ? sm.tab[y[k]] : __ldca(a.best + y[k]);
+          out.u[ob + i] = x[k];
+          out.v[ob + i] = y[k];
+          out.w[ob + i] = w;
+          out.id[ob + i] = id[k];
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < E; ++k) {
+        if (tab) {
+          if (kx[k] < cx[k]) atomicMin(&sm.tab[x[k]], kx[k]);
+          if (ky[k] < cy[k]) atomicMin(&sm.tab[y[k]], ky[k]);
+        } else {
+          relax(a.best, x[k], kx[k], cx[k]);
+          relax(a.best, y[k], ky[k], cy[k]);
+        }
+        if (!kl.packed && kx[k] != KEY_INF) {
+          a.cur_u[id[k]] = x[k];
+          a.cur_v[id[k]] = y[k];
+        }
+      }
+    }
+    __syncthreads();  // the output stage, s_warp and s_base are reused by the next tile
+  }
+}
+
+// The call's vertices (act) back to representatives in the caller's numbering:
+// parent[v] = the representative of v's final component.
+__device__ __forceinline__ void compose_phase(const RoundsArgs &a, const uint64_t *s_off, int levels) {
+  const uint64_t cnt = a.st->ca;
+  for (uint64_t i = (uint64_t)blockIdx.x * RB + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * RB) {
+    const uint32_t v = __ldca(a.act + i);
+    uint32_t d = a.parent[v] & ~ROOT;
+    int l = 1;
+    for (; l < levels; ++l) {
+      const uint32_t q = __ldca(a.link + s_off[l] + d);
+      if (q == FIN) break;
+      d = q & ~ROOT;
+    }
+    a.parent[v] = __ldca(a.rep + s_off[l] + d);
+  }
+}
+
+__global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ RoundsArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_dyn[];
+  Smem &sm = *reinterpret_cast<Smem *>(smem_dyn);
+  __shared__ uint32_t s_warp[RW + 1], s_base[2];
+  // the round's edges, vertices, next round's vertices, vertices to jump, and each round's part of link and rep
+  __shared__ uint64_t s_m, s_nc, s_nn, s_cnt, s_off[ROUNDS_MAX + 2];
+  GridSync g{gridDim.x, blockIdx.x, &a.st->bar, a.err, 0, gridDim.x == 1};
+
+  const uint64_t m0 = a.m_dev ? min((uint64_t)*a.m_dev, a.m) : a.m;
+  const KeyLayout kl = resolve_layout(a.kl, a.max_w);
+  if (!a.best_ready) {
+    min_edges_phase(a, kl, m0, g.nb, g.bid);
+    if (!g.sync()) return;
+  }
+  if (*(volatile uint32_t *)a.err & (ERR_VERTEX | ERR_OVERFLOW)) return;  // the same in every block: set before the barrier
+
+  const bool rec0 = a.ends_rec || a.record_first;
+  if (threadIdx.x == 0) {
+    s_m = m0;
+    s_off[0] = 0;
+    s_off[1] = 0;
+    s_nc = a.n;
+  }
+  __syncthreads();
+  int r = 0;
+  uint32_t pass = 0;
+  bool ok = true, alone = false;
+  for (; s_m > 0 && s_nc > 0; ++r) {
+    if (r >= (int)a.max_rounds) {
+      if (threadIdx.x == 0) atomicOr(a.err, ERR_JUMP);
+      break;
+    }
+    if (s_nc >= (uint64_t)4 * RB * g.nb)
+      hook_phase<HI>(a, kl, r, s_nc, s_off[r], r > 0 || rec0, g.nb, g.bid, sm, s_warp, s_base);
+    else
+      hook_phase<1>(a, kl, r, s_nc, s_off[r], r > 0 || rec0, g.nb, g.bid, sm, s_warp, s_base);
+    if (!(ok = g.sync())) break;
+    if (threadIdx.x == 0) {  // components left with a root, vertices to jump
+      s_nn = __ldca(&a.st->cv[r]);
+      s_cnt = r == 0 ? __ldca(&a.st->ca) : s_nc;
+      if (r > 0) s_off[r + 1] = s_off[r] + s_nc;
+    }
+    __syncthreads();
+    if (s_nn == 0) {  // no vertex had an edge
+      ++r;
+      break;
+    }
+    for (uint32_t tries = 0;; ++tries, ++pass) {
+      uint32_t *flag = &a.st->jflag[pass & 3];
+      if (g.bid == 0 && threadIdx.x == 0) a.st->jflag[(pass + 2) & 3] = 0;
+      jump_phase(a, r, s_cnt, s_off[r], tries == 0, flag, g.nb, g.bid);
+      if (!(ok = g.sync()) || !__ldca(flag)) break;
+      if (tries >= RPASSES) {
+        if (threadIdx.x == 0) atomicOr(a.err, ERR_JUMP);
+        ok = false;
+        break;
+      }
+    }
+    ++pass;
+    if (!ok) break;
+    const bool tab = s_nn <= STAB;
+    if (tab) {
+      for (uint32_t i = threadIdx.x; i < (uint32_t)s_nn; i += RB) sm.tab[i] = KEY_INF;
+      __syncthreads();
+    }
+    if (s_m >= (uint64_t)RT * g.nb)
+      relabel_phase<RI>(a, kl, r, s_m, s_off[r], tab, g.nb, g.bid, sm, s_warp, s_base);
+    else
+      relabel_phase<1>(a, kl, r, s_m, s_off[r], tab, g.nb, g.bid, sm, s_warp, s_base);
+    if (tab) {  // one atomic per component and block at most
+      for (uint32_t i = threadIdx.x; i < (uint32_t)s_nn; i += RB) {
+        const u64 k = sm.tab[i];
+        if (k != KEY_INF) relax(a.best, i, k, __ldca(a.best + i));
+      }
+    }
+    if (!(ok = g.sync())) break;
+    if (threadIdx.x == 0) {
+      s_m = __ldca(&a.st->ce[r]);
+      s_nc = s_nn;
+    }
+    __syncthreads();
+    if (!g.solo && s_m > 0 && s_m <= SOLO_EDGES && s_nc <= SOLO_VERTS) {  // block 0 finishes alone
+      alone = true;
+      if (blockIdx.x != 0) break;
+      g.solo = true;
+      g.nb = 1;
+    }
+  }
+  if (!ok || !a.want_parent) return;
+  __syncthreads();
+  if (alone) {  // the other blocks come back for the last pass and learn the rounds they missed
+    if (blockIdx.x == 0) {
+      for (int i = threadIdx.x; i <= r; i += RB) a.st->off[i] = s_off[i];
+      if (threadIdx.x == 0) a.st->levels = (uint32_t)r;
+    }
+    g.solo = false;
+    g.nb = gridDim.x;
+    if (!g.sync()) return;
+    if (blockIdx.x != 0) {
+      r = (int)__ldcg(&a.st->levels);
+      for (int i = threadIdx.x; i <= r; i += RB) s_off[i] = __ldcg(&a.st->off[i]);
+    }
+    __syncthreads();
+  }
+  compose_phase(a, s_off, r);
+}
+
+}  // namespace
+
+bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, int sms, cudaStream_t s) {
+  // resident blocks per SM (0: not available); set once per process
+  static const int per_sm = []() -> int {
+    int b = 0;
+    if (cudaFuncSetAttribute(rounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, rounds_kernel, RB, sizeof(Smem)) != cudaSuccess)
+      b = 0;
+    cudaGetLastError();
+    return b < 2 ? b : 2;
+  }();
+  if (per_sm <= 0 || a.n >= ROOT) return false;
+  if (cudaMemsetAsync(a.st, 0, sizeof(RoundsState), s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  // as many blocks as the first round's tiles can use; a graph that fits one
+  // block's last rounds from the start needs no grid barrier at all
+  const uint64_t want = std::max(max_edges, (uint64_t)a.n) / RB + 1;
+  unsigned grid = (unsigned)std::min<uint64_t>(want, (uint64_t)sms * per_sm);
+  if (max_edges <= SOLO_EDGES && a.n <= SOLO_VERTS) grid = 1;
+  RoundsArgs arg = a;
+  void *args[] = {&arg};
+  if (cudaLaunchCooperativeKernel((const void *)rounds_kernel, dim3(grid), dim3(RB), args, sizeof(Smem), s) ==
+      cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
+}
+
+}  // namespace mstgpu

@@ -57,7 +57,6 @@ struct mst_ctx {
   };
   bool prof_on = false;
   uint32_t prof_mask = ~0u;  // classes that get event timing (the others: launches and bytes only)
-  cudaStream_t cap_stream = nullptr;  // stream the round graphs are captured on
   cudaStream_t copy_stream = nullptr; // input copies of mst_solve_host_many
   cudaEvent_t in_ready[2] = {nullptr, nullptr}, in_free[2] = {nullptr, nullptr};
   // device buffers of the host entry points (inputs, two sets; the forest),
@@ -68,19 +67,10 @@ struct mst_ctx {
   void *hout = nullptr;
   size_t hout_cap = 0;
   // the two ping-pong edge lists of the Borůvka rounds (u, v, w, id each),
-  // kept by the handle and grown on demand: with stable addresses and a stable
-  // capacity bound, one captured round graph serves every Borůvka call (and
-  // every later solve) of the handle
+  // kept by the handle and grown on demand
   void *rl_mem = nullptr;
   uint64_t rl_cap = 0;  // edges per list
-  GraphRounds *grounds = nullptr;     // device state of the graph round loop
-  struct RoundGraph {
-    u64 sig;  // every pointer and size the graph was built with
-    cudaGraph_t graph;
-    cudaGraphExec_t exec;
-  };
-  std::vector<RoundGraph> round_graphs;  // most recently used first
-  std::vector<u64> round_sigs_seen;      // shapes met once (a graph is built on the second meeting)
+  RoundsState *rstate = nullptr;  // device state of the one-launch rounds
   std::vector<cudaEvent_t> ev_pool;
   std::vector<ProfRec> prof_pending;
   mst_kernel_stats prof[MST_K_COUNT];
@@ -201,7 +191,7 @@ struct RoundList {
 // edges.  The growth is stream-ordered on s: the old lists are freed after the
 // work queued on s so far (calls return only after their work is done, so no
 // earlier call still reads them), and nothing waits for the whole device, which
-// other threads may be using (or capturing graphs on) at the same time.
+// other threads may be using at the same time.
 mst_status round_lists(mst_ctx *c, uint64_t need, RoundList &X, RoundList &Y, cudaStream_t s) {
   if (!c->rl_mem || c->rl_cap < need) {
     const uint64_t want = round_up(std::max<uint64_t>(need + need / 4, 1ULL << 16), 1ULL << 16);
@@ -464,7 +454,7 @@ struct Solve {
   cudaStream_t s;
   uint32_t n;
   uint64_t m;
-  Buf best_b, parent_b, act_b[2], bits_b;
+  Buf best_b, parent_b, act_b[2], link_b, bits_b;
   const uint32_t *src = nullptr, *dst = nullptr;  // input endpoints, indexed by edge id
   const uint32_t *w_in = nullptr;                 // input weights
   KeyLayout kl{0, 0, 0};  // unpacked unless choose_layout() packs
@@ -480,6 +470,16 @@ struct Solve {
     cur_v = (uint32_t *)((char *)cur_b.p + stride);
     return MST_OK;
   }
+  // Scratch of the one-launch rounds: links and representatives of the rounds.
+  uint32_t *link = nullptr, *reps = nullptr;
+  mst_status rounds_alloc() {
+    if (link) return MST_OK;
+    const uint64_t stride = round_up((uint64_t)n * 4 + 16, 256);
+    TRY(link_b.alloc(c, stride * 2, s));
+    link = link_b.as<uint32_t>();
+    reps = (uint32_t *)((char *)link_b.p + stride);
+    return MST_OK;
+  }
   // Sets the recording of ends by id on a pass that writes a list (unpacked keys).
   void record_ends(CompactArgs &a) const {
     a.cur_u = (layout_set && !kl.packed) ? cur_u : nullptr;
@@ -489,6 +489,7 @@ struct Solve {
   uint32_t *parent = nullptr, *act[2] = {nullptr, nullptr}, *bits = nullptr;
   int wbits = 32;  // bits of the largest weight (set with the key layout)
   int rounds = 0;
+  bool want_parent = true;  // representatives are read after a Borůvka call (the filter contracts them)
   int shape = 0;   // tile shape of the partition / filter compactions and the hook (shape_index)
   int rshape = 1;  // tile shape of the relabel compaction (relabel_shape_index)
 
@@ -507,10 +508,8 @@ struct Solve {
       parent = parent_b.as<uint32_t>();
     }
     launch_iota(parent, n, c->sms, s);
-    for (int i = 0; i < 2; ++i) {
-      TRY(act_b[i].alloc(c, (size_t)n * 4, s));
-      act[i] = act_b[i].as<uint32_t>();
-    }
+    TRY(act_b[0].alloc(c, (size_t)n * 4, s));
+    act[0] = act_b[0].as<uint32_t>();
     if (bits_external) {
       bits = bits_external;
     } else {
@@ -536,10 +535,14 @@ struct Solve {
     return cur_alloc();
   }
   // From the largest weight in hs->max_w (read back by the caller).
+  void layout_bits() {
+    kl.vbits = n > 1 ? 64 - __builtin_clzll((unsigned long long)(n - 1)) : 1;
+    kl.idbits = m > 1 ? 64 - __builtin_clzll((unsigned long long)(m - 1)) : 1;
+  }
   void set_layout() {
     layout_set = true;
-    const int vb = n > 1 ? 64 - __builtin_clzll((unsigned long long)(n - 1)) : 1;
-    const int ib = m > 1 ? 64 - __builtin_clzll((unsigned long long)(m - 1)) : 1;
+    layout_bits();
+    const int vb = kl.vbits, ib = kl.idbits;
     const uint32_t mw = c->hs->max_w;
     const int wb = mw ? 32 - __builtin_clz(mw) : 0;
     wbits = wb;
@@ -599,6 +602,15 @@ struct Solve {
   // hook of the first round walks from the input ends.
   mst_status boruvka(EdgeList E, uint64_t mE, bool validate, bool best_ready = false, bool ends_rec = false) {
     if (mE == 0) return MST_OK;
+    if (device_rounds()) {
+      bool ran = false;
+      TRY(boruvka_device(E, mE, validate, best_ready, ends_rec, ran));
+      if (ran) return MST_OK;
+    }
+    if (!act[1]) {
+      TRY(act_b[1].alloc(c, (size_t)n * 4, s));
+      act[1] = act_b[1].as<uint32_t>();
+    }
     if (!layout_set) TRY(choose_layout(w_in ? w_in : E.w));
     // round 0: minEdges straight from the stored list (atomic minima, or
     // segmented minima over the ends sorted by vertex), then hook and jump
@@ -648,18 +660,6 @@ struct Solve {
     for (int r = 1; n_act > 0; ++r) {
       if (r > bound) return MST_ERR_INTERNAL;
       if (base_case_fits(cur, cur_m, n_act)) return base_case(cur, cur_m, act[a], (uint32_t)n_act);
-      if (c->cfg.graph_rounds && cur.u == X.out.u && cur.id && !want_dedupe(r, cur_m)) {
-        bool used = false, done = false;
-        int ran = 0;
-        TRY(graph_rounds(X, Y, cur, cur_m, n_act, a, bound - r, used, done, ran));
-        if (used) {
-          r += ran;
-          rounds += ran;
-          if (done || n_act == 0 || cur_m == 0) return MST_OK;
-          --r;  // the loop's ++r
-          continue;
-        }
-      }
       RoundList &out = (cur.u == X.out.u) ? Y : X;
       TRY(zero_round_state(c, s));
       CompactArgs ca{};
@@ -756,196 +756,77 @@ struct Solve {
     return MST_OK;
   }
 
-  // The round graph over lists X, Y and active lists A (see build_round_graph),
-  // from the handle's cache.  Not cached yet: built at once when `always`,
-  // else only when the same shape is asked for again (a graph pays for its
-  // capture and instantiation only when its shape comes back); exec stays
-  // null when it is not built.  err_handback: the device-driven mode's error
-  // word (see launch_round_pre), or null.
-  mst_status round_graph(RoundList &X, RoundList &Y, uint32_t *const A[2], uint32_t max_iter, uint32_t *err_handback,
-                         bool always, cudaGraphExec_t &exec) {
-    exec = nullptr;
-    // launch bounds baked into the graph: the lists' capacity and n (the
-    // kernels read the actual counts from device memory), so the graph does
-    // not depend on this call's sizes
-    const uint64_t cap = std::min(X.cap, Y.cap), nmax = n;
-    if (!c->grounds) CK(cudaMalloc(&c->grounds, sizeof(GraphRounds)));
-    if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
-    const int base_ok = (c->cfg.base_case && !err_handback) ? 1 : 0;
-    const int jl = c->cfg.graph_jump_launches;
-    const RoundList *L[2] = {&X, &Y};
-    // A built graph is reused when every value baked into it is unchanged.
-    u64 sig = 0x2302121990ULL;
-    auto fold = [&](u64 v) { sig = host_mix64(sig ^ (v + 0x9e3779b97f4a7c15ULL)); };
-    for (int i = 0; i < 2; ++i) {
-      fold((u64)L[i]->out.u), fold((u64)L[i]->out.v), fold((u64)L[i]->out.w), fold((u64)L[i]->out.id);
-      fold((u64)A[i]);
-    }
-    const u64 vals[] = {(u64)parent,  (u64)best,    (u64)bits,     (u64)cur_u,  (u64)cur_v,
-                        (u64)src,     (u64)dst,     (u64)c->status, (u64)c->ds,  (u64)c->grounds,
-                        (u64)kl.packed, (u64)kl.vbits, (u64)kl.idbits, (u64)n,     (u64)cap,
-                        (u64)nmax,    (u64)jl,      (u64)base_ok,  (u64)max_iter, (u64)c->sms,
-                        (u64)shape,   (u64)err_handback};
-    for (u64 v : vals) fold(v);
-    for (size_t i = 0; i < c->round_graphs.size(); ++i)
-      if (c->round_graphs[i].sig == sig) {
-        const mst_ctx::RoundGraph hit = c->round_graphs[i];
-        c->round_graphs.erase(c->round_graphs.begin() + i);
-        c->round_graphs.insert(c->round_graphs.begin(), hit);
-        exec = hit.exec;
-        return MST_OK;
-      }
-    if (!always) {
-      auto &seen = c->round_sigs_seen;
-      const bool again = std::find(seen.begin(), seen.end(), sig) != seen.end();
-      if (!again) {
-        seen.insert(seen.begin(), sig);
-        if (seen.size() > 64) seen.pop_back();
-        return MST_OK;
-      }
-    }
-    return build_round_graph(sig, L, A, cap, nmax, base_ok, jl, max_iter, err_handback, exec);
+  // The rounds of a call run in one cooperative launch (rounds.cu) unless an
+  // option needs the host between them.
+  static constexpr uint64_t MIN_EDGES_KERNEL = 1ULL << 20;
+  bool device_rounds() const {
+    return c->cfg.graph_rounds && c->cfg.dedupe != MST_DEDUPE_HASH && c->cfg.dedupe != MST_DEDUPE_SORT;
   }
-
-  // Rounds of a Borůvka call as one CUDA graph launch (the round loop without
-  // host round trips): a conditional WHILE node repeats a body of two rounds
-  // (list X -> Y, then Y -> X; the active lists alternate the same way) while
-  // the device sees active vertices and edges.  It hands the state back to the
-  // host when the base case fits, when a round's pointer jumping needs more
-  // than the four launches a round holds, or at the round bound.  Counts live
-  // in device memory; nothing in the body waits for the host.
-  mst_status graph_rounds(RoundList &X, RoundList &Y, EdgeList &cur, uint64_t &cur_m, uint64_t &n_act, int &a,
-                          int rounds_left, bool &used, bool &done, int &ran) {
-    used = false;
-    done = false;
-    ran = 0;
-    const uint32_t max_iter = (uint32_t)(rounds_left > 2 ? rounds_left / 2 : 1);
-    uint32_t *A[2] = {act[a], act[1 - a]};
-    cudaGraphExec_t exec = nullptr;
-    TRY(round_graph(X, Y, A, max_iter, nullptr, false, exec));
-    if (!exec) return MST_OK;  // the first time, the host runs the rounds
-    GraphRounds *g = c->grounds;
-    used = true;
-    launch_round_init(g, cur_m, n_act, s);
-    PROF(MST_K_GRAPH, 0.0, -1, 0.0, -1, 0.0, CK(cudaGraphLaunch(exec, s)));
-    TRY(readback(c, s));
-    const u64 info = c->hs->count[CNT_TMP];
-    const uint32_t reason = (uint32_t)(info & 0xff), slot = (uint32_t)((info >> 8) & 0xff);
-    ran = 2 * (int)(info >> 16);
-    if (reason == ROUNDS_BOUND || reason == ROUNDS_RUNNING || slot > 1) return MST_ERR_INTERNAL;
-    cur_m = c->hs->count[CNT_EDGES];
-    n_act = c->hs->count[CNT_ACTIVE];
-    cur = (slot == 0 ? X : Y).list();
-    if (slot == 1) a = 1 - a;
-    if (reason == ROUNDS_DONE) {
-      done = true;
-      return MST_OK;
-    }
-    if (reason == ROUNDS_JUMP) TRY(jump_until_stars(act[a], nullptr, n_act, n_act, 0));
-    return MST_OK;
+  RoundsArgs rounds_args(RoundList &X, RoundList &Y) {
+    RoundsArgs ra{};
+    ra.list[0] = X.out;
+    ra.list[1] = Y.out;
+    ra.kl = kl;
+    ra.best = best;
+    ra.parent = parent;
+    ra.link = link;
+    ra.rep = reps;
+    ra.act = act[0];
+    ra.src = src;
+    ra.dst = dst;
+    ra.cur_u = cur_u;
+    ra.cur_v = cur_v;
+    ra.chosen_bits = bits;
+    ra.wsum = c->wsum;
+    ra.n = n;
+    ra.max_rounds = (uint32_t)std::min(ROUNDS_MAX, 2 * (ceil_log2(n) + 2));
+    ra.st = c->rstate;
+    ra.err = &c->ds->err;
+    return ra;
   }
-
-  // Captures and instantiates the round graph: an entry kernel that decides
-  // whether the loop runs at all, then a conditional WHILE node whose body is
-  // two rounds (slot 0 -> 1, slot 1 -> 0), each compaction (relabel + minEdges
-  // relaxation), hooking, `jl` pointer-jumping launches and a check; the body
-  // ends with the kernel that sets the loop condition.
-  mst_status build_round_graph(u64 sig, const RoundList *const L[2], uint32_t *const A[2], uint64_t cap, uint64_t nmax,
-                               int base_ok, int jl, uint32_t max_iter, uint32_t *err_handback,
-                               cudaGraphExec_t &exec_out) {
-    GraphRounds *g = c->grounds;
-    cudaStream_t cs = c->cap_stream;
-    struct Owned {
-      cudaGraph_t graph = nullptr;
-      cudaGraphExec_t exec = nullptr;
-      cudaStream_t capturing = nullptr;
-      ~Owned() {
-        if (capturing) {  // an error during capture: end it so the stream is usable again
-          cudaGraph_t dummy = nullptr;
-          cudaStreamEndCapture(capturing, &dummy);
-          cudaGetLastError();
-        }
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
-      }
-    } o;
-    CK(cudaGraphCreate(&o.graph, 0));
-    cudaGraphConditionalHandle h;
-    CK(cudaGraphConditionalHandleCreate(&h, o.graph, 0, cudaGraphCondAssignDefault));
-    // entry: the kernel that decides whether the loop runs at all
-    CK(cudaStreamBeginCaptureToGraph(cs, o.graph, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-    o.capturing = cs;
-    launch_round_pre(g, h, &c->ds->count[CNT_EDGES], err_handback, cs);
-    {
-      cudaGraph_t captured = nullptr;
-      o.capturing = nullptr;
-      CK(cudaStreamEndCapture(cs, &captured));
+  // boruvka() as one launch; nothing is read back (an error it sets stays
+  // latched until the next readback).  ran: false when it was not launched.
+  mst_status boruvka_device(EdgeList E, uint64_t mE, bool validate, bool best_ready, bool ends_rec, bool &ran) {
+    ran = false;
+    const bool sorted = !best_ready && c->cfg.min_edges_sort && 2 * mE < (1ULL << 32);
+    if (!layout_set && sorted) TRY(choose_layout(w_in ? w_in : E.w));
+    RoundList X, Y;
+    TRY(round_lists(c, mE, X, Y, s));
+    TRY(rounds_alloc());
+    const uint32_t *max_w = nullptr;
+    if (!layout_set) {  // the kernel picks the key layout from the largest weight
+      CK(cudaMemsetAsync(&c->ds->max_w, 0, sizeof(uint32_t), s));
+      launch_max_weight(w_in ? w_in : E.w, m, &c->ds->max_w, c->sms, s);
+      max_w = &c->ds->max_w;
+      layout_bits();
+      if (32 + kl.idbits + kl.vbits > 63) TRY(cur_alloc());  // the keys may not pack
     }
-    cudaGraphNode_t pre = nullptr;
-    size_t nodes = 1;
-    CK(cudaGraphGetNodes(o.graph, &pre, &nodes));
-    if (nodes != 1 || !pre) return MST_ERR_INTERNAL;
-    cudaGraphNodeParams cp{};
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = h;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    cudaGraphNode_t node;
-    CK(cudaGraphAddNode(&node, o.graph, &pre, nullptr, 1, &cp));
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-    o.capturing = cs;
-    for (int half = 0; half < 2; ++half) {
-      const int in = half, out = 1 - half;
-      CompactArgs ca{};
-      ca.shape = rshape;
-      ca.in = L[in]->list();
-      ca.m = cap;
-      ca.m_dev = &g->ce[in];
-      ca.out = L[out]->out;
-      ca.label = parent;
-      ca.n = n;
-      ca.kl = kl;
-      ca.best = best;
-      record_ends(ca);
-      ca.st = ScanState{c->status, c->ds->tile_ctr, 0, &g->ce[out], &c->ds->err, c->cfg.spin_limit};
-      launch_compact(CM_RELABEL, ca, cap, cs);
-      HookArgs hb{};
-      hb.shape = shape;
-      hb.cand = A[in];
-      hb.ncand_dev = &g->ca[in];
-      hb.best = best;
-      hb.kl = kl;
-      hb.src = cur_u ? cur_u : src;
-      hb.dst = cur_v ? cur_v : dst;
-      hb.parent = parent;
-      hb.chosen_bits = bits;
-      hb.active_out = A[out];
-      hb.counter = &g->ca[out];
-      hb.err = &c->ds->err;
-      hb.wsum = c->wsum;
-      launch_hook(hb, nmax, cs);
-      // pointer jumping: jl launches of up to 256 steps each; only the last
-      // launch reports a vertex short of its root
-      for (int k = 0; k < jl; ++k)
-        launch_jump(A[out], &g->ca[out], 0, nmax, parent, best, k == 0 ? 1 : 0, k == jl - 1 ? &g->jflag : &g->jdummy,
-                    c->sms, cs, 256);
-      if (half == 0) launch_round_check(g, base_ok, err_handback, cs);
+    if (sorted) {
+      Buf me_b;
+      TRY(me_b.alloc(c, min_edges_sort_scratch_bytes(mE, c->sms), s));
+      const double passes = (double)((ceil_log2((uint64_t)n + 1) + 7) / 8);
+      PROF(MST_K_MIN_EDGES, (12.0 + 24.0 + 2.0 * (32.0 * passes + 20.0)) * (double)mE, -1, 0.0, -1, 0.0,
+           best_ready = launch_min_edges_sort(E, mE, n, validate ? 1 : 0, kl, best, &c->ds->err, me_b.p, c->sms, s));
     }
-    launch_round_cond(g, h, base_ok, max_iter, &c->ds->count[CNT_EDGES], err_handback, cs);
-    cudaGraph_t captured = nullptr;
-    o.capturing = nullptr;
-    CK(cudaStreamEndCapture(cs, &captured));
-    CK(cudaGraphInstantiate(&o.exec, o.graph, 0));
-    c->round_graphs.insert(c->round_graphs.begin(), mst_ctx::RoundGraph{sig, o.graph, o.exec});
-    exec_out = o.exec;
-    o.graph = nullptr;
-    o.exec = nullptr;
-    while (c->round_graphs.size() > 16) {
-      cudaGraphExecDestroy(c->round_graphs.back().exec);
-      cudaGraphDestroy(c->round_graphs.back().graph);
-      c->round_graphs.pop_back();
+    RoundsArgs ra = rounds_args(X, Y);
+    ra.ends_rec = (ends_rec && cur_u) ? 1 : 0;
+    ra.record_first = (!best_ready && !ra.ends_rec && E.id && cur_u) ? 1 : 0;
+    // a long list's minEdges runs in its own kernel, whose eight edges per
+    // thread at full occupancy hide more latency than the resident blocks can
+    if (!best_ready && !ra.record_first && mE >= MIN_EDGES_KERNEL) {
+      PROF(MST_K_MIN_EDGES, 12.0 * (double)mE, -1, 0.0, -1, 0.0,
+           launch_min_edges(E, mE, n, validate ? 1 : 0, kl, best, &c->ds->err, c->sms, s, max_w));
+      best_ready = true;
     }
+    ra.in = E;
+    ra.m = mE;
+    ra.first_slot = E.u == X.out.u ? 1 : 0;
+    ra.best_ready = best_ready ? 1 : 0;
+    ra.validate = validate ? 1 : 0;
+    ra.max_w = max_w;
+    ra.want_parent = want_parent ? 1 : 0;
+    PROF(MST_K_GRAPH, 0.0, -1, 0.0, -1, 0.0, ran = launch_rounds(ra, mE, c->sms, s));
+    if (ran) ++rounds;
     return MST_OK;
   }
 
@@ -1265,16 +1146,15 @@ struct Solve {
   // isSparse and gives each list a capacity a little above q of its parent's.
   // The levels then run without the host reading anything:
   // pivot and partition from device counts, and the deepest light list and
-  // each level's filtered heavy edges solved by Borůvka rounds whose first
-  // hooking runs before the round graph and whose loop the device ends.  A
-  // list that outgrows its capacity (ERR_OVERFLOW), a round that would need
-  // the host (ERR_HANDBACK) or a contraction left short (the jump flag) makes
-  // the result unusable, and the caller starts over on the host-driven path.
-  // Where the estimate stops the recursion a level early or late the forest
-  // is the same: isSparse only steers the work.
+  // each level's filtered heavy edges solved by Borůvka rounds in one launch
+  // each.  A list that outgrows its capacity (ERR_OVERFLOW) or a contraction
+  // left short (the jump flag) makes the result unusable, and the caller
+  // starts over on the host-driven path.  Where the estimate stops the
+  // recursion a level early or late the forest is the same: isSparse only
+  // steers the work.
   bool plan_eligible() const {
     const mst_config &f = c->cfg;
-    return f.filter_plan && f.graph_rounds && !f.filter_carry && !f.filter_split && !f.min_edges_sort &&
+    return f.filter_plan && f.graph_rounds && n < (1u << 31) && !f.filter_carry && !f.filter_split && !f.min_edges_sort &&
            f.dedupe != MST_DEDUPE_HASH && f.dedupe != MST_DEDUPE_SORT && !is_sparse(m);
   }
   // Capacity planned for the light list of a list of at most `cap` edges:
@@ -1298,32 +1178,20 @@ struct Solve {
 
   // Borůvka rounds on the list in round list X whose length is count[slot]
   // (best[] holds its minEdges; ends_rec: its ends were recorded by id as it
-  // was written): the first hooking over all n vertices and its pointer
-  // jumping, then the round graph.
-  mst_status boruvka_planned(RoundList &X, RoundList &Y, int slot, bool ends_rec, cudaGraphExec_t exec) {
-    GraphRounds *g = c->grounds;
-    launch_round_init_dev(g, &c->ds->count[slot], std::min(X.cap, Y.cap), s);
-    HookArgs ha{};
-    ha.shape = shape;
-    ha.cand = nullptr;
-    ha.ncand = n;
-    ha.best = best;
-    ha.kl = kl;
-    const bool rec = ends_rec && cur_u;
-    ha.src = rec ? cur_u : src;
-    ha.dst = rec ? cur_v : dst;
-    ha.parent = parent;
-    ha.chosen_bits = bits;
-    ha.active_out = act[0];
-    ha.counter = &g->ca[0];
-    ha.err = &c->ds->err;
-    ha.wsum = c->wsum;
-    PROF(MST_K_HOOK, 8.0 * (double)n, -1, 0.0, -1, 0.0, launch_hook(ha, n, s));
-    const int jl = c->cfg.graph_jump_launches;
-    PROF(MST_K_JUMP, 0.0, -1, 0.0, -1, 0.0,
-         for (int k = 0; k < jl; ++k) launch_jump(act[0], &g->ca[0], 0, n, parent, best, k == 0 ? 1 : 0,
-                                                  k == jl - 1 ? &g->jflag : &g->jdummy, c->sms, s, 256));
-    PROF(MST_K_GRAPH, 0.0, -1, 0.0, -1, 0.0, CK(cudaGraphLaunch(exec, s)));
+  // was written), in one launch.  last: nothing reads the representatives
+  // afterwards.
+  mst_status boruvka_planned(RoundList &X, RoundList &Y, int slot, bool ends_rec, bool last) {
+    RoundsArgs ra = rounds_args(X, Y);
+    ra.in = X.list();
+    ra.m = std::min(X.cap, Y.cap);
+    ra.m_dev = &c->ds->count[slot];
+    ra.first_slot = 1;
+    ra.best_ready = 1;
+    ra.want_parent = last ? 0 : 1;
+    ra.ends_rec = (ends_rec && cur_u) ? 1 : 0;
+    bool ran = false;
+    PROF(MST_K_GRAPH, 0.0, -1, 0.0, -1, 0.0, ran = launch_rounds(ra, ra.m, c->sms, s));
+    if (!ran) return MST_ERR_CUDA;
     ++rounds;
     return MST_OK;
   }
@@ -1398,10 +1266,7 @@ struct Solve {
     if (need > X.cap) TRY(round_lists(c, need, X, Y, s));  // (not when leaf_top: X already holds list 1)
     planned = true;
     CK(cudaMemsetAsync(&c->ds->jump_flag, 0, sizeof(uint32_t), s));
-    uint32_t *A[2] = {act[0], act[1]};
-    cudaGraphExec_t exec = nullptr;
-    TRY(round_graph(X, Y, A, (uint32_t)(ceil_log2(n) + 2), &c->ds->err, true, exec));
-    if (!exec) return MST_ERR_INTERNAL;
+    TRY(rounds_alloc());
 
     // light lists 2 .. K (list K into X, relaxing best[] for its first round)
     std::unique_ptr<ListBuf[]> Lb(new ListBuf[K + 1]);
@@ -1436,7 +1301,7 @@ struct Solve {
                  ProfTerm{CNT_LVL + k, 16.0, 16.0}, ProfTerm{CNT_LVL + k + 1, 16.0, 16.0});
       E[k + 1] = last ? X.list() : Lb[k + 1].list();
     }
-    TRY(boruvka_planned(X, Y, CNT_LVL + K, cur_u != nullptr, exec));
+    TRY(boruvka_planned(X, Y, CNT_LVL + K, cur_u != nullptr, false));
 
     // levels K-1 .. 0: contract P and mark the giant component, filter the
     // level's heavy edges into X, and solve them
@@ -1471,7 +1336,7 @@ struct Solve {
       PROF_TERMS(MST_K_FILTER, fixed, fixed, launch_compact(CM_FILTER, cf, caps[k], s),
                  ProfTerm{k == 0 ? -1 : CNT_LVL + k, per, per}, ProfTerm{CNT_LVL + k + 1, 0.0, -per},
                  ProfTerm{CNT_LVL + LVL_MAX + k, 16.0, 16.0});
-      TRY(boruvka_planned(X, Y, CNT_LVL + LVL_MAX + k, cur_u != nullptr, exec));
+      TRY(boruvka_planned(X, Y, CNT_LVL + LVL_MAX + k, cur_u != nullptr, k == 0));
     }
     return MST_OK;
   }
@@ -1542,7 +1407,7 @@ mst_status solve_device(mst_ctx *c, uint32_t n, uint64_t m, const uint32_t *src,
       TRY(S.filter_planned(planned));
       if (planned) {
         ++c->planned;
-        constexpr uint32_t replan = ERR_OVERFLOW | ERR_HANDBACK;
+        constexpr uint32_t replan = ERR_OVERFLOW;
         TRY(S.finalize(out_ids, out_count, total_weight, replan));
         if (!(c->hs->err & replan) && !c->hs->jump_flag) return MST_OK;
         ++c->plan_fallbacks;
@@ -1551,6 +1416,7 @@ mst_status solve_device(mst_ctx *c, uint32_t n, uint64_t m, const uint32_t *src,
     }
     TRY(S.filter(in, m, true, 0));
   } else {
+    S.want_parent = false;
     TRY(S.boruvka(in, m, true));
   }
   return S.finalize(out_ids, out_count, total_weight);
@@ -1886,6 +1752,7 @@ mst_status mst_create(mst_handle *out, const mst_config *cfg) {
   ok = ok && ensure_sample(c) == MST_OK;
   ok = ok && cudaMalloc(&c->pivot_scratch, pivot_scratch_bytes()) == cudaSuccess;
   ok = ok && cudaMalloc(&c->wsum, WSUM_SLOTS * sizeof(u64)) == cudaSuccess;
+  ok = ok && cudaMalloc(&c->rstate, sizeof(RoundsState)) == cudaSuccess;
   ok = ok && cudaDeviceSynchronize() == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -1913,17 +1780,12 @@ void mst_destroy(mst_handle h) {
     if (h->sample_buf) cudaFree(h->sample_buf);
     if (h->pivot_scratch) cudaFree(h->pivot_scratch);
     if (h->wsum) cudaFree(h->wsum);
-    if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
     for (int k = 0; k < 2; ++k) {
       if (h->in_ready[k]) cudaEventDestroy(h->in_ready[k]);
       if (h->in_free[k]) cudaEventDestroy(h->in_free[k]);
     }
-    for (auto &rg : h->round_graphs) {
-      cudaGraphExecDestroy(rg.exec);
-      cudaGraphDestroy(rg.graph);
-    }
-    if (h->grounds) cudaFree(h->grounds);
+    if (h->rstate) cudaFree(h->rstate);
     if (h->pool) cudaMemPoolDestroy(h->pool);
     for (auto &r : h->prof_pending) {
       if (r.a) h->ev_pool.push_back(r.a);
@@ -1988,10 +1850,13 @@ uint64_t mst_workspace_bytes(uint32_t n, uint64_t m, const mst_config *cfg) {
   mst_config def;
   mst_config_default(&def);
   if (!cfg) cfg = &def;
-  const uint64_t vert = (uint64_t)n * (8 + 4 + 4 + 4);  // best, parent, two active lists
+  const uint64_t vert = (uint64_t)n * (8 + 4 + 4 + 4 + 4) + 4096;  // best, parent, active list, links, representatives
   const uint64_t bits = (m + 31) / 32 * 4;
   const uint64_t list = 16 * m + 1024;
-  uint64_t edges = 2 * (list + list / 4 + (16ULL << 16));       // the handle's ping-pong round lists (grown with
+  const int vb = n > 1 ? 64 - __builtin_clzll((unsigned long long)(n - 1)) : 1;
+  const int ib = m > 1 ? 64 - __builtin_clzll((unsigned long long)(m - 1)) : 1;
+  uint64_t edges = 32 + vb + ib > 63 ? 8 * m + 1024 : 0;         // ends by id, where the keys may not pack
+  edges += 2 * (list + list / 4 + (16ULL << 16));                // the handle's ping-pong round lists (grown with
                                                                  // a quarter of headroom, in steps of 2^16 edges)
   if (cfg->dedupe != MST_DEDUPE_NONE) edges += list + 32 * m + 16384;  // dedupe list + hash table
   if (cfg->variant != MST_VARIANT_BORUVKA) edges += 2 * list;   // partition levels and filtered lists
