@@ -38,6 +38,18 @@ __device__ __forceinline__ bool same_edge(const KeyLayout &kl, u64 a, u64 b) {
   return kl.packed ? (a >> kl.vbits) == (b >> kl.vbits) : a == b;
 }
 
+__device__ __forceinline__ u64 mix64(u64 z) {  // splitmix64 finaliser
+  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
+  z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
+  return z ^ (z >> 31);
+}
+
+// Output #i of the splitmix64 sequence whose state starts at `state`
+// (Steele, Lea, Flood, OOPSLA 2014).
+__device__ __forceinline__ u64 splitmix64_at(u64 state, u64 i) {
+  return mix64(state + (i + 1ULL) * 0x9e3779b97f4a7c15ULL);
+}
+
 // Exclusive block-wide scan of one uint32 per thread (B threads; s_warp holds
 // B / 32 + 1 words).
 template <int B = 256>

@@ -274,6 +274,37 @@ struct RoundsArgs {
 // (nothing ran).
 bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, int sms, cudaStream_t s);
 
+// Whole graphs solved by one block each (block.cu).
+constexpr uint32_t BLOCK_MAX_N = 65536;   // 16-bit labels
+constexpr uint64_t BLOCK_MAX_M = 1ULL << 22;
+// Vertices up to which a graph runs in a block of 256 threads (four per SM),
+// and of 512 (two per SM): their minima fill the blocks' shared memory.
+constexpr uint32_t BLOCK_SMALL_N = 12288, BLOCK_MID_N = 28416;
+struct BlockArgs {
+  const uint32_t *gn;          // vertices per graph
+  const uint64_t *edge_off, *vert_off;
+  const uint32_t *src, *dst, *w;
+  uint64_t m_total;            // edges of the arrays
+  const uint32_t *order;       // graphs, largest first
+  uint32_t first, num;         // this launch's part of order
+  uint32_t *queue;             // zero before the launch
+  uint2 *ends0;                // [m_total] scratch
+  uint32_t *uv;                // [m_total] scratch
+  u64 *key;                    // [m_total] scratch
+  u64 *gbest;                  // [vertices] scratch
+  uint32_t *bits;              // chosen-edge bitmap
+  u64 *totals;                 // forest weight and size, and 1 in solved, of each graph
+  uint32_t *sizes;
+  uint32_t *solved;
+  uint32_t *err;
+  uint32_t smem;               // set by the launchers
+};
+// kind: 0 the large graphs, 1 the middle ones, 2 the small ones.
+bool launch_block_batch(const BlockArgs &a, int kind, cudaStream_t s);
+// The one graph (n, m) of the arrays; clears *err, bits and writes the forest.
+bool launch_block_single(const BlockArgs &a, uint32_t n, uint32_t m, uint32_t *out_ids, uint32_t *out_count,
+                         cudaStream_t s);
+
 // single-block base case: the last rounds of a Borůvka call in one launch
 constexpr uint32_t BASE_MAX_N = 4096;  // live components (16-bit local ends; shared-memory vertex arrays)
 constexpr uint64_t BASE_MAX_M = 6144;  // live edges (fit the tile kernel's shared-memory edge capacity)

@@ -73,18 +73,6 @@ __device__ __forceinline__ u64 pair_of(uint32_t a, uint32_t b) {
   return a < b ? (((u64)a << 32) | b) : (((u64)b << 32) | a);
 }
 
-__device__ __forceinline__ u64 mix64(u64 z) {  // splitmix64 finaliser
-  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
-  z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
-  return z ^ (z >> 31);
-}
-
-// Output #i of the splitmix64 sequence whose state starts at `state`
-// (Steele, Lea, Flood, OOPSLA 2014).
-__device__ __forceinline__ u64 splitmix64_at(u64 state, u64 i) {
-  return mix64(state + (i + 1ULL) * 0x9e3779b97f4a7c15ULL);
-}
-
 // Decoupled look-back by the whole block.  Publishes the tile's aggregate,
 // then examines LB_WINDOW = BLOCK * LB_PER_THREAD predecessors per round (each
 // thread polls LB_PER_THREAD status words, bounded), adds the values up to the

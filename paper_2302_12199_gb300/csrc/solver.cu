@@ -16,6 +16,7 @@
 
 #include <cuda_runtime.h>
 
+#include "device.cuh"
 #include "internal.h"
 #include "mst.h"
 
@@ -70,6 +71,9 @@ struct mst_ctx {
   // kept by the handle and grown on demand
   void *rl_mem = nullptr;
   uint64_t rl_cap = 0;  // edges per list
+  void *small_mem = nullptr;      // scratch of graphs that one block solves (SmallScratch)
+  cudaStream_t kind_stream[2] = {nullptr, nullptr};  // block solves of the middle and the small graphs of a batch
+  cudaEvent_t kind_ev[3] = {nullptr, nullptr, nullptr};
   RoundsState *rstate = nullptr;  // device state of the one-launch rounds
   std::vector<cudaEvent_t> ev_pool;
   std::vector<ProfRec> prof_pending;
@@ -446,6 +450,17 @@ mst_status zero_round_state(mst_ctx *c, cudaStream_t s) {
   CK(cudaMemsetAsync(&c->ds->jump_flag, 0, offsetof(DevState, count) + 3 * sizeof(u64) - offsetof(DevState, jump_flag),
                      s));
   return MST_OK;
+}
+
+// Graphs up to these sizes are solved by one block (block.cu) unless an option
+// asks for other passes: one launch and one readback.
+constexpr uint64_t SINGLE_MAX_M = 1ULL << 15;
+constexpr uint32_t SINGLE_MAX_N = BLOCK_SMALL_N;
+constexpr size_t SMALL_KEY = SINGLE_MAX_M * 8, SMALL_ARR = SINGLE_MAX_M * 4, SMALL_BEST = SINGLE_MAX_N * 8;
+constexpr size_t SMALL_BYTES = SMALL_KEY + SMALL_BEST + 3 * SMALL_ARR + SINGLE_MAX_M / 8;
+bool block_solves(const mst_config &f) {
+  return f.base_case && f.graph_rounds && f.tile_contract == 0 && !f.min_edges_sort && f.dedupe != MST_DEDUPE_HASH &&
+         f.dedupe != MST_DEDUPE_SORT;
 }
 
 // Per-solve state: vertex arrays and the chosen-edge bitmap.
@@ -1356,7 +1371,9 @@ struct Solve {
 
   // The ids come from the chosen-edge bitmap; the total from the counters the
   // hooking kernels added each chosen edge's weight into (no gather of w).
+  // Without out_ids the bitmap is all the caller wants.
   mst_status finalize(uint32_t *out_ids, uint32_t *out_count, u64 *total_weight, uint32_t tolerated = 0) {
+    if (!out_ids) return readback(c, s, tolerated);
     PROF(MST_K_FINALIZE, (double)((m + 31) / 32 * 4), CNT_AUX, 4.0, -1, 0.0,
          launch_finalize(bits, m, nullptr, out_ids, out_count, total_weight, next_scan(c, CNT_AUX), s);
          launch_wsum_total(c->wsum, total_weight, s));
@@ -1370,11 +1387,37 @@ bool use_filter(const mst_config &cfg, uint32_t n, uint64_t m) {
   return m >= (1ULL << 20) && 2.0 * (double)m > 8.0 * (double)n;
 }
 
+// A graph that one block solves: one launch, one readback.
+mst_status solve_small(mst_ctx *c, uint32_t n, uint32_t m, const uint32_t *src, const uint32_t *dst, const uint32_t *w,
+                       uint32_t *out_ids, uint32_t *out_count, u64 *total_weight, cudaStream_t s, bool &ran) {
+  char *b = static_cast<char *>(c->small_mem);
+  BlockArgs a{};
+  a.src = src;
+  a.dst = dst;
+  a.w = w;
+  a.m_total = m;
+  a.key = (u64 *)b;
+  a.gbest = (u64 *)(b += SMALL_KEY);
+  a.ends0 = (uint2 *)(b += SMALL_BEST);
+  a.uv = (uint32_t *)(b += 2 * SMALL_ARR);
+  a.bits = (uint32_t *)(b += SMALL_ARR);
+  a.totals = total_weight;
+  a.err = &c->ds->err;
+  PROF(MST_K_BASE, 12.0 * (double)m + 4.0 * (double)n, -1, 0.0, -1, 0.0,
+       ran = launch_block_single(a, n, m, out_ids, out_count, s));
+  if (!ran) return MST_OK;
+  ++c->solves;
+  return readback(c, s);
+}
+
+// bits_out (zeroed by the caller): the forest as a bitmap over the edges
+// instead of ids, count and weight.
 mst_status solve_device(mst_ctx *c, uint32_t n, uint64_t m, const uint32_t *src, const uint32_t *dst,
                         const uint32_t *w, uint32_t *out_ids, uint32_t *out_count, u64 *total_weight,
-                        cudaStream_t s) {
+                        cudaStream_t s, uint32_t *bits_out = nullptr) {
   if (m >= (1ULL << 32)) return MST_ERR_TOO_LARGE;
-  if (!out_count || !total_weight || (m > 0 && (!src || !dst || !w || !out_ids))) return MST_ERR_INVALID_ARG;
+  if (!bits_out && (!out_count || !total_weight || (m > 0 && (!src || !dst || !w || !out_ids))))
+    return MST_ERR_INVALID_ARG;
   if (!aligned4(src) || !aligned4(dst) || !aligned4(w) || !aligned4(out_ids)) return MST_ERR_INVALID_ARG;
   if (n == 0 || m == 0) {
     if (m > 0 && n == 0) return MST_ERR_VERTEX_RANGE;
@@ -1383,9 +1426,14 @@ mst_status solve_device(mst_ctx *c, uint32_t n, uint64_t m, const uint32_t *src,
     CK(cudaStreamSynchronize(s));
     return MST_OK;
   }
+  if (!bits_out && n <= SINGLE_MAX_N && m <= SINGLE_MAX_M && block_solves(c->cfg)) {
+    bool ran = false;
+    TRY(solve_small(c, n, (uint32_t)m, src, dst, w, out_ids, out_count, total_weight, s, ran));
+    if (ran) return MST_OK;
+  }
   Solve S(c, s, n, m);
-  TRY(S.init());
-  ++c->solves;
+  TRY(S.init(nullptr, bits_out));
+  if (!bits_out) ++c->solves;
   S.src = src;
   S.dst = dst;
   S.w_in = w;
@@ -1501,6 +1549,8 @@ __device__ __forceinline__ uint32_t batch_graph_of(const uint64_t *off, uint32_t
 // totals[1] = edge_off[G] (all edges); ERR_TABLE if edge_off[0] != 0 or the
 // offsets decrease somewhere.
 constexpr int TAB_THREADS = 1024;
+// A block solves a graph of this many edges whatever the batch: about 0.2 ms.
+constexpr uint64_t BLOCK_MIN_LIMIT = 1ULL << 17;
 __global__ void __launch_bounds__(TAB_THREADS) batch_tables_kernel(const uint32_t *gn, const uint64_t *edge_off,
                                                                   uint32_t G, uint64_t *vert_off, u64 *totals,
                                                                   uint32_t *err) {
@@ -1550,12 +1600,132 @@ __global__ void __launch_bounds__(TAB_THREADS) batch_tables_kernel(const uint32_
   }
 }
 
-// Union vertex ids: edge e of graph g gets its ends offset by vert_off[g].
+// Which graphs of a batch one block each solves, and in which order: those
+// with at most BLOCK_MAX_N vertices and at most mlim edges (no block should
+// run much longer than the batch's share per SM), the large ones first, then
+// the middle and the small ones, each kind by falling size (half powers of
+// two).  counts: their three numbers and their edges.
+__global__ void __launch_bounds__(TAB_THREADS) batch_order_kernel(const uint32_t *gn, const uint64_t *edge_off,
+                                                                  uint32_t G, uint64_t mlim, int sms,
+                                                                  uint32_t *order, u64 *counts) {
+  constexpr int BUCKETS = 64;
+  __shared__ uint32_t s_n[3 * BUCKETS];
+  __shared__ u64 s_edges;
+  const uint64_t lim = max(mlim, (uint64_t)edge_off[G] / (uint64_t)sms);
+  if (threadIdx.x < 3 * BUCKETS) s_n[threadIdx.x] = 0;
+  if (threadIdx.x == 0) s_edges = 0;
+  __syncthreads();
+  auto bucket = [&](uint32_t g) -> int {
+    const uint64_t m = edge_off[g + 1] - edge_off[g];
+    const uint32_t n = gn[g];
+    if (m > 0 && (n > BLOCK_MAX_N || m > lim || m > BLOCK_MAX_M)) return -1;
+    const int lg = 63 - __clzll((long long)(m | 1));
+    const int half = lg > 0 ? (int)(m >> (lg - 1) & 1) : 0;
+    const int kind = m == 0 || n <= BLOCK_SMALL_N ? 2 : n <= BLOCK_MID_N ? 1 : 0;
+    return kind * BUCKETS + BUCKETS - 1 - (2 * lg + half);
+  };
+  u64 edges = 0;
+  for (uint32_t g = threadIdx.x; g < G; g += TAB_THREADS) {
+    const int b = bucket(g);
+    if (b < 0) continue;
+    atomicAdd(&s_n[b], 1u);
+    edges += edge_off[g + 1] - edge_off[g];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) edges += __shfl_xor_sync(0xffffffffu, edges, o);
+  if ((threadIdx.x & 31) == 0 && edges) atomicAdd(&s_edges, edges);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t sum = 0;
+    for (int kind = 0; kind < 3; ++kind) {
+      const uint32_t before = sum;
+      for (int b = kind * BUCKETS; b < (kind + 1) * BUCKETS; ++b) {
+        const uint32_t x = s_n[b];
+        s_n[b] = sum;
+        sum += x;
+      }
+      counts[kind] = sum - before;
+    }
+    counts[3] = s_edges;
+  }
+  __syncthreads();
+  for (uint32_t g = threadIdx.x; g < G; g += TAB_THREADS) {
+    const int b = bucket(g);
+    if (b >= 0) order[atomicAdd(&s_n[b], 1u)] = g;
+  }
+}
+
+// Segment offsets of the per-graph forests from their sizes (one block).
+__global__ void __launch_bounds__(TAB_THREADS) batch_msf_off_kernel(const uint32_t *counts, uint32_t G,
+                                                                    uint64_t *msf_off) {
+  __shared__ u64 s_warp[TAB_THREADS / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // a thread takes `per` graphs in a row
+  const uint32_t per = (G + TAB_THREADS - 1) / TAB_THREADS;
+  const uint64_t g0 = min((uint64_t)G, (uint64_t)threadIdx.x * per), g1 = min((uint64_t)G, g0 + per);
+  u64 sum = 0;
+  for (uint64_t g = g0; g < g1; ++g) sum += counts[g];
+  u64 incl = sum;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const u64 y = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += y;
+  }
+  if (lane == 31) s_warp[wid] = incl;
+  __syncthreads();
+  u64 before = incl - sum;
+  for (int i = 0; i < wid; ++i) before += s_warp[i];
+  for (uint64_t g = g0; g < g1; ++g) {
+    msf_off[g] = before;
+    before += counts[g];
+  }
+  if (threadIdx.x == TAB_THREADS - 1) msf_off[G] = before;
+}
+
+// The graphs' forests as ascending graph-local ids, from the chosen-edge
+// bitmap: a block per graph (taken from a queue, the largest first), a word of
+// the bitmap per thread and step.
+constexpr int EMIT_THREADS = 512;
+__global__ void __launch_bounds__(EMIT_THREADS) batch_emit_kernel(const uint32_t *bits, const uint64_t *edge_off,
+                                                                 const uint32_t *order, uint32_t G,
+                                                                 const uint64_t *msf_off, uint32_t *queue,
+                                                                 uint32_t *out_ids) {
+  __shared__ uint32_t s_warp[EMIT_THREADS / 32 + 1], s_next;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_next = atomicAdd(queue, 1u);
+    __syncthreads();
+    if (s_next >= G) return;
+    const uint32_t g = order[s_next];
+    const uint64_t lo = edge_off[g], hi = edge_off[g + 1];
+    uint64_t base = msf_off[g];
+    if (base == msf_off[g + 1]) continue;
+    for (uint64_t w0 = lo >> 5; w0 * 32 < hi; w0 += EMIT_THREADS) {
+      const uint64_t e0 = (w0 + threadIdx.x) * 32;
+      uint32_t word = e0 < hi ? bits[w0 + threadIdx.x] : 0u;
+      if (e0 < lo) word &= ~((1u << (lo - e0)) - 1u);             // (the graph before)
+      if (e0 < hi && hi - e0 < 32) word &= (1u << (hi - e0)) - 1u;  // (the graph after)
+      uint32_t total;
+      uint64_t p = base + block_exclusive_scan<EMIT_THREADS>((uint32_t)__popc(word), total, s_warp);
+      for (; word; word &= word - 1) out_ids[p++] = (uint32_t)(e0 - lo) + (uint32_t)__ffs(word) - 1;
+      base += total;
+      __syncthreads();  // s_warp is reused
+    }
+  }
+}
+
+__global__ void or_bits_kernel(uint32_t *x, const uint32_t *y, uint64_t words) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x)
+    x[i] |= y[i];
+}
+
+// Union vertex ids: edge e of graph g gets its ends offset by vert_off[g]; an
+// edge of a graph that is already solved becomes a self-loop.
 // Each block takes a contiguous chunk of edges (so a thread walks forward
 // through few graphs), independent of how the edges split into graphs.
 __global__ void batch_offset_kernel(const uint32_t *src, const uint32_t *dst, const uint64_t *edge_off,
                                     const uint64_t *vert_off, uint32_t *usrc, uint32_t *udst, const uint32_t *gn,
-                                    uint32_t G, uint64_t m, uint32_t *err) {
+                                    uint32_t G, uint64_t m, const uint32_t *solved, uint32_t *err) {
   const uint64_t chunk = ((m + gridDim.x - 1) / gridDim.x + blockDim.x - 1) / blockDim.x * blockDim.x;
   const uint64_t lo = (uint64_t)blockIdx.x * chunk, hi = min(m, lo + chunk);
   uint64_t e = lo + threadIdx.x;
@@ -1564,6 +1734,10 @@ __global__ void batch_offset_kernel(const uint32_t *src, const uint32_t *dst, co
   for (; e < hi; e += blockDim.x) {
     while (edge_off[g + 1] <= e) ++g;
     const uint32_t vo = (uint32_t)vert_off[g], ng = gn[g];
+    if (solved && solved[g]) {
+      usrc[e] = udst[e] = 0;
+      continue;
+    }
     const uint32_t a = src[e], b = dst[e];
     if (a >= ng || b >= ng) atomicOr(err, ERR_VERTEX);
     usrc[e] = a < ng ? a + vo : vo;
@@ -1589,11 +1763,12 @@ __global__ void batch_seg_kernel(const uint32_t *ids, const uint32_t *count, con
   msf_off[g] = lo;
 }
 
-// Graph-local ids and per-graph weight sums (total_weight zeroed before).
+// Graph-local ids, and the weight sums of the graphs not solved yet
+// (total_weight zeroed before).
 // Contiguous chunks per block; a warp adds up the weights of each run of ids
 // of one graph and issues one atomic per run.
 __global__ void batch_split_kernel(const uint32_t *ids, const uint32_t *count, const uint64_t *edge_off, uint32_t G,
-                                   const uint32_t *w, uint32_t *out_ids, u64 *total_weight) {
+                                   const uint32_t *w, const uint32_t *solved, uint32_t *out_ids, u64 *total_weight) {
   const uint64_t k = *count;
   const uint64_t chunk = ((k + gridDim.x - 1) / gridDim.x + blockDim.x - 1) / blockDim.x * blockDim.x;
   const uint64_t lo = (uint64_t)blockIdx.x * chunk, hi = min(k, lo + chunk);
@@ -1613,8 +1788,10 @@ __global__ void batch_split_kernel(const uint32_t *ids, const uint32_t *count, c
       }
       while (edge_off[g + 1] <= id) ++g;
       out_ids[i] = (uint32_t)((uint64_t)id - edge_off[g]);
-      v = w[id];
-      gi = g;
+      if (!solved || !solved[g]) {
+        v = w[id];
+        gi = g;
+      }
     }
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {  // segmented inclusive sum over runs of equal graph
@@ -1623,7 +1800,7 @@ __global__ void batch_split_kernel(const uint32_t *ids, const uint32_t *count, c
       if (lane >= o && pg == gi) v += pv;
     }
     const uint32_t ng = __shfl_down_sync(0xffffffffu, gi, 1);
-    if (in && (lane == 31 || ng != gi)) atomicAdd(total_weight + gi, v);
+    if (gi != 0xffffffffu && (lane == 31 || ng != gi)) atomicAdd(total_weight + gi, v);
   }
 }
 
@@ -1752,6 +1929,7 @@ mst_status mst_create(mst_handle *out, const mst_config *cfg) {
   ok = ok && ensure_sample(c) == MST_OK;
   ok = ok && cudaMalloc(&c->pivot_scratch, pivot_scratch_bytes()) == cudaSuccess;
   ok = ok && cudaMalloc(&c->wsum, WSUM_SLOTS * sizeof(u64)) == cudaSuccess;
+  ok = ok && cudaMalloc(&c->small_mem, SMALL_BYTES) == cudaSuccess;
   ok = ok && cudaMalloc(&c->rstate, sizeof(RoundsState)) == cudaSuccess;
   ok = ok && cudaDeviceSynchronize() == cudaSuccess;
   if (!ok) {
@@ -1786,6 +1964,11 @@ void mst_destroy(mst_handle h) {
       if (h->in_free[k]) cudaEventDestroy(h->in_free[k]);
     }
     if (h->rstate) cudaFree(h->rstate);
+    for (cudaStream_t ks : h->kind_stream)
+      if (ks) cudaStreamDestroy(ks);
+    for (cudaEvent_t e : h->kind_ev)
+      if (e) cudaEventDestroy(e);
+    if (h->small_mem) cudaFree(h->small_mem);
     if (h->pool) cudaMemPoolDestroy(h->pool);
     for (auto &r : h->prof_pending) {
       if (r.a) h->ev_pool.push_back(r.a);
@@ -2025,38 +2208,144 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
   if (clear_device_flags(h, s) != MST_OK) return record_cuda(h, __LINE__);
   batch_tables_kernel<<<1, TAB_THREADS, 0, s>>>(d_n, d_edge_off, num_graphs, d_voff, &h->ds->count[CNT_AUX],
                                                 &h->ds->err);
+  // tables of the block solves: the order of the graphs, their forests' sizes,
+  // which are solved, four queues
+  const bool blocks = block_solves(h->cfg);
+  Buf tab_b;
+  uint32_t *order = nullptr, *sizes = nullptr, *solved = nullptr, *queue = nullptr;
+  if (blocks) {
+    st = tab_b.alloc(h, ((size_t)num_graphs * 3 + 4) * 4, s);
+    if (st != MST_OK) return record(h, st);
+    order = tab_b.as<uint32_t>();
+    sizes = order + num_graphs;
+    solved = sizes + num_graphs;
+    queue = solved + num_graphs;
+    if (cudaMemsetAsync(solved, 0, ((size_t)num_graphs + 4) * 4, s) != cudaSuccess) return record_cuda(h, __LINE__);
+    batch_order_kernel<<<1, TAB_THREADS, 0, s>>>(d_n, d_edge_off, num_graphs, BLOCK_MIN_LIMIT, h->sms, order,
+                                                          &h->ds->count[CNT_LVL]);
+  }
   st = readback(h, s);
   if (st != MST_OK) return record(h, st);
   const uint64_t n_total = h->hs->count[CNT_AUX], m = h->hs->count[CNT_AUX + 1];
   if (n_total >= (1ULL << 32) || m >= (1ULL << 32)) return record(h, MST_ERR_TOO_LARGE);
   if (m > 0 && (!d_src || !d_dst || !d_w || !d_msf_ids)) return record(h, MST_ERR_INVALID_ARG);
   const uint32_t n = (uint32_t)n_total;
-  // union endpoints, union ids
-  Buf uni_b, ids_b;
-  const uint64_t stride = round_up(m * 4 + 16, 256);
-  st = uni_b.alloc(h, stride * 2, s);
-  const uint64_t cap = m < (uint64_t)n ? m : (uint64_t)n;
-  // ids, then (256-byte aligned) the forest size, then 256 bytes on, its weight
-  if (st == MST_OK) st = ids_b.alloc(h, round_up(cap * 4, 256) + 512, s);
-  if (st != MST_OK) return record(h, st);
-  uint32_t *usrc = uni_b.as<uint32_t>(), *udst = (uint32_t *)((char *)uni_b.p + stride);
-  uint32_t *ids = ids_b.as<uint32_t>();
-  uint32_t *d_count = (uint32_t *)((char *)ids + round_up(cap * 4, 256));
-  u64 *d_sum = (u64 *)((char *)d_count + 256);
-  const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((m + 2047) / 2048, (uint64_t)h->sms * 8));
-  if (m > 0)
-    batch_offset_kernel<<<grid, 256, 0, s>>>(d_src, d_dst, d_edge_off, d_voff, usrc, udst, d_n, num_graphs, m,
-                                             &h->ds->err);
-  st = readback(h, s);
-  if (st != MST_OK) return record(h, st);
-  st = solve_device(h, n, m, usrc, udst, d_w, ids, d_count, d_sum, s);
-  if (st != MST_OK) return record(h, st);
+  const uint64_t cap = m < (uint64_t)n ? m : (uint64_t)n, words = (m + 31) / 32;
+  // the forest's union ids, then (256-byte aligned) its size, then 256 bytes on, its weight
+  Buf ids_b, bits_b;
+  uint32_t *ids = nullptr, *d_count = nullptr;
+  u64 *d_sum = nullptr;
+  auto union_ids = [&]() -> mst_status {
+    TRY(ids_b.alloc(h, round_up(cap * 4, 256) + 512, s));
+    ids = ids_b.as<uint32_t>();
+    d_count = (uint32_t *)((char *)ids + round_up(cap * 4, 256));
+    d_sum = (u64 *)((char *)d_count + 256);
+    return MST_OK;
+  };
   if (cudaMemsetAsync(d_total_weight, 0, (size_t)num_graphs * 8, s) != cudaSuccess) return record_cuda(h, __LINE__);
+
+  // Graphs that fit a block each, when they hold at least half of the edges
+  // (below that the union passes below dominate, and a block per graph only
+  // adds its own time in front of them).
+  const u64 *kinds = &h->hs->count[CNT_LVL];
+  const uint64_t mblk = h->hs->count[CNT_LVL + 3];
+  const bool use_blocks = blocks && m > 0 && 2 * mblk >= m;
+  if (use_blocks) {
+    Buf scr_b;
+    const uint64_t stride = round_up(m * 4 + 16, 256);
+    st = scr_b.alloc(h, stride * 5 + (size_t)n * 8 + 256, s);
+    if (st == MST_OK) st = bits_b.alloc(h, words * 4, s);
+    if (st == MST_OK) st = ensure_status(h, words, s);
+    if (st != MST_OK) return record(h, st);
+    if (cudaMemsetAsync(bits_b.p, 0, words * 4, s) != cudaSuccess) return record_cuda(h, __LINE__);
+    char *b = scr_b.as<char>();
+    BlockArgs a{};
+    a.gn = d_n;
+    a.edge_off = d_edge_off;
+    a.vert_off = d_voff;
+    a.src = d_src;
+    a.dst = d_dst;
+    a.w = d_w;
+    a.m_total = m;
+    a.order = order;
+    a.key = (u64 *)b;
+    a.ends0 = (uint2 *)(b + 2 * stride);
+    a.uv = (uint32_t *)(b + 4 * stride);
+    a.gbest = (u64 *)(b + 5 * stride);
+    a.bits = bits_b.as<uint32_t>();
+    a.totals = (u64 *)d_total_weight;
+    a.sizes = sizes;
+    a.solved = solved;
+    a.err = &h->ds->err;
+    mst_ctx *c = h;
+    bool ok = true;
+    // The three kinds run side by side: a kind's last blocks leave SMs idle
+    // that the next kind's fill.
+    const bool fork = kinds[0] + kinds[1] + kinds[2] >= (uint64_t)h->sms;
+    if (fork && !h->kind_ev[2]) {
+      for (int k = 0; k < 2; ++k)
+        if (!h->kind_stream[k] && cudaStreamCreateWithFlags(&h->kind_stream[k], cudaStreamNonBlocking) != cudaSuccess)
+          return record_cuda(h, __LINE__);
+      for (int k = 0; k < 3; ++k)
+        if (!h->kind_ev[k] && cudaEventCreateWithFlags(&h->kind_ev[k], cudaEventDisableTiming) != cudaSuccess)
+          return record_cuda(h, __LINE__);
+    }
+    const int p = prof_begin(c, s, MST_K_BASE);
+    if (fork && cudaEventRecord(h->kind_ev[2], s) != cudaSuccess) return record_cuda(h, __LINE__);
+    for (int kind = 0; kind < 3; ++kind) {
+      a.num = (uint32_t)kinds[kind];
+      a.queue = queue + kind;
+      const bool own = fork && kind > 0 && a.num > 0;
+      cudaStream_t ks = own ? h->kind_stream[kind - 1] : s;
+      if (own) ok = ok && cudaStreamWaitEvent(ks, h->kind_ev[2], 0) == cudaSuccess;
+      ok = ok && launch_block_batch(a, kind, ks);
+      if (own)  // s goes on after every kind, also after an error
+        ok = cudaEventRecord(h->kind_ev[kind - 1], ks) == cudaSuccess &&
+             cudaStreamWaitEvent(s, h->kind_ev[kind - 1], 0) == cudaSuccess && ok;
+      a.first += a.num;
+    }
+    prof_end(c, s, p, MST_K_BASE, 12.0 * (double)mblk);
+    if (!ok) return record_cuda(h, __LINE__);
+    if (mblk == m) {  // every graph: straight to the output
+      ++h->solves;
+      batch_msf_off_kernel<<<1, TAB_THREADS, 0, s>>>(sizes, num_graphs, d_msf_off);
+      batch_emit_kernel<<<(unsigned)std::min<uint64_t>(num_graphs, (uint64_t)h->sms * 4), EMIT_THREADS, 0, s>>>(
+          bits_b.as<uint32_t>(), d_edge_off, order, num_graphs, d_msf_off, queue + 3, d_msf_ids);
+      return record(h, readback(h, s));
+    }
+  }
+  st = union_ids();
+  if (st != MST_OK) return record(h, st);
+  {  // the disjoint union of the (other) graphs
+    Buf uni_b, gb_b;
+    const uint64_t stride = round_up(m * 4 + 16, 256);
+    st = uni_b.alloc(h, stride * 2, s);
+    if (st == MST_OK && use_blocks) st = gb_b.alloc(h, words * 4, s);
+    if (st != MST_OK) return record(h, st);
+    uint32_t *usrc = uni_b.as<uint32_t>(), *udst = (uint32_t *)((char *)uni_b.p + stride);
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((m + 2047) / 2048, (uint64_t)h->sms * 8));
+    if (m > 0)
+      batch_offset_kernel<<<grid, 256, 0, s>>>(d_src, d_dst, d_edge_off, d_voff, usrc, udst, d_n, num_graphs, m,
+                                               use_blocks ? solved : nullptr, &h->ds->err);
+    st = readback(h, s);
+    if (st != MST_OK) return record(h, st);
+    if (use_blocks && cudaMemsetAsync(gb_b.p, 0, words * 4, s) != cudaSuccess) return record_cuda(h, __LINE__);
+    st = solve_device(h, n, m, usrc, udst, d_w, use_blocks ? nullptr : ids, d_count, d_sum, s,
+                      use_blocks ? gb_b.as<uint32_t>() : nullptr);
+    if (st != MST_OK) return record(h, st);
+    if (use_blocks) {
+      ++h->solves;
+      or_bits_kernel<<<(unsigned)std::min<uint64_t>((words + 255) / 256, (uint64_t)h->sms * 8), 256, 0, s>>>(
+          bits_b.as<uint32_t>(), gb_b.as<uint32_t>(), words);
+    }
+  }
+  if (use_blocks)
+    launch_finalize(bits_b.as<uint32_t>(), m, nullptr, ids, d_count, d_sum, next_scan(h, CNT_AUX), s);
   batch_seg_kernel<<<(num_graphs + 1 + 255) / 256, 256, 0, s>>>(ids, d_count, d_edge_off, num_graphs, d_msf_off);
   const unsigned sgrid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((cap + 2047) / 2048, (uint64_t)h->sms * 8));
-  batch_split_kernel<<<sgrid, 256, 0, s>>>(ids, d_count, d_edge_off, num_graphs, d_w, d_msf_ids, (u64 *)d_total_weight);
-  if (cudaStreamSynchronize(s) != cudaSuccess) return record_cuda(h, __LINE__);
-  return record(h, MST_OK);
+  batch_split_kernel<<<sgrid, 256, 0, s>>>(ids, d_count, d_edge_off, num_graphs, d_w, use_blocks ? solved : nullptr,
+                                           d_msf_ids, (u64 *)d_total_weight);
+  return record(h, readback(h, s));
 }
 
 // ---------------------------------------------------------------- steps
