@@ -16,6 +16,13 @@
 // Keys are w << pb | position in the list being contracted; the lists keep the
 // order of the edge ids, so keys order edges by (w, id).  They take 32 bits
 // where the graph's weights allow (w <= 255 and up to 2^22 edges), else 64.
+//
+// GB300, 4096 graphs of 2^8 to 2^16 vertices (337 M edges): 12.1 ms as a union,
+// 5.5 ms here, of which 0.14 ms for the ids.  What bounds it is latency between
+// barriers with one or two graphs per SM: half of the issue slots and half of
+// L1's throughput are used (ncu, 224 KB blocks).  An edge's record is one
+// 16-byte store and a live edge 8 bytes (three arrays: 5.63 ms); separate warps'
+// lists instead of block-wide ones behind a scan: 5.63 against 5.95 ms.
 #include <algorithm>
 #include <cstdint>
 
@@ -56,9 +63,8 @@ struct Shared {
 struct Work {
   uint32_t n, m;
   uint64_t off;          // position of the graph's first edge
-  uint2 *ends0;          // ends (16 bits each) and edge id of a listed edge, by position
-  u64 *key;              // the warps' live edges: keys (as 32-bit words for 32-bit keys)
-  uint32_t *uv;          // and ends
+  uint4 *ent;            // a listed edge by position: ends (16 bits each), edge id, weight
+  uint2 *live;           // the warps' live edges: ends, key (64-bit keys: position)
   u64 *gbest;            // [n] minima that do not fit shared memory
   // this warp's edges, as positions from the graph's first edge rounded down to
   // a multiple of four (that is skip edges earlier)
@@ -123,7 +129,6 @@ template <class K, bool HEAVY>
 __device__ __forceinline__ uint32_t stream_pass(const BlockArgs &a, const Work &g, uint32_t pw, uint32_t pb,
                                                 uint32_t wlim, const uint16_t *lab, K *best, bool relax,
                                                 uint32_t &bad) {
-  K *gkey = reinterpret_cast<K *>(g.key);
   const uint64_t first = g.off - g.skip;
   const uint32_t *ps = a.src + first, *pd = a.dst + first, *pw4 = a.w + first;
   const uint32_t lim = (uint32_t)min(a.m_total - first, (uint64_t)0xffffffffu);
@@ -145,7 +150,7 @@ __device__ __forceinline__ uint32_t stream_pass(const BlockArgs &a, const Work &
       load4(pd, j + 128, lo, hi, lim, vec, nv);
       load4(pw4, j + 128, lo, hi, lim, vec, nw);
     }
-    uint32_t keep = 0, cu[4], cv[4];
+    uint32_t keep = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const bool in = j + k >= lo && j + k < hi;
@@ -158,9 +163,7 @@ __device__ __forceinline__ uint32_t stream_pass(const BlockArgs &a, const Work &
         if (sizeof(K) == 4 && w[k] >= wlim) bad |= 2u;
       }
       ok = ok && (HEAVY ? w[k] > pw : (w[k] <= pw && u[k] != v[k]));
-      cu[k] = HEAVY ? (ok ? lab[u[k]] : 0u) : u[k];
-      cv[k] = HEAVY ? (ok ? lab[v[k]] : 0u) : v[k];
-      if (HEAVY) ok = ok && cu[k] != cv[k];
+      if (HEAVY) ok = ok && lab[u[k]] != lab[v[k]];
       keep |= (ok ? 1u : 0u) << k;
     }
     const uint32_t c = (uint32_t)__popc(keep);
@@ -172,34 +175,47 @@ __device__ __forceinline__ uint32_t stream_pass(const BlockArgs &a, const Work &
     }
     uint32_t p = g.base + len + incl - c;
     len += __shfl_sync(0xffffffffu, incl, 31);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (!(keep >> k & 1)) continue;
-      const K key = ((K)w[k] << pb) | p;
-      g.ends0[p] = make_uint2(u[k] | (v[k] << 16), j + k - g.skip);
-      g.uv[p] = u[k] | (v[k] << 16);
-      gkey[p] = key;
+    // few lanes keep more than one edge: as many steps as the busiest one has
+    for (; keep; keep &= keep - 1, ++p) {
+      const uint32_t k = (uint32_t)__ffs(keep) - 1;
+      const uint32_t x = k & 2 ? (k & 1 ? u[3] : u[2]) : (k & 1 ? u[1] : u[0]);
+      const uint32_t y = k & 2 ? (k & 1 ? v[3] : v[2]) : (k & 1 ? v[1] : v[0]);
+      const uint32_t z = k & 2 ? (k & 1 ? w[3] : w[2]) : (k & 1 ? w[1] : w[0]);
+      g.ent[p] = make_uint4(x | (y << 16), j + k - g.skip, z, 0);
       if (relax) {
-        if (key < best[cu[k]]) atomicMin(best + cu[k], key);
-        if (key < best[cv[k]]) atomicMin(best + cv[k], key);
+        const K key = ((K)z << pb) | p;
+        const uint32_t c0 = HEAVY ? lab[x] : x, c1 = HEAVY ? lab[y] : y;
+        if (key < best[c0]) atomicMin(best + c0, key);
+        if (key < best[c1]) atomicMin(best + c1, key);
       }
-      ++p;
     }
   }
   __syncwarp();
   return len;
 }
 
+// Ends and key of the warp's live edge i (first: the list as the pass left it).
+template <class K>
+__device__ __forceinline__ uint32_t live_edge(const Work &g, uint32_t i, uint32_t pb, bool first, K &key) {
+  if (first) {
+    const uint4 e = g.ent[g.base + i];
+    key = ((K)e.z << pb) | (g.base + i);
+    return e.x;
+  }
+  const uint2 e = g.live[g.base + i];
+  key = sizeof(K) == 4 ? (K)e.y : ((K)g.ent[e.y].z << pb) | e.y;
+  return e.x;
+}
+
 // The minima of the live edges over components [lo, hi) into best[0..hi-lo).
 template <int T, class K>
-__device__ __forceinline__ void relax_range(const Work &g, uint32_t len, bool identity, const uint16_t *lab,
-                                            uint32_t lo, uint32_t hi, K *best) {
-  const K *gkey = reinterpret_cast<const K *>(g.key) + g.base;
+__device__ __forceinline__ void relax_range(const Work &g, uint32_t len, uint32_t pb, bool first, bool identity,
+                                            const uint16_t *lab, uint32_t lo, uint32_t hi, K *best) {
   for (uint32_t i = threadIdx.x; i < hi - lo; i += T) best[i] = Entry<K>::INF;
   __syncthreads();
   for (uint32_t i = threadIdx.x & 31; i < len; i += 32) {
-    const uint32_t x = g.uv[g.base + i];
-    const K key = gkey[i];
+    K key;
+    const uint32_t x = live_edge<K>(g, i, pb, first, key);
     const uint32_t c0 = identity ? (x & 0xffffu) : lab[x & 0xffffu], c1 = identity ? (x >> 16) : lab[x >> 16];
     if (c0 >= lo && c0 < hi && key < best[c0 - lo]) atomicMin(best + (c0 - lo), key);
     if (c1 >= lo && c1 < hi && key < best[c1 - lo]) atomicMin(best + (c1 - lo), key);
@@ -222,13 +238,17 @@ __device__ __forceinline__ uint32_t contract(const BlockArgs &a, const Work &g, 
   volatile K *vb = B;
   for (uint32_t b = threadIdx.x; b < k; b += Q * T) {
     K key[Q], ob[Q];
-    uint2 e[Q];
+    uint2 e[Q];  // ends and edge id
     uint32_t other[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       const uint32_t c = b + q * T;
       key[q] = c < k ? vb[c] : (K)Entry<K>::INF;
-      e[q] = key[q] != Entry<K>::INF ? g.ends0[(uint32_t)key[q] & pmask] : make_uint2(0, 0);
+      e[q] = make_uint2(0, 0);
+      if (key[q] != Entry<K>::INF) {
+        const uint4 t = g.ent[(uint32_t)key[q] & pmask];
+        e[q] = make_uint2(t.x, t.y);
+      }
     }
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
@@ -266,9 +286,9 @@ __device__ __forceinline__ uint32_t contract(const BlockArgs &a, const Work &g, 
     live += x == Entry<K>::ROOT ? 1u : 0u;
     dead += x == Entry<K>::LONE ? 1u : 0u;
   }
-  uint32_t total;
+  uint32_t total, dead_total;
   uint32_t id = scan<T>(sh, flip, live, total);
-  uint32_t dd = dead ? atomicAdd(&sh.dead, dead) : 0u;
+  uint32_t dd = sh.dead + scan<T>(sh, flip, dead, dead_total);
 #pragma unroll 4
   for (uint32_t c = c0; c < c1; ++c) {
     const K x = B[c];
@@ -278,6 +298,7 @@ __device__ __forceinline__ uint32_t contract(const BlockArgs &a, const Work &g, 
       B[c] = Entry<K>::ROOT | (DEAD_TOP - dd++);
   }
   __syncthreads();
+  if (threadIdx.x == 0) sh.dead += dead_total;  // (read again after later barriers)
   // pointer jumping: every pass reaches (JSTEPS + 1) times as far
   for (int pass = 0; pass < 32; ++pass) {
     bool left = false;
@@ -308,13 +329,12 @@ __device__ __forceinline__ uint32_t contract(const BlockArgs &a, const Work &g, 
   return total;
 }
 
-// Drops the edges inside components from the warp's list, in place; relaxes
-// the others into best[] in shared memory if asked to.  Returns the list's new
-// length.
+// Drops the edges inside components from the warp's list, in place (first:
+// from the list as the pass left it); relaxes the others into best[] in shared
+// memory if asked to.  Returns the list's new length.
 template <class K>
-__device__ __forceinline__ uint32_t drop_inner(const Work &g, uint32_t len, const uint16_t *lab, K *best, bool relax) {
-  K *gkey = reinterpret_cast<K *>(g.key) + g.base;
-  uint32_t *uv = g.uv + g.base;
+__device__ __forceinline__ uint32_t drop_inner(const Work &g, uint32_t len, uint32_t pb, bool first,
+                                               const uint16_t *lab, K *best, bool relax) {
   const int lane = threadIdx.x & 31;
   const uint32_t below = (1u << lane) - 1u;
   uint32_t kept = 0;
@@ -324,8 +344,8 @@ __device__ __forceinline__ uint32_t drop_inner(const Work &g, uint32_t len, cons
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const uint32_t i = t0 + q * 32 + lane;
-      x[q] = i < len ? uv[i] : 0u;
-      key[q] = i < len ? gkey[i] : 0;
+      x[q] = 0, key[q] = 0;
+      if (i < len) x[q] = live_edge<K>(g, i, pb, first, key[q]);
     }
     __syncwarp();  // every lane has read its edges: survivors overwrite them
 #pragma unroll
@@ -334,9 +354,8 @@ __device__ __forceinline__ uint32_t drop_inner(const Work &g, uint32_t len, cons
       const bool ok = t0 + q * 32 + lane < len && c0 != c1;
       const uint32_t b = __ballot_sync(0xffffffffu, ok);
       if (ok) {
-        const uint32_t p = kept + __popc(b & below);
-        uv[p] = x[q];
-        gkey[p] = key[q];
+        g.live[g.base + kept + __popc(b & below)] =
+            make_uint2(x[q], sizeof(K) == 4 ? (uint32_t)key[q] : (uint32_t)key[q] & ((1u << pb) - 1u));
         if (relax) {
           if (key[q] < best[c0]) atomicMin(best + c0, key[q]);
           if (key[q] < best[c1]) atomicMin(best + c1, key[q]);
@@ -372,12 +391,12 @@ __device__ __forceinline__ void rounds(const BlockArgs &a, const Work &g, Shared
     if (spilled) {  // ranges of components in turn, collected in global memory
       for (uint32_t lo = 0; lo < k; lo += cap) {
         const uint32_t hi = min(k, lo + cap);
-        relax_range<T, K>(g, len, identity, lab, lo, hi, B);
+        relax_range<T, K>(g, len, pb, round == 0, identity, lab, lo, hi, B);
         for (uint32_t i = threadIdx.x; i < hi - lo; i += T) gb[lo + i] = B[i];
         __syncthreads();
       }
     } else if (!relaxed) {
-      relax_range<T, K>(g, len, identity, lab, 0, k, B);
+      relax_range<T, K>(g, len, pb, round == 0, identity, lab, 0, k, B);
     }
     const uint32_t live = spilled ? contract<T, K>(a, g, sh, flip, gb, k, pb, identity, lab, wacc, chosen)
                                   : contract<T, K>(a, g, sh, flip, B, k, pb, identity, lab, wacc, chosen);
@@ -412,7 +431,7 @@ __device__ __forceinline__ void rounds(const BlockArgs &a, const Work &g, Shared
     if (relaxed)
       for (uint32_t i = threadIdx.x; i < k; i += T) behind[i] = Entry<K>::INF;
     __syncthreads();
-    len = drop_inner<K>(g, len, lab, behind, relaxed);
+    len = drop_inner<K>(g, len, pb, round == 0, lab, behind, relaxed);
   }
 }
 
@@ -511,7 +530,7 @@ __global__ void __launch_bounds__(T, MINB) block_batch_kernel(const __grid_const
     if (i >= a.num) return;
     const uint32_t gi = a.order[a.first + i];
     const uint64_t off = a.edge_off[gi], v0 = a.vert_off[gi];
-    const Work g{a.gn[gi], (uint32_t)(a.edge_off[gi + 1] - off), off, a.ends0 + off, a.key + off, a.uv + off,
+    const Work g{a.gn[gi], (uint32_t)(a.edge_off[gi + 1] - off), off, a.ent + off, a.live + off,
                  a.gbest + v0, 0, 0, 0, 0};
     if (g.m > 0 && g.n > 0) {
       solve_graph<T>(a, g, sh, buf);
@@ -539,7 +558,7 @@ __global__ void __launch_bounds__(T, 1) block_single_kernel(const __grid_constan
   for (uint32_t i = threadIdx.x; i < words; i += T) a.bits[i] = 0;
   if (threadIdx.x == 0) *a.err = 0;
   __syncthreads();
-  const Work g{n, m, 0, a.ends0, a.key, a.uv, a.gbest, 0, 0, 0, 0};
+  const Work g{n, m, 0, a.ent, a.live, a.gbest, 0, 0, 0, 0};
   solve_graph<T>(a, g, sh, buf);
   __threadfence_block();
   __syncthreads();

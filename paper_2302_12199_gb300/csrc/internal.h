@@ -288,9 +288,8 @@ struct BlockArgs {
   const uint32_t *order;       // graphs, largest first
   uint32_t first, num;         // this launch's part of order
   uint32_t *queue;             // zero before the launch
-  uint2 *ends0;                // [m_total] scratch
-  uint32_t *uv;                // [m_total] scratch
-  u64 *key;                    // [m_total] scratch
+  uint4 *ent;                  // [m_total] scratch
+  uint2 *live;                 // [m_total] scratch
   u64 *gbest;                  // [vertices] scratch
   uint32_t *bits;              // chosen-edge bitmap
   u64 *totals;                 // forest weight and size, and 1 in solved, of each graph

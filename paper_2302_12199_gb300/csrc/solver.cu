@@ -456,8 +456,8 @@ mst_status zero_round_state(mst_ctx *c, cudaStream_t s) {
 // asks for other passes: one launch and one readback.
 constexpr uint64_t SINGLE_MAX_M = 1ULL << 15;
 constexpr uint32_t SINGLE_MAX_N = BLOCK_SMALL_N;
-constexpr size_t SMALL_KEY = SINGLE_MAX_M * 8, SMALL_ARR = SINGLE_MAX_M * 4, SMALL_BEST = SINGLE_MAX_N * 8;
-constexpr size_t SMALL_BYTES = SMALL_KEY + SMALL_BEST + 3 * SMALL_ARR + SINGLE_MAX_M / 8;
+constexpr size_t SMALL_BYTES = SINGLE_MAX_M * (sizeof(uint4) + sizeof(uint2)) + SINGLE_MAX_N * sizeof(u64) +
+                               SINGLE_MAX_M / 8;
 bool block_solves(const mst_config &f) {
   return f.base_case && f.graph_rounds && f.tile_contract == 0 && !f.min_edges_sort && f.dedupe != MST_DEDUPE_HASH &&
          f.dedupe != MST_DEDUPE_SORT;
@@ -1396,11 +1396,10 @@ mst_status solve_small(mst_ctx *c, uint32_t n, uint32_t m, const uint32_t *src, 
   a.dst = dst;
   a.w = w;
   a.m_total = m;
-  a.key = (u64 *)b;
-  a.gbest = (u64 *)(b += SMALL_KEY);
-  a.ends0 = (uint2 *)(b += SMALL_BEST);
-  a.uv = (uint32_t *)(b += 2 * SMALL_ARR);
-  a.bits = (uint32_t *)(b += SMALL_ARR);
+  a.ent = (uint4 *)b;
+  a.live = (uint2 *)(b += SINGLE_MAX_M * sizeof(uint4));
+  a.gbest = (u64 *)(b += SINGLE_MAX_M * sizeof(uint2));
+  a.bits = (uint32_t *)(b += SINGLE_MAX_N * sizeof(u64));
   a.totals = total_weight;
   a.err = &c->ds->err;
   PROF(MST_K_BASE, 12.0 * (double)m + 4.0 * (double)n, -1, 0.0, -1, 0.0,
@@ -1918,7 +1917,18 @@ mst_status mst_create(mst_handle *out, const mst_config *cfg) {
     uint64_t thr = ~0ULL;
     ok = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &thr) == cudaSuccess;
   }
-  ok = ok && cudaMalloc(&c->ds, sizeof(DevState)) == cudaSuccess;
+  // the fixed-size device state, in one allocation
+  const size_t b_ds = round_up(sizeof(DevState), 256), b_piv = round_up(pivot_scratch_bytes(), 256),
+               b_ws = round_up(WSUM_SLOTS * sizeof(u64), 256), b_rs = round_up(sizeof(RoundsState), 256);
+  char *fixed = nullptr;
+  ok = ok && cudaMalloc(&fixed, b_ds + b_piv + b_ws + b_rs + SMALL_BYTES) == cudaSuccess;
+  if (ok) {
+    c->ds = (DevState *)fixed;
+    c->pivot_scratch = fixed + b_ds;
+    c->wsum = (u64 *)(fixed + b_ds + b_piv);
+    c->rstate = (RoundsState *)(fixed + b_ds + b_piv + b_ws);
+    c->small_mem = fixed + b_ds + b_piv + b_ws + b_rs;
+  }
   ok = ok && cudaMemset(c->ds, 0, sizeof(DevState)) == cudaSuccess;
   ok = ok && cudaHostAlloc(&c->hs, sizeof(DevState), cudaHostAllocMapped) == cudaSuccess;
   ok = ok && cudaHostGetDevicePointer((void **)&c->hs_dev, c->hs, 0) == cudaSuccess;
@@ -1927,10 +1937,6 @@ mst_status mst_create(mst_handle *out, const mst_config *cfg) {
   if (ok) *c->hflag = 0;
   ok = ok && cudaMallocHost(&c->hres, 2 * sizeof(u64)) == cudaSuccess;
   ok = ok && ensure_sample(c) == MST_OK;
-  ok = ok && cudaMalloc(&c->pivot_scratch, pivot_scratch_bytes()) == cudaSuccess;
-  ok = ok && cudaMalloc(&c->wsum, WSUM_SLOTS * sizeof(u64)) == cudaSuccess;
-  ok = ok && cudaMalloc(&c->small_mem, SMALL_BYTES) == cudaSuccess;
-  ok = ok && cudaMalloc(&c->rstate, sizeof(RoundsState)) == cudaSuccess;
   ok = ok && cudaDeviceSynchronize() == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -1946,7 +1952,7 @@ void mst_destroy(mst_handle h) {
   {
     DeviceGuard g(h->device);
     cudaDeviceSynchronize();
-    if (h->ds) cudaFree(h->ds);
+    if (h->ds) cudaFree(h->ds);  // with the rest of the fixed-size state
     if (h->hs) cudaFreeHost(h->hs);
     if (h->hflag) cudaFreeHost(h->hflag);
     if (h->hres) cudaFreeHost(h->hres);
@@ -1956,19 +1962,15 @@ void mst_destroy(mst_handle h) {
     if (h->rl_mem) cudaFree(h->rl_mem);
     if (h->status) cudaFree(h->status);
     if (h->sample_buf) cudaFree(h->sample_buf);
-    if (h->pivot_scratch) cudaFree(h->pivot_scratch);
-    if (h->wsum) cudaFree(h->wsum);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
     for (int k = 0; k < 2; ++k) {
       if (h->in_ready[k]) cudaEventDestroy(h->in_ready[k]);
       if (h->in_free[k]) cudaEventDestroy(h->in_free[k]);
     }
-    if (h->rstate) cudaFree(h->rstate);
     for (cudaStream_t ks : h->kind_stream)
       if (ks) cudaStreamDestroy(ks);
     for (cudaEvent_t e : h->kind_ev)
       if (e) cudaEventDestroy(e);
-    if (h->small_mem) cudaFree(h->small_mem);
     if (h->pool) cudaMemPoolDestroy(h->pool);
     for (auto &r : h->prof_pending) {
       if (r.a) h->ev_pool.push_back(r.a);
@@ -2252,8 +2254,8 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
   const bool use_blocks = blocks && m > 0 && 2 * mblk >= m;
   if (use_blocks) {
     Buf scr_b;
-    const uint64_t stride = round_up(m * 4 + 16, 256);
-    st = scr_b.alloc(h, stride * 5 + (size_t)n * 8 + 256, s);
+    const uint64_t ent_bytes = round_up(m * sizeof(uint4), 256), live_bytes = round_up(m * sizeof(uint2), 256);
+    st = scr_b.alloc(h, ent_bytes + live_bytes + (size_t)n * sizeof(u64) + 256, s);
     if (st == MST_OK) st = bits_b.alloc(h, words * 4, s);
     if (st == MST_OK) st = ensure_status(h, words, s);
     if (st != MST_OK) return record(h, st);
@@ -2268,10 +2270,9 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
     a.w = d_w;
     a.m_total = m;
     a.order = order;
-    a.key = (u64 *)b;
-    a.ends0 = (uint2 *)(b + 2 * stride);
-    a.uv = (uint32_t *)(b + 4 * stride);
-    a.gbest = (u64 *)(b + 5 * stride);
+    a.ent = (uint4 *)b;
+    a.live = (uint2 *)(b + ent_bytes);
+    a.gbest = (u64 *)(b + ent_bytes + live_bytes);
     a.bits = bits_b.as<uint32_t>();
     a.totals = (u64 *)d_total_weight;
     a.sizes = sizes;
