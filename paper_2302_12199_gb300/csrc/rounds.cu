@@ -38,6 +38,15 @@ constexpr uint32_t RPASSES = 256;       // jump passes per round (each multiplie
 // components left took 46 us, most of it those atomics queueing; 12 us with
 // the table.
 constexpr uint32_t STAB = 4096;
+// Components up to which a round keeps only the lightest edge between each two
+// (pair_phase): their pairs and the byte labels fill the shared memory that a
+// block has anyway.
+constexpr uint32_t PAIR_COMPS = 124, PAIRS = PAIR_COMPS * (PAIR_COMPS - 1) / 2;
+constexpr uint32_t NO_PAIRS = 0xffffffffu;
+// Labels of up to LABS components are then read from shared memory.  A gather
+// answered by L1 costs a cycle per line, so up to 32 per warp, however few
+// lines the table has; in shared memory about four.
+constexpr uint32_t LABS = 4096;
 // A call's last rounds run in one block from this size on.
 constexpr uint64_t SOLO_EDGES = 4096, SOLO_VERTS = 4096;
 constexpr uint32_t BAR_SPINS = 1u << 24;  // polls of the grid barrier before giving up
@@ -46,6 +55,7 @@ struct Smem {
   uint32_t out[4][RT];  // a tile's survivors (hooking: its vertices)
   u64 tab[STAB];        // per-block minima of a round with few components
 };
+static_assert(PAIRS * sizeof(u64) + LABS <= sizeof(Smem), "pairs and labels fit");
 
 // All blocks of the launch are resident (cooperative launch), so a wait for
 // the others ends; it is bounded all the same.
@@ -424,6 +434,145 @@ __device__ __forceinline__ void relabel_phase(const RoundsArgs &a, KeyLayout kl,
   }
 }
 
+// Clears the pairs' table.  It lies where the round's survivors would have gone
+// (room for all of the round's edges, at least 4 np entries of 4 bytes).
+__device__ __noinline__ void pair_clear(uint32_t *table_mem, uint32_t np, uint32_t nb, uint32_t bid) {
+  for (uint32_t i = bid * RB + threadIdx.x; i < np; i += nb * RB) reinterpret_cast<u64 *>(table_mem)[i] = KEY_INF;
+}
+
+// Relabel of a round that leaves few components (at most PAIR_COMPS): of the
+// edges between two components only the lightest can be in the forest, so the
+// list shrinks to one entry per pair at once, and block 0 finishes the call
+// alone.  Every block collects its pairs' minima in shared memory and then
+// sends them to the table; nothing is staged or written per edge, and an edge's
+// id is read only where its weight is not above the pair's minimum.  Bound by
+// reading 12 bytes per edge: RMAT n=2^22 m=2^26, which keeps 64 million edges
+// until its last rounds, passes over them in 227 us (3.4 TB/s; the shared-memory
+// lookups are the rest), where relabel, minEdges and three more rounds took
+// 1260 us; GNM n=2^16 m=2^20 ends in 50 us instead of 75.  The pair functions
+// are calls, with their arguments by value: inlined, their registers cost the
+// long phases spills (RGG2D's first relabel 200 -> 223 us).
+template <int I>
+__device__ __noinline__ void pair_phase(EdgeList in, const uint32_t *link, uint64_t m, uint32_t nc, uint32_t np,
+                                        uint32_t *table_mem, uint32_t nb, uint32_t bid) {
+  extern __shared__ __align__(128) unsigned char smem_dyn[];
+  u64 *pt = reinterpret_cast<u64 *>(smem_dyn), *table = reinterpret_cast<u64 *>(table_mem);
+  const bool lab = nc <= LABS;
+  uint8_t *s_lab = reinterpret_cast<uint8_t *>(pt + PAIRS);
+  for (uint32_t i = threadIdx.x; i < np; i += RB) pt[i] = KEY_INF;
+  if (lab)
+    for (uint32_t i = threadIdx.x; i < nc; i += RB) s_lab[i] = (uint8_t)__ldca(link + i);
+  __syncthreads();
+  constexpr uint64_t T = (uint64_t)RB * I;
+  const uint64_t nfull = I == RI && aligned16_list(in) ? m / T : 0;
+  uint32_t fu[I], fv[I], fw[I];  // the next tile
+  const auto fetch = [&](uint64_t tile) {
+    const uint64_t j0 = tile * T + (uint64_t)I * threadIdx.x;
+    if constexpr (I == RI) {
+      if (tile < nfull) {
+        const uint4 x = __ldcg(reinterpret_cast<const uint4 *>(in.u + j0));
+        const uint4 y = __ldcg(reinterpret_cast<const uint4 *>(in.v + j0));
+        const uint4 z = __ldcg(reinterpret_cast<const uint4 *>(in.w + j0));
+        fu[0] = x.x, fu[1] = x.y, fu[2] = x.z, fu[3] = x.w;
+        fv[0] = y.x, fv[1] = y.y, fv[2] = y.z, fv[3] = y.w;
+        fw[0] = z.x, fw[1] = z.y, fw[2] = z.z, fw[3] = z.w;
+        return;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+      const bool ok = j0 + k < m;
+      fu[k] = ok ? __ldca(in.u + j0 + k) : 0u;
+      fv[k] = ok ? __ldca(in.v + j0 + k) : fu[k];
+      fw[k] = ok ? __ldca(in.w + j0 + k) : 0u;
+    }
+  };
+  fetch(bid);
+  for (uint64_t tile = bid; tile * T < m; tile += nb) {
+    const uint64_t j0 = tile * T + (uint64_t)I * threadIdx.x;
+    uint32_t pi[I], ew[I];  // pair (PAIRS: both ends in one component) and weight
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+      // the ends of an edge that is not there are equal
+      const uint32_t x = lab ? s_lab[fu[k]] : __ldca(link + fu[k]) & ~ROOT;
+      const uint32_t y = lab ? s_lab[fv[k]] : __ldca(link + fv[k]) & ~ROOT;
+      const uint32_t hi = max(x, y);
+      pi[k] = x == y ? PAIRS : hi * (hi - 1) / 2 + min(x, y);
+      ew[k] = fw[k];
+    }
+    fetch(tile + nb);
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+      if (pi[k] == PAIRS) continue;
+      const u64 cur = pt[pi[k]];
+      if (ew[k] > (uint32_t)(cur >> 32)) continue;
+      const u64 key = (u64)ew[k] << 32 | (in.id ? __ldca(in.id + j0 + k) : (uint32_t)(j0 + k));
+      if (key < cur) atomicMin(pt + pi[k], key);
+    }
+  }
+  __syncthreads();
+  // each block begins at another pair, so that they do not queue at the same ones
+  const uint32_t first = (uint32_t)((uint64_t)np * bid / nb);
+  for (uint32_t t = threadIdx.x; t < np; t += RB) {
+    const uint32_t i = t + first < np ? t + first : t + first - np;
+    const u64 k = pt[i];
+    if (k != KEY_INF) relax(table, i, k, __ldca(table + i));
+  }
+}
+
+// The pairs that have an edge as the next round's list, with its minEdges; one
+// block.  Returns the edges.
+__device__ __noinline__ uint32_t pair_list(EdgeOut out, KeyLayout kl, uint32_t *cur_u, uint32_t *cur_v, u64 *best,
+                                           uint32_t nn, uint32_t *s_warp) {
+  extern __shared__ __align__(128) unsigned char smem_dyn[];
+  u64 *pt = reinterpret_cast<u64 *>(smem_dyn);
+  const uint32_t np = nn * (nn - 1) / 2;
+  // the list overlays the table
+  for (uint32_t i = threadIdx.x; i < np; i += RB) pt[i] = __ldcg(reinterpret_cast<u64 *>(out.u) + i);
+  __syncthreads();
+  // warp w writes the pairs [w * per, (w + 1) * per)
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t per = ((np + RW - 1) / RW + 31u) & ~31u, i0 = wid * per, i1 = min(np, i0 + per);
+  uint32_t cnt = 0, total;
+  for (uint32_t b = i0; b < i1; b += 32)
+    cnt += __popc(__ballot_sync(0xffffffffu, b + lane < i1 && pt[b + lane] != KEY_INF));
+  uint32_t o = block_exclusive_scan<RB>(lane == 0 ? cnt : 0u, total, s_warp);
+  o = __shfl_sync(0xffffffffu, o, 0);
+  for (uint32_t b = i0; b < i1; b += 32) {
+    const uint32_t i = b + lane;
+    const u64 k = i < i1 ? pt[i] : KEY_INF;
+    const uint32_t has = __ballot_sync(0xffffffffu, k != KEY_INF);
+    if (k != KEY_INF) {
+      uint32_t hi = (uint32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)i)) * 0.5f);  // hi (hi - 1) / 2 <= i, one off at most
+      if (hi * (hi - 1) / 2 > i) --hi;
+      if (hi * (hi + 1) / 2 <= i) ++hi;
+      const uint32_t lo = i - hi * (hi - 1) / 2, id = (uint32_t)k, p = o + __popc(has & ((1u << lane) - 1u));
+      out.u[p] = hi, out.v[p] = lo, out.w[p] = (uint32_t)(k >> 32), out.id[p] = id;
+      if (!kl.packed) cur_u[id] = hi, cur_v[id] = lo;
+    }
+    o += __popc(has);
+  }
+  // minEdges: a warp per component, over its pairs
+  for (uint32_t c = wid; c < nn; c += RW) {
+    u64 k = KEY_INF;
+    uint32_t other = 0;
+    for (uint32_t d = lane; d < nn; d += 32) {
+      const uint32_t h = max(c, d);
+      const u64 q = c == d ? KEY_INF : pt[h * (h - 1) / 2 + min(c, d)];
+      if (q < k) k = q, other = d;
+    }
+#pragma unroll
+    for (int x = 16; x > 0; x >>= 1) {
+      const u64 q = __shfl_xor_sync(0xffffffffu, k, x);
+      const uint32_t d = __shfl_xor_sync(0xffffffffu, other, x);
+      if (q < k) k = q, other = d;
+    }
+    if (lane == 0 && k != KEY_INF) best[c] = relax_key(kl, (uint32_t)(k >> 32), (uint32_t)k, other);
+  }
+  __syncthreads();
+  return total;
+}
+
 // The call's vertices (act) back to representatives in the caller's numbering:
 // parent[v] = the representative of v's final component.
 __device__ __forceinline__ void compose_phase(const RoundsArgs &a, const uint64_t *s_off, int levels) {
@@ -447,6 +596,7 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
   __shared__ uint32_t s_warp[RW + 1], s_base[2];
   // the round's edges, vertices, next round's vertices, vertices to jump, and each round's part of link and rep
   __shared__ uint64_t s_m, s_nc, s_nn, s_cnt, s_off[ROUNDS_MAX + 2];
+  __shared__ uint32_t s_np;  // pairs of the next round's components, if the round ends by pairs
   GridSync g{gridDim.x, blockIdx.x, &a.st->bar, a.err, 0, gridDim.x == 1};
 
   const uint64_t m0 = a.m_dev ? min((uint64_t)*a.m_dev, a.m) : a.m;
@@ -482,6 +632,9 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
       s_nn = __ldca(&a.st->cv[r]);
       s_cnt = r == 0 ? __ldca(&a.st->ca) : s_nc;
       if (r > 0) s_off[r + 1] = s_off[r] + s_nc;
+      // pairs where they are few beside the edges
+      const uint32_t np = s_nn <= PAIR_COMPS ? (uint32_t)(s_nn * (s_nn - 1) / 2) : 0u;
+      s_np = s_nn <= PAIR_COMPS && s_m > SOLO_EDGES && s_m >= (uint64_t)4 * np ? np : NO_PAIRS;
     }
     __syncthreads();
     if (s_nn == 0) {  // no vertex had an edge
@@ -492,6 +645,7 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
       uint32_t *flag = &a.st->jflag[pass & 3];
       if (g.bid == 0 && threadIdx.x == 0) a.st->jflag[(pass + 2) & 3] = 0;
       jump_phase(a, r, s_cnt, s_off[r], tries == 0, flag, g.nb, g.bid);
+      if (tries == 0 && s_np != NO_PAIRS) pair_clear(a.list[(a.first_slot + r) & 1].u, s_np, g.nb, g.bid);
       if (!(ok = g.sync()) || !__ldca(flag)) break;
       if (tries >= RPASSES) {
         if (threadIdx.x == 0) atomicOr(a.err, ERR_JUMP);
@@ -501,6 +655,27 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
     }
     ++pass;
     if (!ok) break;
+    if (s_np != NO_PAIRS) {
+      const EdgeOut out = a.list[(a.first_slot + r) & 1], prev = a.list[(a.first_slot + r + 1) & 1];
+      const EdgeList in = r == 0 ? a.in : EdgeList{prev.u, prev.v, prev.w, prev.id};
+      const uint32_t *link = r == 0 ? a.parent : a.link + s_off[r];
+      if (s_m >= (uint64_t)RT * g.nb)
+        pair_phase<RI>(in, link, s_m, (uint32_t)s_nc, s_np, out.u, g.nb, g.bid);
+      else
+        pair_phase<1>(in, link, s_m, (uint32_t)s_nc, s_np, out.u, g.nb, g.bid);
+      if (!(ok = g.sync())) break;
+      alone = alone || !g.solo;
+      if (blockIdx.x != 0) break;
+      const uint32_t left = pair_list(out, kl, a.cur_u, a.cur_v, a.best, (uint32_t)s_nn, s_warp);
+      if (threadIdx.x == 0) {
+        s_m = left;
+        s_nc = s_nn;
+      }
+      __syncthreads();
+      g.solo = true;
+      g.nb = 1;
+      continue;
+    }
     const bool tab = s_nn <= STAB;
     if (tab) {
       for (uint32_t i = threadIdx.x; i < (uint32_t)s_nn; i += RB) sm.tab[i] = KEY_INF;
