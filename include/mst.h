@@ -101,8 +101,8 @@ typedef struct {
                                   half of a tile's edges first and drop heavy edges that fall inside a
                                   component (recursive filtering in local preprocessing, Section 6.2);
                                   0 (default, measured faster on GB300): every edge from the first round */
-  uint32_t spin_limit;         /* polls of a predecessor's status word in the ordered output scan before the
-                                  wait gives up (>= 1; default 2^21, about a second); a wait that runs out
+  uint32_t spin_limit;         /* polls of the barrier in the ordered output scan before the wait
+                                  gives up (>= 1; default 2^21, about a second); a wait that runs out
                                   makes the call return MST_ERR_INTERNAL.  Small values exist to exercise
                                   that error path */
   uint32_t block_threads;      /* threads per block of the relabel / partition compactions and the hooking

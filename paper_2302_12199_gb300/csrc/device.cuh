@@ -1,19 +1,8 @@
-// Device helpers shared by the kernel files: memory-order loads and stores, the
-// edge and relaxation keys, the block-wide scan and the weight counters.
+// Device helpers shared by the kernel files: the edge and relaxation keys, the block-wide scan and the weight counters.
 #pragma once
 #include "internal.h"
 
 namespace mstgpu {
-
-__device__ __forceinline__ u64 ld_relaxed(const u64 *p) {
-  u64 v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void st_relaxed(u64 *p, u64 v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
 
 __device__ __forceinline__ u64 edge_key(uint32_t w, uint32_t id) { return ((u64)w << 32) | (u64)id; }
 

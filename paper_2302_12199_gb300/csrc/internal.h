@@ -12,7 +12,7 @@ constexpr u64 KEY_INF = ~0ULL;
 // Device-side error bits, latched in DevState::err.
 enum : uint32_t {
   ERR_VERTEX = 1u,    // an input vertex id >= n
-  ERR_LOOKBACK = 2u,  // a scan predecessor never published (bounded wait ran out)
+  ERR_LOOKBACK = 2u,  // the output scan's barrier was not reached in time (bounded wait ran out)
   ERR_HASH = 4u,      // hash table probe sequence exhausted
   ERR_JUMP = 8u,      // pointer doubling did not reach a root within its bound
   ERR_TMA = 16u,      // a bulk copy never completed (bounded mbarrier wait ran out); tiles were skipped
@@ -25,7 +25,7 @@ constexpr int LVL_MAX = 32;  // recursion levels of a planned Filter-Borůvka
 struct DevState {
   uint32_t err;
   uint32_t jump_flag;   // set when a pointer-jump launch left a vertex short of its root
-  uint32_t tile_ctr[2]; // reserved
+  uint32_t scan_ctr[2]; // blocks of the output scan that have arrived at its barrier, and that have ended
   u64 count[6 + 2 * LVL_MAX];  // counts written by the last tile of a scan kernel; from CNT_LVL on,
                                //   the list lengths of a planned Filter-Borůvka (see CNT_LVL)
   u64 pivot;            // result of the pivot selection
@@ -46,15 +46,15 @@ enum { CNT_EDGES = 0, CNT_ACTIVE = 1, CNT_TMP = 2, CNT_AUX = 3, CNT_USER = 4, CN
 
 // Output bookkeeping of a compaction launch.  Unordered compactions claim
 // their output ranges by atomic adds on *total (zero before the launch); the
-// ordered scan of the output ids uses the look-back status words, and its last
-// tile writes *total.
+// ordered scan of the output ids exchanges its blocks' counts and writes *total.
+constexpr int FINISH_BLOCKS = 1024;  // of the ordered scan, at most
 struct ScanState {
-  u64 *status;       // one status word per tile: epoch(30) | flag(2) | value(32)
-  uint32_t *tile_ctr;  // unused
-  uint32_t epoch;    // 1 .. 2^30-1, different for every ordered launch
+  uint32_t *count;     // [FINISH_BLOCKS] set bits of each block's words
+  uint32_t *arrived;   // blocks that have written theirs (zero between launches)
+  uint32_t *ended;     // blocks that have ended (zero between launches)
   u64 *total;
   uint32_t *err;
-  uint32_t spin_limit;  // polls of a predecessor's status word before the wait gives up (ERR_LOOKBACK)
+  uint32_t spin_limit;  // polls of the barrier before the wait gives up (ERR_LOOKBACK)
 };
 
 struct HashSlot {
@@ -162,7 +162,6 @@ inline uint32_t shape_tile(int shape) {
 constexpr int WSUM_SLOTS = 256;
 
 // ---- launchers (kernels.cu); all asynchronous on `s` ----
-int max_scan_tiles(uint64_t count);
 void launch_compact(CompactMode mode, const CompactArgs &a, uint64_t max_count, cudaStream_t s);
 // max_w: as in RoundsArgs.
 void launch_min_edges(EdgeList in, uint64_t m, uint32_t n, int validate, KeyLayout kl, u64 *best, uint32_t *err,
@@ -190,11 +189,34 @@ void launch_pivot(EdgeList in, uint64_t m, const u64 *m_dev, u64 state, uint32_t
 size_t pivot_scratch_bytes();
 bool launch_pivot_coop(EdgeList in, uint64_t m, u64 state, uint32_t sample, u64 *keys, void *scratch,
                        u64 *pivot_out, cudaStream_t s, const u64 *m_dev = nullptr, uint32_t rank = ~0u);
-// w == nullptr: ids and count only (total_weight untouched).
-void launch_finalize(const uint32_t *bits, uint64_t m, const uint32_t *w, uint32_t *out_ids, uint32_t *out_count,
-                     u64 *total_weight, ScanState st, cudaStream_t s);
-// *total = the sum of the WSUM_SLOTS counters.
-void launch_wsum_total(const u64 *wsum, u64 *total, cudaStream_t s);
+// What a solve starts from.
+struct InitArgs {
+  u64 *best;         // [n] KEY_INF
+  uint32_t *parent;  // [n] own index
+  uint32_t n;
+  uint32_t *bits;    // [words] zero
+  uint64_t words;
+  uint32_t *zero;    // [zero_words] zero: the handle's counters
+  uint64_t zero_words;
+};
+void launch_init(const InitArgs &a, int sms, cudaStream_t s);
+// The bitmap's ids in ascending order and their number.
+struct FinishArgs {
+  const uint32_t *bits;
+  uint64_t nwords;
+  const uint32_t *w;  // weights to add up into *total_weight (zero before), or nullptr
+  uint32_t *out_ids, *out_count;
+  u64 *total_weight;
+  ScanState st;
+  // with state: behind everything else the total from the WSUM_SLOTS counters
+  // (if wsum), the state to its host mirror, and seq to the host's flag
+  const u64 *wsum;
+  const DevState *state;
+  DevState *mirror;
+  uint32_t *flag;
+  uint32_t seq;
+};
+void launch_finish(const FinishArgs &a, int sms, cudaStream_t s);
 // The giant component's root: the most frequent root among the labels of
 // sampled edge ends (P is walked to the roots); launch_giant_bits also marks
 // its vertices (bit v set iff P[v] is that root; P fully contracted).
@@ -270,9 +292,11 @@ struct RoundsArgs {
   RoundsState *st;
   uint32_t *err;
 };
-// max_edges: bound on the list's length.  False if the launch was refused
-// (nothing ran).
-bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, int sms, cudaStream_t s);
+// States that a solve's start clears; its later launches clear the last again.
+constexpr int ROUNDS_STATES = 8;
+// max_edges: bound on the list's length; clear: a.st is not zero yet.  False if
+// the launch was refused (nothing ran).
+bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, bool clear, int sms, cudaStream_t s);
 
 // Whole graphs solved by one block each (block.cu).
 constexpr uint32_t BLOCK_MAX_N = 65536;   // 16-bit labels

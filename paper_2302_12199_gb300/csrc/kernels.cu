@@ -11,9 +11,9 @@
 // and claims its output range with one atomic add.  The filter pass streams
 // per warp instead (stream_warp_kernel).  Lists therefore come out in an
 // unspecified order; nothing downstream depends on list order, because edges
-// are keyed by id and a vertex finds its chosen edge through the input arrays.  The output ids (finalize) are the one
-// ordered compaction: a decoupled look-back scan (Merrill & Garland, 2016).
-// Every wait is bounded.
+// are keyed by id and a vertex finds its chosen edge through the input arrays.
+// The output ids (finish_kernel) are the one ordered compaction.  Every wait is
+// bounded.
 #include <algorithm>
 #include <cstdint>
 
@@ -71,138 +71,6 @@ __device__ __forceinline__ bool aligned16_dev(const void *p) { return ((uintptr_
 
 __device__ __forceinline__ u64 pair_of(uint32_t a, uint32_t b) {
   return a < b ? (((u64)a << 32) | b) : (((u64)b << 32) | a);
-}
-
-// Decoupled look-back by the whole block.  Publishes the tile's aggregate,
-// then examines LB_WINDOW = BLOCK * LB_PER_THREAD predecessors per round (each
-// thread polls LB_PER_THREAD status words, bounded), adds the values up to the
-// nearest tile whose inclusive prefix is published, and continues further back
-// only if none in the window has one; finally publishes its own inclusive
-// prefix and returns the exclusive one.  A window as wide as the number of
-// tiles in flight keeps the walk to one round.  Status word layout:
-// epoch (bits 63..34) | flag (33..32: 1 aggregate, 2 inclusive, 3 error) | value.
-constexpr int LB_PER_THREAD = 4;
-constexpr int LB_WINDOW = BLOCK * LB_PER_THREAD;
-
-struct LookbackShared {
-  uint32_t first;    // smallest window offset holding an inclusive prefix
-  uint32_t error;
-  uint32_t sum[BLOCK / 32];
-};
-
-__device__ uint32_t decoupled_lookback(const ScanState &st, uint32_t tile, uint32_t aggregate, bool &error,
-                                       LookbackShared &sh) {
-  const u64 tag = (u64)st.epoch << 34;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (tile == 0) {
-    if (threadIdx.x == 0) st_relaxed(&st.status[0], tag | (2ULL << 32) | aggregate);
-    error = false;
-    return 0;
-  }
-  if (threadIdx.x == 0) st_relaxed(&st.status[tile], tag | (1ULL << 32) | aggregate);
-  uint32_t exclusive = 0;
-  long long top = (long long)tile - 1;  // newest predecessor of the current window
-  for (;;) {
-    if (threadIdx.x == 0) {
-      sh.first = LB_WINDOW;
-      sh.error = 0;
-    }
-    __syncthreads();
-    uint32_t val[LB_PER_THREAD], flag[LB_PER_THREAD];
-#pragma unroll
-    for (int k = 0; k < LB_PER_THREAD; ++k) {
-      const long long pred = top - (long long)(k * BLOCK + threadIdx.x);  // window offset k*BLOCK+tid
-      val[k] = 0;
-      flag[k] = 2;
-      if (pred >= 0) {
-        uint32_t spins = 0;
-        for (;;) {
-          const u64 s = ld_relaxed(&st.status[pred]);
-          flag[k] = ((uint32_t)(s >> 34) == st.epoch) ? (uint32_t)((s >> 32) & 3u) : 0u;
-          val[k] = (uint32_t)s;
-          if (flag[k] != 0) break;
-          if (++spins >= st.spin_limit) {  // bounded: the predecessor never published
-            flag[k] = 3;
-            break;
-          }
-          __nanosleep(32);
-        }
-      }
-      if (flag[k] == 3) atomicOr(&sh.error, 1u);
-      if (flag[k] == 2) atomicMin(&sh.first, (uint32_t)(k * BLOCK + threadIdx.x));
-    }
-    __syncthreads();
-    if (sh.error) {
-      error = true;
-      break;
-    }
-    const uint32_t first = sh.first;
-    uint32_t part = 0;
-#pragma unroll
-    for (int k = 0; k < LB_PER_THREAD; ++k)
-      if ((uint32_t)(k * BLOCK + threadIdx.x) <= first) part += val[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if (lane == 0) sh.sum[wid] = part;
-    __syncthreads();
-    uint32_t win = 0;
-#pragma unroll
-    for (int i = 0; i < BLOCK / 32; ++i) win += sh.sum[i];
-    exclusive += win;
-    if (first < LB_WINDOW) {
-      error = false;
-      break;
-    }
-    top -= LB_WINDOW;
-    __syncthreads();  // sh.sum is rewritten in the next round
-  }
-  if (threadIdx.x == 0) {
-    if (error)
-      st_relaxed(&st.status[tile], tag | (3ULL << 32));
-    else
-      st_relaxed(&st.status[tile], tag | (2ULL << 32) | (u64)(exclusive + aggregate));
-  }
-  return exclusive;
-}
-
-// Tile bookkeeping shared by the scan kernels.  Tile t is processed by block t
-// (blocks are dispatched in index order, so every predecessor of a waiting
-// block is already resident or finished).  Returns false when this block has
-// no tile (the count is read on the device and the grid was sized for an upper
-// bound).
-struct TileInfo {
-  uint32_t tile, ntiles;
-};
-
-__device__ __forceinline__ bool acquire_tile(const ScanState &st, uint64_t count, TileInfo &t) {
-  t.ntiles = (uint32_t)((count + TILE - 1) / TILE);
-  t.tile = blockIdx.x;
-  if (t.tile >= t.ntiles) {
-    if (t.ntiles == 0 && t.tile == 0 && threadIdx.x == 0) *st.total = 0;
-    return false;
-  }
-  return true;
-}
-
-// Scan + look-back for one tile.  `packed` holds this thread's chunk-0 count in
-// the low and chunk-1 count in the high 16 bits (each block total is at most
-// TILE / 2, so the halves never carry).  Returns the packed exclusive scan, the
-// packed tile total and the tile's output offset; false on a look-back error
-// (the tile then writes nothing).
-__device__ __forceinline__ bool tile_offsets(const ScanState &st, const TileInfo &t, uint32_t packed,
-                                             uint32_t &excl_p, uint32_t &total_p, uint64_t &tile_base,
-                                             uint32_t *s_warp, LookbackShared &sh) {
-  excl_p = block_exclusive_scan(packed, total_p, s_warp);
-  const uint32_t tile_total = (total_p & 0xffffu) + (total_p >> 16);
-  bool err = false;
-  const uint32_t ex = decoupled_lookback(st, t.tile, tile_total, err, sh);
-  if (err) {
-    if (threadIdx.x == 0) atomicOr(st.err, ERR_LOOKBACK);
-    return false;
-  }
-  tile_base = ex;
-  if (t.tile == t.ntiles - 1 && threadIdx.x == 0) *st.total = tile_base + tile_total;
-  return true;
 }
 
 // Claims `total` output slots for this block's tile with one atomic add on the
@@ -1426,16 +1294,29 @@ __global__ void __launch_bounds__(SEL_THREADS) pivot_select_kernel(const u64 *ke
 }
 
 // The same selection spread over PSEL_BLOCKS blocks of a cooperative launch:
-// every thread draws its samples, then each pass histograms the next 12 bits
-// (below the bits shared by all candidates) in shared memory, adds the block's
-// bins to a global histogram, and after a grid-wide barrier every block reads
-// the histogram and fixes the same digit.  The first pass starts below the
-// bits that the sample's minimum and maximum share.
+// every thread draws its samples (the first stays in a register), then a pass
+// histograms the next 12 bits (below the bits shared by all candidates) in
+// shared memory, adds the block's bins to a global histogram, and after a
+// grid-wide barrier every block reads the histogram and fixes the same digit.
+// The first pass starts below the bits that the sample's minimum and maximum
+// share.  Once at most PSEL_CAND samples share the digits fixed so far (after
+// one pass unless many weights are equal), they are collected and block 0
+// ranks them by comparison: the passes over the remaining bits were all
+// barriers.  Latency-bound; 2^16 samples: 29 us with weights up to 255 (four
+// passes) and 38 us with 32-bit weights (six) before, 13 us now (18 where the
+// samples come cold from 3 GB).
+//
+// The scratch is all zero between launches: cleared at its allocation, and by
+// every launch behind its last reader.
 constexpr int PSEL_BLOCKS = 64, PSEL_THREADS = 1024, PSEL_BITS = 12, PSEL_BINS = 1 << PSEL_BITS;
+constexpr int PSEL_PASSES = (64 + PSEL_BITS - 1) / PSEL_BITS;
+constexpr uint32_t PSEL_CAND = 256;
 
 struct PivotScratch {
-  u64 min, max;
-  uint32_t hist[2][PSEL_BINS];
+  u64 nmin, max;     // ~(smallest key), largest key
+  uint32_t cands;    // collected candidates
+  u64 cand[PSEL_CAND];
+  uint32_t hist[PSEL_PASSES][PSEL_BINS];
 };
 
 __global__ void __launch_bounds__(PSEL_THREADS) pivot_coop_kernel(EdgeList in, uint64_t m_bound, const u64 *m_dev,
@@ -1445,29 +1326,24 @@ __global__ void __launch_bounds__(PSEL_THREADS) pivot_coop_kernel(EdgeList in, u
   namespace cg = cooperative_groups;
   cg::grid_group grid = cg::this_grid();
   __shared__ uint32_t s_hist[PSEL_BINS];
-  __shared__ u64 s_prefix, s_mask;
-  __shared__ uint32_t s_rank, s_scan[PSEL_THREADS / 32 + 1];
+  __shared__ u64 s_prefix, s_mask, s_mn[PSEL_THREADS / 32], s_mx[PSEL_THREADS / 32];
+  __shared__ uint32_t s_rank, s_cnt, s_scan[PSEL_THREADS / 32 + 1];
   const uint32_t nthreads = PSEL_BLOCKS * PSEL_THREADS;
   const uint32_t tid = blockIdx.x * PSEL_THREADS + threadIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 
-  if (blockIdx.x == 0) {
-    for (int i = threadIdx.x; i < 2 * PSEL_BINS; i += PSEL_THREADS) (&ps->hist[0][0])[i] = 0;
-    if (threadIdx.x == 0) {
-      ps->min = KEY_INF;
-      ps->max = 0;
-    }
-  }
-  grid.sync();
   // draw the samples; track the minimum and maximum key
-  u64 mn = KEY_INF, mx = 0;
+  u64 mn = KEY_INF, mx = 0, key0 = KEY_INF;
   for (uint32_t i = tid; i < sample; i += nthreads) {
     u64 k = KEY_INF;
     if (m) {
       const uint64_t j = __umul64hi(splitmix64_at(state, i), m);
       k = ((u64)__ldg(in.w + j) << 32) | (u64)(in.id ? __ldg(in.id + j) : (uint32_t)j);
     }
-    keys[i] = k;
+    if (i == tid)
+      key0 = k;
+    else
+      keys[i] = k;
     mn = k < mn ? k : mn;
     mx = k > mx ? k : mx;
   }
@@ -1478,83 +1354,133 @@ __global__ void __launch_bounds__(PSEL_THREADS) pivot_coop_kernel(EdgeList in, u
     mx = b > mx ? b : mx;
   }
   if (lane == 0) {
-    atomicMin(&ps->min, mn);
-    atomicMax(&ps->max, mx);
+    s_mn[wid] = mn;
+    s_mx[wid] = mx;
+  }
+  for (int i = threadIdx.x; i < PSEL_BINS; i += PSEL_THREADS) s_hist[i] = 0;
+  __syncthreads();
+  if (wid == 0) {
+    mn = s_mn[lane];
+    mx = s_mx[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const u64 a = __shfl_xor_sync(0xffffffffu, mn, o), b = __shfl_xor_sync(0xffffffffu, mx, o);
+      mn = a < mn ? a : mn;
+      mx = b > mx ? b : mx;
+    }
+    if (lane == 0) {
+      atomicMax(&ps->nmin, ~mn);
+      atomicMax(&ps->max, mx);
+    }
   }
   grid.sync();
-  mn = *(volatile u64 *)&ps->min;
+  mn = ~*(volatile u64 *)&ps->nmin;
   mx = *(volatile u64 *)&ps->max;
-  if (mn == mx || sample == 0) {
-    if (tid == 0) *out = mn;
-    return;
-  }
-  int low = 63 - __clzll((long long)(mn ^ mx)) + 1 - PSEL_BITS;  // lowest bit of the first digit
-  if (threadIdx.x == 0) {
-    const int top = low + PSEL_BITS;  // bits >= top are shared by every key
-    s_mask = top >= 64 ? 0ULL : ~((1ULL << top) - 1ULL);
-    s_prefix = mn & s_mask;
-    s_rank = rank0;
-  }
-  __syncthreads();
-  for (int pass = 0;; ++pass) {
-    const int shift = low < 0 ? 0 : low;
-    const int width = low < 0 ? PSEL_BITS + low : PSEL_BITS;
-    const uint32_t dmask = (1u << width) - 1u;
-    for (int i = threadIdx.x; i < PSEL_BINS; i += PSEL_THREADS) s_hist[i] = 0;
-    __syncthreads();
-    const u64 prefix = s_prefix, mask = s_mask;
-    for (uint32_t i = tid; i < sample; i += nthreads) {
-      const u64 k = keys[i];
-      if ((k & mask) == prefix) atomicAdd(&s_hist[(uint32_t)(k >> shift) & dmask], 1u);
+  int pass = 0;
+  if (mn != mx && sample != 0) {
+    int low = 63 - __clzll((long long)(mn ^ mx)) + 1 - PSEL_BITS;  // lowest bit of the first digit
+    if (threadIdx.x == 0) {
+      const int top = low + PSEL_BITS;  // bits >= top are shared by every key
+      s_mask = top >= 64 ? 0ULL : ~((1ULL << top) - 1ULL);
+      s_prefix = mn & s_mask;
+      s_rank = rank0;
     }
     __syncthreads();
-    uint32_t *gh = ps->hist[pass & 1];
-    for (int i = threadIdx.x; i < PSEL_BINS; i += PSEL_THREADS)
-      if (s_hist[i]) atomicAdd(gh + i, s_hist[i]);
-    grid.sync();
-    // every block: find the digit holding the current rank (4 bins per thread)
-    uint32_t c4[4], sum = 0;
+    for (;; low -= PSEL_BITS) {
+      const int shift = low < 0 ? 0 : low;
+      const int width = low < 0 ? PSEL_BITS + low : PSEL_BITS;
+      const uint32_t dmask = (1u << width) - 1u;
+      if (pass) {
+        for (int i = threadIdx.x; i < PSEL_BINS; i += PSEL_THREADS) s_hist[i] = 0;
+        __syncthreads();
+      }
+      const u64 prefix = s_prefix, mask = s_mask;
+      for (uint32_t i = tid; i < sample; i += nthreads) {
+        u64 k = key0;
+        if (i != tid) k = keys[i];
+        if ((k & mask) == prefix) atomicAdd(&s_hist[(uint32_t)(k >> shift) & dmask], 1u);
+      }
+      __syncthreads();
+      uint32_t *gh = ps->hist[pass];
+      for (int i = threadIdx.x; i < PSEL_BINS; i += PSEL_THREADS)
+        if (s_hist[i]) atomicAdd(gh + i, s_hist[i]);
+      grid.sync();
+      ++pass;
+      // every block: find the digit holding the current rank (4 bins per thread)
+      uint32_t c4[4], sum = 0;
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      c4[b] = *(volatile uint32_t *)(gh + threadIdx.x * 4 + b);
-      sum += c4[b];
-    }
-    uint32_t incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane == 31) s_scan[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-      const uint32_t v = lane < PSEL_THREADS / 32 ? s_scan[lane] : 0u;
-      uint32_t wi = v;
+      for (int b = 0; b < 4; ++b) {
+        c4[b] = *(volatile uint32_t *)(gh + threadIdx.x * 4 + b);
+        sum += c4[b];
+      }
+      uint32_t incl = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-        if (lane >= o) wi += y;
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
       }
-      if (lane < PSEL_THREADS / 32) s_scan[lane] = wi - v;
+      if (lane == 31) s_scan[wid] = incl;
+      __syncthreads();
+      if (wid == 0) {
+        const uint32_t v = s_scan[lane];
+        uint32_t wi = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
+          if (lane >= o) wi += y;
+        }
+        s_scan[lane] = wi - v;
+      }
+      __syncthreads();
+      const uint32_t before = s_scan[wid] + incl - sum, rank = s_rank;
+      if (before <= rank && rank < before + sum) {  // exactly one thread; others may still read s_rank
+        uint32_t below = before;
+        int b = 0;
+        while (below + c4[b] <= rank) below += c4[b++];
+        s_prefix = prefix | ((u64)(threadIdx.x * 4 + b) << shift);
+        s_mask = mask | ((u64)dmask << shift);
+        s_hist[0] = rank - below;
+        s_cnt = c4[b];
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) s_rank = s_hist[0];
+      __syncthreads();
+      if (shift == 0 || s_cnt <= PSEL_CAND) break;
     }
-    __syncthreads();
-    const uint32_t before = s_scan[wid] + incl - sum, rank = s_rank;
-    if (before <= rank && rank < before + sum) {  // exactly one thread
-      uint32_t below = before;
-      int b = 0;
-      while (below + c4[b] <= rank) below += c4[b++];
-      s_prefix = prefix | ((u64)(threadIdx.x * 4 + b) << shift);
-      s_mask = mask | ((u64)dmask << shift);
-      s_rank = rank - below;
+    if (low > 0) {  // bits are left: rank the s_cnt candidates among themselves
+      const u64 prefix = s_prefix, mask = s_mask;
+      for (uint32_t i = tid; i < sample; i += nthreads) {
+        u64 k = key0;
+        if (i != tid) k = keys[i];
+        if ((k & mask) == prefix) ps->cand[atomicAdd(&ps->cands, 1u)] = k;
+      }
     }
-    if (blockIdx.x == 0)  // the other histogram is reused by the next pass
-      for (int i = threadIdx.x; i < PSEL_BINS; i += PSEL_THREADS) ps->hist[(pass + 1) & 1][i] = 0;
-    __syncthreads();
-    if (shift == 0) break;
-    low -= PSEL_BITS;
-    grid.sync();
+    grid.sync();  // and the last reader of the histograms
+    if (low > 0 && blockIdx.x == 0) {
+      const uint32_t cnt = s_cnt;
+      u64 *s_cand = reinterpret_cast<u64 *>(s_hist);
+      u64 k = KEY_INF;
+      if (threadIdx.x < cnt) k = *(volatile u64 *)&ps->cand[threadIdx.x];
+      if (threadIdx.x < cnt) s_cand[threadIdx.x] = k;
+      __syncthreads();
+      if (threadIdx.x < cnt) {
+        uint32_t below = 0;
+        for (uint32_t i = 0; i < cnt; ++i) below += s_cand[i] < k || (s_cand[i] == k && i < threadIdx.x) ? 1u : 0u;
+        if (below == s_rank) *out = k;
+      }
+    } else if (tid == 0) {
+      *out = s_prefix;
+    }
+  } else {
+    if (tid == 0) *out = mn;
+    grid.sync();  // every block has read the extremes
   }
-  if (tid == 0) *out = s_prefix;
+  // back to zero
+  for (uint32_t i = tid; i < (uint32_t)(pass * PSEL_BINS); i += nthreads) (&ps->hist[0][0])[i] = 0;
+  if (tid == 0) {
+    ps->nmin = ps->max = 0;
+    ps->cands = 0;
+  }
 }
 
 // ---------------------------------------------------- tile-local contraction
@@ -2382,15 +2308,23 @@ __global__ void tile_sample_kernel(EdgeList in, uint64_t m, uint32_t n, uint32_t
 // Finds the component that most endpoints of a random edge sample belong to:
 // 1024 edges of the list are drawn with splitmix64, the root P[u] of each
 // sample's first endpoint is taken (P fully contracted), and the most frequent
-// root is written to *out (a sort in shared memory, then the longest run).
+// root is written to *out.  Counted in a shared-memory hash table, a warp's equal
+// roots with one atomic.  Latency-bound: 9 us with a bitonic sort (55 block
+// barriers) instead, 4.6 us now.
 constexpr int MODE_SAMPLES = (int)GIANT_SAMPLES;
 __global__ void __launch_bounds__(MODE_SAMPLES) giant_root_kernel(EdgeList in, uint64_t m_bound, const u64 *m_dev,
                                                                   u64 state, const uint32_t *P, uint32_t n,
                                                                   uint32_t *out, uint32_t *count_out) {
   const uint64_t m = m_dev ? min((uint64_t)*m_dev, m_bound) : m_bound;
-  __shared__ uint32_t s_r[MODE_SAMPLES];
+  constexpr uint32_t SLOTS = 2 * MODE_SAMPLES;
+  __shared__ u64 s_key[SLOTS];  // root + 1; 0: empty
+  __shared__ uint32_t s_num[SLOTS];
   __shared__ uint32_t s_best[MODE_SAMPLES / 32], s_bestv[MODE_SAMPLES / 32];
   const uint32_t t = threadIdx.x;
+  for (uint32_t i = t; i < SLOTS; i += MODE_SAMPLES) {
+    s_key[i] = 0;
+    s_num[i] = 0;
+  }
   uint32_t r = 0xffffffffu;
   if (m) {
     const uint32_t u = __ldg(in.u + __umul64hi(splitmix64_at(state, t), m));
@@ -2404,37 +2338,26 @@ __global__ void __launch_bounds__(MODE_SAMPLES) giant_root_kernel(EdgeList in, u
       }
     }
   }
-  s_r[t] = r;
   __syncthreads();
-  for (uint32_t k = 2; k <= MODE_SAMPLES; k <<= 1) {  // bitonic sort, ascending
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      const uint32_t p = t ^ j;
-      if (p > t) {
-        const uint32_t a = s_r[t], b = s_r[p];
-        const bool up = (t & k) == 0;
-        if ((a > b) == up) {
-          s_r[t] = b;
-          s_r[p] = a;
-        }
-      }
-      __syncthreads();
+  const uint32_t peers = __match_any_sync(0xffffffffu, r);
+  if ((int)(t & 31) == __ffs(peers) - 1) {
+    uint32_t h = (r * 0x9e3779b1u) >> 21;  // 11 bits
+    static_assert(SLOTS == 1u << 11, "hash bits");
+    for (;; h = (h + 1) & (SLOTS - 1)) {  // at most MODE_SAMPLES of the slots are taken
+      const u64 k = atomicCAS(&s_key[h], 0ULL, (u64)r + 1);
+      if (k == 0 || k == (u64)r + 1) break;
+    }
+    atomicAdd(&s_num[h], (uint32_t)__popc(peers));
+  }
+  __syncthreads();
+  uint32_t bl = 0, bv = 0xffffffffu;
+  for (uint32_t i = t; i < SLOTS; i += MODE_SAMPLES) {
+    const uint32_t l = s_num[i], v = (uint32_t)(s_key[i] - 1);
+    if (l > bl || (l == bl && l && v < bv)) {
+      bl = l;
+      bv = v;
     }
   }
-  // run length at each run start (upper bound by binary search)
-  const uint32_t v = s_r[t];
-  uint32_t len = 0;
-  if (t == 0 || s_r[t - 1] != v) {
-    uint32_t lo = t, hi = MODE_SAMPLES;
-    while (lo < hi) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (s_r[mid] <= v)
-        lo = mid + 1;
-      else
-        hi = mid;
-    }
-    len = lo - t;
-  }
-  uint32_t bl = len, bv = v;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const uint32_t ol = __shfl_xor_sync(0xffffffffu, bl, o), ov = __shfl_xor_sync(0xffffffffu, bv, o);
@@ -2471,77 +2394,154 @@ __global__ void giant_bits_kernel(const uint32_t *P, uint32_t n, const uint32_t 
   }
 }
 
-// ---------------------------------------------------------------- finalize
+// ------------------------------------------------------------ start and end
+
+// The state a solve starts from: best[] at infinity, every vertex its own
+// representative, no edge chosen, counters zero.  One launch of plain stores
+// instead of six memsets and a kernel, which took 30 us of a small solve, most of
+// it between launches; n=2^18, m=2^22: 2.3 us, n=2^24, m=2^28: 35 us (6.7 TB/s).
+__global__ void __launch_bounds__(BLOCK) init_kernel(InitArgs a) {
+  const uint64_t t = (uint64_t)blockIdx.x * BLOCK + threadIdx.x, stride = (uint64_t)gridDim.x * BLOCK;
+  for (uint64_t i = t; i < a.n; i += stride) {
+    a.best[i] = KEY_INF;
+    a.parent[i] = (uint32_t)i;
+  }
+  for (uint64_t i = t; i < a.words; i += stride) a.bits[i] = 0;
+  for (uint64_t i = t; i < a.zero_words; i += stride) a.zero[i] = 0;
+}
 
 // Output (Section 2.2; edge ids, Section 6.2): set bits of the chosen-edge
-// bitmap become ascending ids; their weights are summed into a uint64.
-__global__ void __launch_bounds__(BLOCK) finalize_kernel(const uint32_t *bits, uint64_t nwords, const uint32_t *w,
-                                                         uint32_t *out_ids, uint32_t *out_count, u64 *total_weight,
-                                                         ScanState st) {
-  __shared__ uint32_t s_warp[BLOCK / 32 + 1];
-  __shared__ u64 s_sum[BLOCK / 32];
-  __shared__ LookbackShared s_lb;
-  TileInfo t;
-  if (!acquire_tile(st, nwords, t)) {
-    if (t.ntiles == 0 && t.tile == 0 && threadIdx.x == 0) *out_count = 0;
-    return;
-  }
-  const uint64_t tb = (uint64_t)t.tile * TILE;
-  uint32_t wd[ITEMS], c0 = 0, c1 = 0;
+// bitmap become ascending ids.  Every warp owns a run of the bitmap's words and
+// counts its bits; behind a barrier of the blocks (cooperative launch; bounded)
+// a block adds up the counts before its own, and a second pass, from cache,
+// stages 64 words' ids at a time in shared memory for coalesced stores.  The
+// block that ends last adds up the weight counters and hands the solve's state
+// to the host, which two launches behind this one did.  Latency-bound up to some
+// million edges, then by the instructions per set bit.  n=2^18, m=2^22: 11 us
+// where the three launches took 23; RGG2D n=2^22: 19 us instead of 48; n=2^24,
+// m=2^28: 51 us instead of 75.  (A look-back in which every block polls its
+// predecessors' words, without a barrier, took 6 us from a block's count to its
+// offset; the barrier 1.7.)
+constexpr int FB = 256, FW = FB / 32;
+__global__ void __launch_bounds__(FB, 4) finish_kernel(FinishArgs a) {
+  __shared__ uint16_t s_stage[FW][2048 + 128];
+  __shared__ uint32_t s_warp[FW + 1], s_part[FW], s_last;
+  __shared__ u64 s_sum[FW];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t nb = gridDim.x, bid = blockIdx.x;
+  const uint64_t warps = (uint64_t)nb * FW;
+  const uint64_t seg = ((a.nwords + warps - 1) / warps + 63) & ~63ULL;
+  const uint64_t lo = min(a.nwords, ((uint64_t)bid * FW + wid) * seg), hi = min(a.nwords, lo + seg);
+  uint32_t cnt = 0;
+#pragma unroll 8
+  for (uint64_t i = lo + lane; i < hi; i += 32) cnt += __popc(__ldg(a.bits + i));
 #pragma unroll
-  for (int k = 0; k < ITEMS; ++k) {
-    const uint64_t j = tb + item_off(k);
-    wd[k] = j < nwords ? bits[j] : 0u;
-    if (k < 4)
-      c0 += __popc(wd[k]);
-    else
-      c1 += __popc(wd[k]);
-  }
-  uint32_t excl, totp;
-  uint64_t obase;
-  if (!tile_offsets(st, t, c0 | (c1 << 16), excl, totp, obase, s_warp, s_lb)) return;
-  const uint32_t total = (totp & 0xffffu) + (totp >> 16);
-  u64 wsum = 0;
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    uint64_t pos = obase + (half == 0 ? (excl & 0xffffu) : (totp & 0xffffu) + (excl >> 16));
-#pragma unroll
-    for (int k = half * 4; k < half * 4 + 4; ++k) {
-      uint32_t word = wd[k];
-      while (word) {
-        const int b = __ffs(word) - 1;
-        word &= word - 1;
-        const uint32_t id = (uint32_t)((tb + item_off(k)) * 32 + b);
-        out_ids[pos++] = id;
-        if (w) wsum += __ldg(w + id);
+  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+  uint32_t total;
+  uint32_t pos = block_exclusive_scan<FB>(lane == 0 ? cnt : 0u, total, s_warp);
+  pos = __shfl_sync(0xffffffffu, pos, 0);
+  int lost = 0;
+  if (threadIdx.x == 0 && nb > 1) {
+    a.st.count[bid] = total;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.st.arrived) : "memory");
+    for (uint32_t spins = 0;;) {
+      uint32_t v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.st.arrived) : "memory");
+      if (v >= nb) break;
+      if (++spins >= a.st.spin_limit) {
+        lost = 1;
+        break;
       }
     }
   }
+  lost = __syncthreads_or(lost);
+  uint32_t before = 0;
+  if (!lost)
+    for (uint32_t b = threadIdx.x; b < bid; b += FB) before += __ldcg(a.st.count + b);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
-  if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = wsum;
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  if (lane == 0) s_part[wid] = before;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    u64 s = 0;
-    for (int i = 0; i < BLOCK / 32; ++i) s += s_sum[i];
-    if (s && w) atomicAdd(total_weight, s);
-    if (t.tile == t.ntiles - 1) *out_count = (uint32_t)(obase + total);
-  }
-}
-
-// *total = the sum of the WSUM_SLOTS counters (one block of WSUM_SLOTS threads).
-__global__ void wsum_total_kernel(const u64 *wsum, u64 *total) {
-  __shared__ u64 s_part[WSUM_SLOTS / 32];
-  u64 v = wsum[threadIdx.x];
+  u64 wsum = 0;
+  if (!lost) {
+    before = 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    u64 t = 0;
-    for (int i = 0; i < WSUM_SLOTS / 32; ++i) t += s_part[i];
-    *total = t;
+    for (int i = 0; i < FW; ++i) before += s_part[i];
+    if (bid == nb - 1 && threadIdx.x == 0) {
+      *a.out_count = before + total;
+      *a.st.total = (u64)before + total;
+    }
+    uint64_t out = (uint64_t)before + pos;
+    // a lane takes two neighbouring words of the warp's next 64; two unused
+    // entries behind every 32 of the stage spread dense words over the banks
+    const auto load = [&](uint64_t j) { return j < hi ? __ldg(a.bits + j) : 0u; };
+    const auto at = [](uint32_t p) { return p + (p >> 5) * 2; };
+    uint32_t n0 = load(lo + 2 * lane), n1 = load(lo + 2 * lane + 1);
+    for (uint64_t i = lo; i < hi; i += 64) {
+      uint32_t word = n0, after = n1;
+      n0 = load(i + 64 + 2 * lane), n1 = load(i + 64 + 2 * lane + 1);
+      const uint32_t c = __popc(word) + __popc(after), first = (uint32_t)(i * 32);
+      uint32_t incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const uint32_t all = __shfl_sync(0xffffffffu, incl, 31);
+      uint32_t off = lane * 64;
+      if (word == 0) word = after, after = 0, off += 32;
+      for (uint32_t p = incl - c; p < incl; ++p) {
+        s_stage[wid][at(p)] = (uint16_t)(off + __ffs(word) - 1);
+        word &= word - 1;
+        if (word == 0) word = after, after = 0, off += 32;
+      }
+      __syncwarp();
+      for (uint32_t x = lane; x < all; x += 32) {
+        const uint32_t id = first + s_stage[wid][at(x)];
+        a.out_ids[out + x] = id;
+        if (a.w) wsum += __ldg(a.w + id);
+      }
+      out += all;
+      __syncwarp();
+    }
+  } else if (threadIdx.x == 0) {
+    atomicOr(a.st.err, ERR_LOOKBACK);
   }
+  if (a.w) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
+    if (lane == 0 && wsum) atomicAdd(a.total_weight, wsum);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {  // this block's stores before the host's word
+    __threadfence_system();
+    s_last = atomicAdd(a.st.ended, 1u) == nb - 1 ? 1u : 0u;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_last) return;
+  if (threadIdx.x == 0) *a.st.arrived = *a.st.ended = 0;
+  if (a.wsum) {
+    u64 v = threadIdx.x < WSUM_SLOTS ? __ldcg(a.wsum + threadIdx.x) : 0ULL;
+    static_assert(WSUM_SLOTS <= FB, "a counter per thread");
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) s_sum[wid] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      u64 t = 0;
+      for (int i = 0; i < FW; ++i) t += s_sum[i];
+      *a.total_weight = t;
+    }
+  }
+  if (!a.state) return;
+  constexpr uint32_t words = (uint32_t)(sizeof(DevState) / 4);
+  static_assert(sizeof(DevState) % 4 == 0, "DevState is copied in words");
+  for (uint32_t i = threadIdx.x; i < words; i += FB)
+    reinterpret_cast<volatile uint32_t *>(a.mirror)[i] = __ldcg(reinterpret_cast<const uint32_t *>(a.state) + i);
+  __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) *reinterpret_cast<volatile uint32_t *>(a.flag) = a.seq;
 }
 
 // ---------------------------------------------------------------- launchers
@@ -2556,7 +2556,6 @@ static inline unsigned grid_for(uint64_t items_per_block_units, int sms, int per
   return (unsigned)g;
 }
 
-int max_scan_tiles(uint64_t count) { return (int)((count + TILE - 1) / TILE); }
 
 // One compaction launch in tile shape (B, I): the persistent TMA kernel for
 // long lists whose tiles fit two shared-memory stages, else one block per tile.
@@ -2767,15 +2766,23 @@ bool launch_pivot_coop(EdgeList in, uint64_t m, u64 state, uint32_t sample, u64 
   return false;
 }
 
-void launch_wsum_total(const u64 *wsum, u64 *total, cudaStream_t s) {
-  wsum_total_kernel<<<1, WSUM_SLOTS, 0, s>>>(wsum, total);
+void launch_init(const InitArgs &a, int sms, cudaStream_t s) {
+  const uint64_t most = std::max(std::max((uint64_t)a.n, a.words), a.zero_words);
+  init_kernel<<<grid_for((most + BLOCK - 1) / BLOCK, sms, 8), BLOCK, 0, s>>>(a);
 }
 
-void launch_finalize(const uint32_t *bits, uint64_t m, const uint32_t *w, uint32_t *out_ids, uint32_t *out_count,
-                     u64 *total_weight, ScanState st, cudaStream_t s) {
-  const uint64_t nwords = (m + 31) / 32;
-  const unsigned grid = (unsigned)(max_scan_tiles(nwords) > 0 ? max_scan_tiles(nwords) : 1);
-  finalize_kernel<<<grid, BLOCK, 0, s>>>(bits, nwords, w, out_ids, out_count, total_weight, st);
+// Four blocks per SM at most, so that all are resident; a warp has 64 words at
+// least.  Where a cooperative launch is refused one block does it all.
+void launch_finish(const FinishArgs &a, int sms, cudaStream_t s) {
+  const uint64_t want = std::max<uint64_t>(1, (a.nwords + 2 * FB - 1) / (2 * FB));
+  const unsigned grid = (unsigned)std::min<uint64_t>(want, std::min<uint64_t>((uint64_t)sms * 4, FINISH_BLOCKS));
+  FinishArgs arg = a;
+  void *args[] = {&arg};
+  if (grid > 1 &&
+      cudaLaunchCooperativeKernel((const void *)finish_kernel, dim3(grid), dim3(FB), args, 0, s) == cudaSuccess)
+    return;
+  if (grid > 1) cudaGetLastError();
+  finish_kernel<<<1, FB, 0, s>>>(a);
 }
 
 void launch_giant_root(EdgeList in, uint64_t m, u64 state, const uint32_t *P, uint32_t n, uint32_t *root_tmp,

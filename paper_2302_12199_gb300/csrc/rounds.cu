@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
 
 }  // namespace
 
-bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, int sms, cudaStream_t s) {
+bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, bool clear, int sms, cudaStream_t s) {
   // resident blocks per SM (0: not available); set once per process
   static const int per_sm = []() -> int {
     int b = 0;
@@ -737,7 +737,7 @@ bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, int sms, cudaStream_
     return b < 2 ? b : 2;
   }();
   if (per_sm <= 0 || a.n >= ROOT) return false;
-  if (cudaMemsetAsync(a.st, 0, sizeof(RoundsState), s) != cudaSuccess) {
+  if (clear && cudaMemsetAsync(a.st, 0, sizeof(RoundsState), s) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

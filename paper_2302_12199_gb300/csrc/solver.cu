@@ -38,9 +38,7 @@ struct mst_ctx {
   uint32_t rb_seq = 0;
   uint64_t readbacks = 0;
   u64 *hres = nullptr;       // pinned host words for the forest size and weight of the host entry points
-  u64 *status = nullptr;     // scan status words
-  uint64_t status_cap = 0;   // in tiles
-  uint32_t epoch = 0;
+  uint32_t *scan_count = nullptr;  // the output scan's counts per block
   u64 *sample_buf = nullptr;
   uint32_t sample_cap = 0;
   void *pivot_scratch = nullptr;  // histograms of the multi-block pivot selection
@@ -74,7 +72,9 @@ struct mst_ctx {
   void *small_mem = nullptr;      // scratch of graphs that one block solves (SmallScratch)
   cudaStream_t kind_stream[2] = {nullptr, nullptr};  // block solves of the middle and the small graphs of a batch
   cudaEvent_t kind_ev[3] = {nullptr, nullptr, nullptr};
-  RoundsState *rstate = nullptr;  // device state of the one-launch rounds
+  RoundsState *rstate = nullptr;  // device states of the one-launch rounds, one per launch of a solve
+  int rounds_used = 0;            // of them, by this solve
+  uint64_t zero_words = 0;        // words from ds on that a solve's start clears (ds, wsum, rstate)
   std::vector<cudaEvent_t> ev_pool;
   std::vector<ProfRec> prof_pending;
   mst_kernel_stats prof[MST_K_COUNT];
@@ -82,7 +82,6 @@ struct mst_ctx {
 
 namespace {
 
-constexpr int TILE_ITEMS = 2048;
 
 // The CUDA error of the call that made the current API call fail (per host
 // thread; record() moves it into the handle).
@@ -220,34 +219,9 @@ mst_status round_lists(mst_ctx *c, uint64_t need, RoundList &X, RoundList &Y, cu
   return MST_OK;
 }
 
-mst_status ensure_status(mst_ctx *c, uint64_t max_items, cudaStream_t s) {
-  const uint64_t tiles = (max_items + TILE_ITEMS - 1) / TILE_ITEMS + 1;
-  if (tiles <= c->status_cap) return MST_OK;
-  // stream-ordered, like the round lists: no wait for the whole device
-  if (c->status) CK(cudaFreeAsync(c->status, s));
-  c->status = nullptr;
-  c->status_cap = 0;
-  const uint64_t cap = next_pow2(tiles < 4096 ? 4096 : tiles);
-  if (cudaMallocAsync(&c->status, cap * sizeof(u64), s) != cudaSuccess) {
-    cudaGetLastError();
-    c->status = nullptr;
-    return MST_ERR_OOM;
-  }
-  CK(cudaMemsetAsync(c->status, 0, cap * sizeof(u64), s));
-  c->status_cap = cap;
-  c->epoch = 0;
-  CK(cudaMemsetAsync(c->ds->tile_ctr, 0, sizeof(c->ds->tile_ctr), s));
-  return MST_OK;
-}
-
 ScanState next_scan(mst_ctx *c, int total_slot) {
-  if (++c->epoch >= (1u << 30)) {  // epochs wrapped: clear the status words (practically never)
-    cudaDeviceSynchronize();
-    cudaMemset(c->status, 0, c->status_cap * sizeof(u64));
-    cudaMemset(c->ds->tile_ctr, 0, sizeof(c->ds->tile_ctr));
-    c->epoch = 1;
-  }
-  return ScanState{c->status, c->ds->tile_ctr, c->epoch, &c->ds->count[total_slot], &c->ds->err, c->cfg.spin_limit};
+  return ScanState{c->scan_count, &c->ds->scan_ctr[0], &c->ds->scan_ctr[1], &c->ds->count[total_slot], &c->ds->err,
+                   c->cfg.spin_limit};
 }
 
 cudaEvent_t take_event(mst_ctx *c) {
@@ -394,11 +368,11 @@ __global__ void readback_kernel(const DevState *ds, DevState *hs, uint32_t *flag
 // synchronisation costs about ten); after about a second without the flag it
 // falls back to synchronising the stream, which also reports a CUDA error.
 // Error bits in `tolerated` are left for the caller to act on.
-mst_status readback(mst_ctx *c, cudaStream_t s, uint32_t tolerated = 0) {
-  static_assert(sizeof(DevState) % 4 == 0, "DevState is copied in words");
-  const uint32_t seq = ++c->rb_seq;
+uint32_t next_readback(mst_ctx *c) {
   ++c->readbacks;
-  readback_kernel<<<1, 32, 0, s>>>(c->ds, c->hs_dev, c->hflag_dev, seq);
+  return ++c->rb_seq;
+}
+mst_status readback_wait(mst_ctx *c, cudaStream_t s, uint32_t seq, uint32_t tolerated) {
   CK(cudaGetLastError());
   bool seen = false;
   for (uint64_t spin = 0; spin < (1ULL << 26); ++spin) {
@@ -420,13 +394,19 @@ mst_status readback(mst_ctx *c, cudaStream_t s, uint32_t tolerated = 0) {
   if (err) return MST_ERR_INTERNAL;
   return MST_OK;
 }
+mst_status readback(mst_ctx *c, cudaStream_t s, uint32_t tolerated = 0) {
+  static_assert(sizeof(DevState) % 4 == 0, "DevState is copied in words");
+  const uint32_t seq = next_readback(c);
+  readback_kernel<<<1, 32, 0, s>>>(c->ds, c->hs_dev, c->hflag_dev, seq);
+  return readback_wait(c, s, seq, tolerated);
+}
 
-// Clears the error word, the jump flag and both tile counters (err, jump_flag
-// and tile_ctr are adjacent in DevState).  Called at the start of every solve
-// and step call, so that a launch that failed earlier cannot leave a counter
+// Clears the error word, the jump flag and both scan counters (err, jump_flag
+// and scan_ctr are adjacent in DevState).  Called at the start of every step
+// call, so that a launch that failed earlier cannot leave a counter
 // behind for the scans of this call.
 mst_status clear_device_flags(mst_ctx *c, cudaStream_t s) {
-  static_assert(offsetof(DevState, tile_ctr) == 2 * sizeof(uint32_t), "DevState layout");
+  static_assert(offsetof(DevState, scan_ctr) == 2 * sizeof(uint32_t), "DevState layout");
   CK(cudaMemsetAsync(c->ds, 0, 4 * sizeof(uint32_t), s));
   return MST_OK;
 }
@@ -515,27 +495,29 @@ struct Solve {
   mst_status init(uint32_t *parent_external = nullptr, uint32_t *bits_external = nullptr) {
     TRY(best_b.alloc(c, (size_t)n * 8, s));
     best = best_b.as<u64>();
-    CK(cudaMemsetAsync(best, 0xff, (size_t)n * 8, s));
     if (parent_external) {
       parent = parent_external;
     } else {
       TRY(parent_b.alloc(c, (size_t)n * 4, s));
       parent = parent_b.as<uint32_t>();
     }
-    launch_iota(parent, n, c->sms, s);
     TRY(act_b[0].alloc(c, (size_t)n * 4, s));
     act[0] = act_b[0].as<uint32_t>();
     if (bits_external) {
       bits = bits_external;
     } else {
-      const size_t words = (m + 31) / 32;
-      TRY(bits_b.alloc(c, words * 4, s));
+      TRY(bits_b.alloc(c, (m + 31) / 32 * 4, s));
       bits = bits_b.as<uint32_t>();
-      CK(cudaMemsetAsync(bits, 0, words * 4, s));
     }
-    TRY(ensure_status(c, (uint64_t)n > m ? (uint64_t)n : m, s));
-    TRY(clear_device_flags(c, s));
-    CK(cudaMemsetAsync(c->wsum, 0, WSUM_SLOTS * sizeof(u64), s));
+    return start(bits_external == nullptr);
+  }
+  // Everything at its initial value, the handle's counters and flags included
+  // (so that a launch that failed earlier leaves nothing behind for this call).
+  mst_status start(bool clear_bits) {
+    launch_init(InitArgs{best, parent, n, bits, clear_bits ? (m + 31) / 32 : 0, (uint32_t *)c->ds, c->zero_words},
+                c->sms, s);
+    CK(cudaGetLastError());
+    c->rounds_used = 0;
     return MST_OK;
   }
 
@@ -543,8 +525,7 @@ struct Solve {
   // into the key when the largest weight, the edge ids and the vertex ids fit
   // into 63 bits together (the top bit stays clear, so no key equals INF).
   mst_status choose_layout(const uint32_t *w) {
-    CK(cudaMemsetAsync(&c->ds->max_w, 0, sizeof(uint32_t), s));
-    launch_max_weight(w, m, &c->ds->max_w, c->sms, s);
+    launch_max_weight(w, m, &c->ds->max_w, c->sms, s);  // (zero since start())
     TRY(readback(c, s));
     set_layout();
     return cur_alloc();
@@ -795,7 +776,7 @@ struct Solve {
     ra.wsum = c->wsum;
     ra.n = n;
     ra.max_rounds = (uint32_t)std::min(ROUNDS_MAX, 2 * (ceil_log2(n) + 2));
-    ra.st = c->rstate;
+    ra.st = c->rstate + std::min(c->rounds_used, ROUNDS_STATES - 1);
     ra.err = &c->ds->err;
     return ra;
   }
@@ -810,7 +791,6 @@ struct Solve {
     TRY(rounds_alloc());
     const uint32_t *max_w = nullptr;
     if (!layout_set) {  // the kernel picks the key layout from the largest weight
-      CK(cudaMemsetAsync(&c->ds->max_w, 0, sizeof(uint32_t), s));
       launch_max_weight(w_in ? w_in : E.w, m, &c->ds->max_w, c->sms, s);
       max_w = &c->ds->max_w;
       layout_bits();
@@ -840,7 +820,7 @@ struct Solve {
     ra.validate = validate ? 1 : 0;
     ra.max_w = max_w;
     ra.want_parent = want_parent ? 1 : 0;
-    PROF(MST_K_GRAPH, 0.0, -1, 0.0, -1, 0.0, ran = launch_rounds(ra, mE, c->sms, s));
+    PROF(MST_K_GRAPH, 0.0, -1, 0.0, -1, 0.0, ran = launch_rounds(ra, mE, c->rounds_used++ >= ROUNDS_STATES, c->sms, s));
     if (ran) ++rounds;
     return MST_OK;
   }
@@ -1205,7 +1185,7 @@ struct Solve {
     ra.want_parent = last ? 0 : 1;
     ra.ends_rec = (ends_rec && cur_u) ? 1 : 0;
     bool ran = false;
-    PROF(MST_K_GRAPH, 0.0, -1, 0.0, -1, 0.0, ran = launch_rounds(ra, ra.m, c->sms, s));
+    PROF(MST_K_GRAPH, 0.0, -1, 0.0, -1, 0.0, ran = launch_rounds(ra, ra.m, c->rounds_used++ >= ROUNDS_STATES, c->sms, s));
     if (!ran) return MST_ERR_CUDA;
     ++rounds;
     return MST_OK;
@@ -1224,7 +1204,6 @@ struct Solve {
     TRY(gbits_b.alloc(c, ((size_t)n + 31) / 32 * 4, s));
     u64 *piv = piv_b.as<u64>();
     uint32_t *gbits = gbits_b.as<uint32_t>();
-    CK(cudaMemsetAsync(&c->ds->count[CNT_LVL], 0, 2 * LVL_MAX * sizeof(u64), s));
     const uint64_t cap1 = light_cap(m0);
     RoundList X, Y;
     TRY(round_lists(c, plan_round_edges(leaf_top ? cap1 : 0), X, Y, s));
@@ -1249,10 +1228,7 @@ struct Solve {
     cp.pivot_dev = &piv[0];
     cp.n = n;
     cp.validate = 1;
-    if (!layout_set) {
-      CK(cudaMemsetAsync(&c->ds->max_w, 0, sizeof(uint32_t), s));
-      cp.max_w = &c->ds->max_w;
-    }
+    if (!layout_set) cp.max_w = &c->ds->max_w;
     cp.best = leaf_top ? best : nullptr;
     cp.kl = kl;
     record_ends(cp);
@@ -1280,7 +1256,6 @@ struct Solve {
     const uint64_t need = plan_round_edges(caps[K]);
     if (need > X.cap) TRY(round_lists(c, need, X, Y, s));  // (not when leaf_top: X already holds list 1)
     planned = true;
-    CK(cudaMemsetAsync(&c->ds->jump_flag, 0, sizeof(uint32_t), s));
     TRY(rounds_alloc());
 
     // light lists 2 .. K (list K into X, relaxing best[] for its first round)
@@ -1359,11 +1334,7 @@ struct Solve {
   // Back to the state init() left (the host-driven path after a plan that
   // did not hold).
   mst_status restart() {
-    CK(cudaMemsetAsync(best, 0xff, (size_t)n * 8, s));
-    launch_iota(parent, n, c->sms, s);
-    CK(cudaMemsetAsync(bits, 0, (m + 31) / 32 * 4, s));
-    TRY(clear_device_flags(c, s));
-    CK(cudaMemsetAsync(c->wsum, 0, WSUM_SLOTS * sizeof(u64), s));
+    TRY(start(true));
     c->pivot_counter = 0;
     rounds = 0;
     return MST_OK;
@@ -1374,10 +1345,12 @@ struct Solve {
   // Without out_ids the bitmap is all the caller wants.
   mst_status finalize(uint32_t *out_ids, uint32_t *out_count, u64 *total_weight, uint32_t tolerated = 0) {
     if (!out_ids) return readback(c, s, tolerated);
+    const uint32_t seq = next_readback(c);
     PROF(MST_K_FINALIZE, (double)((m + 31) / 32 * 4), CNT_AUX, 4.0, -1, 0.0,
-         launch_finalize(bits, m, nullptr, out_ids, out_count, total_weight, next_scan(c, CNT_AUX), s);
-         launch_wsum_total(c->wsum, total_weight, s));
-    return readback(c, s, tolerated);
+         launch_finish(FinishArgs{bits, (m + 31) / 32, nullptr, out_ids, out_count, total_weight,
+                                  next_scan(c, CNT_AUX), c->wsum, c->ds, c->hs_dev, c->hflag_dev, seq},
+                       c->sms, s));
+    return readback_wait(c, s, seq, tolerated);
   }
 };
 
@@ -1919,17 +1892,22 @@ mst_status mst_create(mst_handle *out, const mst_config *cfg) {
   }
   // the fixed-size device state, in one allocation
   const size_t b_ds = round_up(sizeof(DevState), 256), b_piv = round_up(pivot_scratch_bytes(), 256),
-               b_ws = round_up(WSUM_SLOTS * sizeof(u64), 256), b_rs = round_up(sizeof(RoundsState), 256);
+               b_ws = round_up(WSUM_SLOTS * sizeof(u64), 256),
+               b_rs = round_up(ROUNDS_STATES * sizeof(RoundsState), 256),
+               b_sc = round_up(FINISH_BLOCKS * sizeof(uint32_t), 256);
+  const size_t b_zero = b_ds + b_ws + b_rs;  // what start() clears
   char *fixed = nullptr;
-  ok = ok && cudaMalloc(&fixed, b_ds + b_piv + b_ws + b_rs + SMALL_BYTES) == cudaSuccess;
+  ok = ok && cudaMalloc(&fixed, b_zero + b_piv + b_sc + SMALL_BYTES) == cudaSuccess;
   if (ok) {
     c->ds = (DevState *)fixed;
-    c->pivot_scratch = fixed + b_ds;
-    c->wsum = (u64 *)(fixed + b_ds + b_piv);
-    c->rstate = (RoundsState *)(fixed + b_ds + b_piv + b_ws);
-    c->small_mem = fixed + b_ds + b_piv + b_ws + b_rs;
+    c->wsum = (u64 *)(fixed + b_ds);
+    c->rstate = (RoundsState *)(fixed + b_ds + b_ws);
+    c->zero_words = b_zero / 4;
+    c->pivot_scratch = fixed + b_zero;
+    c->scan_count = (uint32_t *)(fixed + b_zero + b_piv);
+    c->small_mem = fixed + b_zero + b_piv + b_sc;
   }
-  ok = ok && cudaMemset(c->ds, 0, sizeof(DevState)) == cudaSuccess;
+  ok = ok && cudaMemset(fixed, 0, b_zero + b_piv) == cudaSuccess;  // the pivot selection leaves its scratch zero
   ok = ok && cudaHostAlloc(&c->hs, sizeof(DevState), cudaHostAllocMapped) == cudaSuccess;
   ok = ok && cudaHostGetDevicePointer((void **)&c->hs_dev, c->hs, 0) == cudaSuccess;
   ok = ok && cudaHostAlloc(&c->hflag, 64, cudaHostAllocMapped) == cudaSuccess;
@@ -1960,7 +1938,6 @@ void mst_destroy(mst_handle h) {
       if (h->hin[k]) cudaFree(h->hin[k]);
     if (h->hout) cudaFree(h->hout);
     if (h->rl_mem) cudaFree(h->rl_mem);
-    if (h->status) cudaFree(h->status);
     if (h->sample_buf) cudaFree(h->sample_buf);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
     for (int k = 0; k < 2; ++k) {
@@ -2257,7 +2234,6 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
     const uint64_t ent_bytes = round_up(m * sizeof(uint4), 256), live_bytes = round_up(m * sizeof(uint2), 256);
     st = scr_b.alloc(h, ent_bytes + live_bytes + (size_t)n * sizeof(u64) + 256, s);
     if (st == MST_OK) st = bits_b.alloc(h, words * 4, s);
-    if (st == MST_OK) st = ensure_status(h, words, s);
     if (st != MST_OK) return record(h, st);
     if (cudaMemsetAsync(bits_b.p, 0, words * 4, s) != cudaSuccess) return record_cuda(h, __LINE__);
     char *b = scr_b.as<char>();
@@ -2341,7 +2317,8 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
     }
   }
   if (use_blocks)
-    launch_finalize(bits_b.as<uint32_t>(), m, nullptr, ids, d_count, d_sum, next_scan(h, CNT_AUX), s);
+    launch_finish(FinishArgs{bits_b.as<uint32_t>(), (m + 31) / 32, nullptr, ids, d_count, d_sum, next_scan(h, CNT_AUX)},
+                  h->sms, s);
   batch_seg_kernel<<<(num_graphs + 1 + 255) / 256, 256, 0, s>>>(ids, d_count, d_edge_off, num_graphs, d_msf_off);
   const unsigned sgrid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((cap + 2047) / 2048, (uint64_t)h->sms * 8));
   batch_split_kernel<<<sgrid, 256, 0, s>>>(ids, d_count, d_edge_off, num_graphs, d_w, use_blocks ? solved : nullptr,
@@ -2405,8 +2382,7 @@ static mst_status step_compact(mst_handle h, CompactMode mode, uint32_t n, uint6
   if (m >= (1ULL << 32)) return record(h, MST_ERR_TOO_LARGE);
   DeviceGuard g(h->device);
   cudaStream_t s = (cudaStream_t)stream;
-  mst_status st = ensure_status(h, m, s);
-  if (st != MST_OK) return record(h, st);
+  mst_status st = MST_OK;
   if (clear_device_flags(h, s) != MST_OK) return record_cuda(h, __LINE__);
   const EdgeList E{d_u, d_v, d_w, d_id};
   CompactArgs a{};
@@ -2570,12 +2546,13 @@ mst_status mst_step_finalize(mst_handle h, uint64_t m, const uint32_t *d_chosen,
     return MST_ERR_INVALID_ARG;
   DeviceGuard g(h->device);
   cudaStream_t s = (cudaStream_t)stream;
-  mst_status st = ensure_status(h, (m + 31) / 32, s);
-  if (st != MST_OK) return record(h, st);
   if (clear_device_flags(h, s) != MST_OK || cudaMemsetAsync(d_total_weight, 0, 8, s) != cudaSuccess)
     return record_cuda(h, __LINE__);
-  launch_finalize(d_chosen, m, d_w, d_msf_ids, d_msf_count, (u64 *)d_total_weight, next_scan(h, CNT_AUX), s);
-  return record(h, readback(h, s));
+  const uint32_t seq = next_readback(h);
+  launch_finish(FinishArgs{d_chosen, (m + 31) / 32, d_w, d_msf_ids, d_msf_count, (u64 *)d_total_weight,
+                           next_scan(h, CNT_AUX), nullptr, h->ds, h->hs_dev, h->hflag_dev, seq},
+                h->sms, s);
+  return record(h, readback_wait(h, s, seq, 0));
 }
 
 }  // extern "C"
