@@ -574,6 +574,7 @@ __global__ void __launch_bounds__(T, 1) block_single_kernel(const __grid_constan
     *out_count = sh.cnt;
     *a.totals = sh.wsum;
   }
+  publish_state(a.rb);
 }
 
 constexpr size_t BIG_SMEM = 224 * 1024, MID_SMEM = BLOCK_MID_N * 4, SMALL_SMEM = BLOCK_SMALL_N * 4;

@@ -68,6 +68,19 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t &t
   return s_warp[wid] + incl - x;
 }
 
+// Copies the device state into the mapped host mirror, then publishes seq in the
+// mapped flag word: by one block, behind its own stores and all it has seen.
+// The system-scope fence orders them and the mirror's words before the flag.
+__device__ __forceinline__ void publish_state(const Readback &rb) {
+  static_assert(sizeof(DevState) % 4 == 0, "DevState is copied in words");
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < (uint32_t)(sizeof(DevState) / 4); i += blockDim.x)
+    reinterpret_cast<volatile uint32_t *>(rb.mirror)[i] = __ldcg(reinterpret_cast<const uint32_t *>(rb.state) + i);
+  __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) *reinterpret_cast<volatile uint32_t *>(rb.flag) = rb.seq;
+}
+
 // Adds this thread's sum of chosen weights into a spread counter: one atomic
 // per warp (all 32 lanes call together).
 __device__ __forceinline__ void wsum_add(u64 *wsum, u64 v) {

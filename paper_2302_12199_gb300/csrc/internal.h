@@ -44,6 +44,14 @@ constexpr uint32_t GIANT_SAMPLES = 1024, GIANT_MIN_COUNT = 512;
 // input); CNT_LVL + LVL_MAX + k: the filtered heavy edges of level k.
 enum { CNT_EDGES = 0, CNT_ACTIVE = 1, CNT_TMP = 2, CNT_AUX = 3, CNT_USER = 4, CNT_CUT = 5, CNT_LVL = 6 };
 
+// Where a kernel that ends a call leaves the device state for the host.
+struct Readback {
+  const DevState *state;
+  DevState *mirror;  // page-locked, mapped
+  uint32_t *flag;    // mapped word that the host polls for seq
+  uint32_t seq;
+};
+
 // Output bookkeeping of a compaction launch.  Unordered compactions claim
 // their output ranges by atomic adds on *total (zero before the launch); the
 // ordered scan of the output ids exchanges its blocks' counts and writes *total.
@@ -208,13 +216,8 @@ struct FinishArgs {
   uint32_t *out_ids, *out_count;
   u64 *total_weight;
   ScanState st;
-  // with state: behind everything else the total from the WSUM_SLOTS counters
-  // (if wsum), the state to its host mirror, and seq to the host's flag
-  const u64 *wsum;
-  const DevState *state;
-  DevState *mirror;
-  uint32_t *flag;
-  uint32_t seq;
+  const u64 *wsum;    // WSUM_SLOTS counters whose sum is the total, or nullptr
+  Readback rb;        // behind everything else, if rb.state
 };
 void launch_finish(const FinishArgs &a, int sms, cudaStream_t s);
 // The giant component's root: the most frequent root among the labels of
@@ -321,6 +324,7 @@ struct BlockArgs {
   uint32_t *solved;
   uint32_t *err;
   uint32_t smem;               // set by the launchers
+  Readback rb;                 // at the end of launch_block_single
 };
 // kind: 0 the large graphs, 1 the middle ones, 2 the small ones.
 bool launch_block_batch(const BlockArgs &a, int kind, cudaStream_t s);

@@ -2534,14 +2534,7 @@ __global__ void __launch_bounds__(FB, 4) finish_kernel(FinishArgs a) {
       *a.total_weight = t;
     }
   }
-  if (!a.state) return;
-  constexpr uint32_t words = (uint32_t)(sizeof(DevState) / 4);
-  static_assert(sizeof(DevState) % 4 == 0, "DevState is copied in words");
-  for (uint32_t i = threadIdx.x; i < words; i += FB)
-    reinterpret_cast<volatile uint32_t *>(a.mirror)[i] = __ldcg(reinterpret_cast<const uint32_t *>(a.state) + i);
-  __threadfence_system();
-  __syncthreads();
-  if (threadIdx.x == 0) *reinterpret_cast<volatile uint32_t *>(a.flag) = a.seq;
+  if (a.rb.state) publish_state(a.rb);
 }
 
 // ---------------------------------------------------------------- launchers

@@ -349,18 +349,7 @@ void prof_resolve(mst_ctx *c) {
     prof_end(c, s, _p, kind, bytes, slot1, per1, slot2, per2, min_bytes);      \
   } while (0)
 
-// Copies the device state into the mapped host mirror, then publishes `seq`
-// in the mapped flag word (one warp, after everything before it on the
-// stream).  The system-scope fence orders the mirror's words before the flag.
-__global__ void readback_kernel(const DevState *ds, DevState *hs, uint32_t *flag, uint32_t seq) {
-  constexpr int words = (int)(sizeof(DevState) / 4);
-  const uint32_t *src = reinterpret_cast<const uint32_t *>(ds);
-  volatile uint32_t *dst = reinterpret_cast<volatile uint32_t *>(hs);
-  for (int i = threadIdx.x; i < words; i += 32) dst[i] = src[i];
-  __threadfence_system();
-  __syncwarp();
-  if (threadIdx.x == 0) *reinterpret_cast<volatile uint32_t *>(flag) = seq;
-}
+__global__ void readback_kernel(Readback rb) { publish_state(rb); }
 
 // The host side of a readback: the state of the device counters and flags
 // after all work queued on s so far.  The host spins on the mapped flag
@@ -368,9 +357,9 @@ __global__ void readback_kernel(const DevState *ds, DevState *hs, uint32_t *flag
 // synchronisation costs about ten); after about a second without the flag it
 // falls back to synchronising the stream, which also reports a CUDA error.
 // Error bits in `tolerated` are left for the caller to act on.
-uint32_t next_readback(mst_ctx *c) {
+Readback next_readback(mst_ctx *c) {
   ++c->readbacks;
-  return ++c->rb_seq;
+  return Readback{c->ds, c->hs_dev, c->hflag_dev, ++c->rb_seq};
 }
 mst_status readback_wait(mst_ctx *c, cudaStream_t s, uint32_t seq, uint32_t tolerated) {
   CK(cudaGetLastError());
@@ -395,10 +384,9 @@ mst_status readback_wait(mst_ctx *c, cudaStream_t s, uint32_t seq, uint32_t tole
   return MST_OK;
 }
 mst_status readback(mst_ctx *c, cudaStream_t s, uint32_t tolerated = 0) {
-  static_assert(sizeof(DevState) % 4 == 0, "DevState is copied in words");
-  const uint32_t seq = next_readback(c);
-  readback_kernel<<<1, 32, 0, s>>>(c->ds, c->hs_dev, c->hflag_dev, seq);
-  return readback_wait(c, s, seq, tolerated);
+  const Readback rb = next_readback(c);
+  readback_kernel<<<1, 128, 0, s>>>(rb);
+  return readback_wait(c, s, rb.seq, tolerated);
 }
 
 // Clears the error word, the jump flag and both scan counters (err, jump_flag
@@ -1345,12 +1333,12 @@ struct Solve {
   // Without out_ids the bitmap is all the caller wants.
   mst_status finalize(uint32_t *out_ids, uint32_t *out_count, u64 *total_weight, uint32_t tolerated = 0) {
     if (!out_ids) return readback(c, s, tolerated);
-    const uint32_t seq = next_readback(c);
+    const Readback rb = next_readback(c);
     PROF(MST_K_FINALIZE, (double)((m + 31) / 32 * 4), CNT_AUX, 4.0, -1, 0.0,
          launch_finish(FinishArgs{bits, (m + 31) / 32, nullptr, out_ids, out_count, total_weight,
-                                  next_scan(c, CNT_AUX), c->wsum, c->ds, c->hs_dev, c->hflag_dev, seq},
+                                  next_scan(c, CNT_AUX), c->wsum, rb},
                        c->sms, s));
-    return readback_wait(c, s, seq, tolerated);
+    return readback_wait(c, s, rb.seq, tolerated);
   }
 };
 
@@ -1375,11 +1363,12 @@ mst_status solve_small(mst_ctx *c, uint32_t n, uint32_t m, const uint32_t *src, 
   a.bits = (uint32_t *)(b += SINGLE_MAX_N * sizeof(u64));
   a.totals = total_weight;
   a.err = &c->ds->err;
+  a.rb = next_readback(c);
   PROF(MST_K_BASE, 12.0 * (double)m + 4.0 * (double)n, -1, 0.0, -1, 0.0,
        ran = launch_block_single(a, n, m, out_ids, out_count, s));
   if (!ran) return MST_OK;
   ++c->solves;
-  return readback(c, s);
+  return readback_wait(c, s, a.rb.seq, 0);
 }
 
 // bits_out (zeroed by the caller): the forest as a bitmap over the edges
@@ -2548,11 +2537,11 @@ mst_status mst_step_finalize(mst_handle h, uint64_t m, const uint32_t *d_chosen,
   cudaStream_t s = (cudaStream_t)stream;
   if (clear_device_flags(h, s) != MST_OK || cudaMemsetAsync(d_total_weight, 0, 8, s) != cudaSuccess)
     return record_cuda(h, __LINE__);
-  const uint32_t seq = next_readback(h);
+  const Readback rb = next_readback(h);
   launch_finish(FinishArgs{d_chosen, (m + 31) / 32, d_w, d_msf_ids, d_msf_count, (u64 *)d_total_weight,
-                           next_scan(h, CNT_AUX), nullptr, h->ds, h->hs_dev, h->hflag_dev, seq},
+                           next_scan(h, CNT_AUX), nullptr, rb},
                 h->sms, s);
-  return record(h, readback_wait(h, s, seq, 0));
+  return record(h, readback_wait(h, s, rb.seq, 0));
 }
 
 }  // extern "C"
