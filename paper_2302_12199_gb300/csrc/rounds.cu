@@ -24,9 +24,10 @@ namespace mstgpu {
 namespace {
 
 constexpr int RB = 512;            // threads per block; two blocks per SM (64 registers)
-constexpr int RI = 4;              // edges per thread and tile of a long list
+constexpr int RI = 4;              // edges per thread at a time of a long list
 constexpr int RT = RB * RI;        // edges per tile of a long list
 constexpr int RW = RB / 32;
+constexpr int GROUP = 4;           // warps that claim output places together
 constexpr int HI = 16;             // vertices per thread and tile of a long hooking pass
 constexpr uint32_t ROOT = 0x80000000u;  // link entry: a root with its next-round id, or a resolved vertex
 constexpr uint32_t FIN = 0xffffffffu;   // link entry: component without edges left
@@ -52,7 +53,7 @@ constexpr uint64_t SOLO_EDGES = 4096, SOLO_VERTS = 4096;
 constexpr uint32_t BAR_SPINS = 1u << 24;  // polls of the grid barrier before giving up
 
 struct Smem {
-  uint32_t out[4][RT];  // a tile's survivors (hooking: its vertices)
+  uint32_t out[4][RT];  // a hooking tile's vertices; the relabel's claims
   u64 tab[STAB];        // per-block minima of a round with few components
 };
 static_assert(PAIRS * sizeof(u64) + LABS <= sizeof(Smem), "pairs and labels fit");
@@ -316,121 +317,92 @@ __device__ __forceinline__ void jump_phase(const RoundsArgs &a, int r, uint64_t 
 }
 
 // Relabel, self-loop removal and compaction of the round's list, with the next
-// round's minEdges on the survivors (Section 4.3).  Tiles of 512 * I edges.
-// Survivors are staged in shared memory for coalesced stores; the minima are
-// relaxed from there, so that a warp's gathers have no idle lanes.  `tab`:
-// collect the minima in shared memory first.  A long list's tiles are bound by
-// the label and best[] gathers (four per edge, one L1 line each), so shared
-// memory is kept small for L1's sake: with the next tile copied ahead into a
-// shared-memory stage (160 KB per SM instead of 128) RMAT n=2^22 m=2^26 took
-// 4.36 ms per plain solve instead of 4.18; 192 KB: 4.53, 224 KB: 5.96.  One
-// block of 1024 threads per SM, or four of 256: 4.45, 4.58.
+// round's minEdges on the survivors (Section 4.3).  A warp takes 32 * I edges at
+// a time; the GROUP warps of a group claim their survivors' places with one
+// atomic, and write them from registers (a store's lanes are dense).  `tab`:
+// collect the minima in shared memory first.  Bound by the label and best[]
+// gathers, four per edge, which warps that wait for no more than their group
+// keep coming: with whole blocks passing from load to gather to a staged store
+// behind barriers, RMAT n=2^22 m=2^26 took 1180 and 840 us for its first two
+// relabels (905 and 610 now, 296 G gathers/s), RGG2D n=2^22 200 and 112 (155 and
+// 92), GNM n=2^16 m=2^20 14.0 (7.5).  A claim per warp queues at the counter
+// and scatters neighbours over the next list (1040, 707; 169, 119); groups of
+// eight wait longer (942, 639; 165, 104).
 template <int I>
 __device__ __forceinline__ void relabel_phase(const RoundsArgs &a, KeyLayout kl, int r, uint64_t m, uint64_t off,
-                                           bool tab, uint32_t nb, uint32_t bid, Smem &sm, uint32_t *s_warp,
-                                           uint32_t *s_base) {
+                                               bool tab, uint32_t nb, uint32_t bid, Smem &sm) {
   const uint32_t *link = r == 0 ? a.parent : a.link + off;
   const EdgeOut out = a.list[(a.first_slot + r) & 1], prev = a.list[(a.first_slot + r + 1) & 1];
   const EdgeList in = r == 0 ? a.in : EdgeList{prev.u, prev.v, prev.w, prev.id};
   u64 *counter = &a.st->ce[r];
-  constexpr uint64_t T = (uint64_t)RB * I;
-  const uint64_t nfull = I == RI && aligned16_list(in) ? m / T : 0;
-  for (uint64_t tile = bid; tile * T < m; tile += nb) {
-    const uint64_t j0 = tile * T + (uint64_t)I * threadIdx.x;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t below = (1u << lane) - 1u;
+  uint32_t *s_tot = &sm.out[0][0], *s_pos = s_tot + RW;  // per warp, per group
+  for (uint64_t tile = (uint64_t)bid * RW + wid; tile / GROUP * GROUP * (32 * I) < m; tile += (uint64_t)nb * RW) {
+    const uint64_t j0 = tile * (32 * I) + lane;
     uint32_t eu[I], ev[I], ew[I], ei[I];
-    uint32_t valid = 0;
-    bool whole = false;
-    if constexpr (I == RI) {
-      if (tile < nfull) {
-        whole = true;
-        const uint4 x = __ldcg(reinterpret_cast<const uint4 *>(in.u + j0));
-        const uint4 y = __ldcg(reinterpret_cast<const uint4 *>(in.v + j0));
-        const uint4 z = __ldcg(reinterpret_cast<const uint4 *>(in.w + j0));
-        eu[0] = x.x, eu[1] = x.y, eu[2] = x.z, eu[3] = x.w;
-        ev[0] = y.x, ev[1] = y.y, ev[2] = y.z, ev[3] = y.w;
-        ew[0] = z.x, ew[1] = z.y, ew[2] = z.z, ew[3] = z.w;
-        if (in.id) {
-          const uint4 t = __ldcg(reinterpret_cast<const uint4 *>(in.id + j0));
-          ei[0] = t.x, ei[1] = t.y, ei[2] = t.z, ei[3] = t.w;
-        } else {
 #pragma unroll
-          for (int k = 0; k < I; ++k) ei[k] = (uint32_t)(j0 + k);
-        }
-        valid = (1u << I) - 1u;
-      }
-    }
-    if (!whole) {
-#pragma unroll
-      for (int k = 0; k < I; ++k) {
-        const bool ok = j0 + k < m;
-        eu[k] = ok ? __ldca(in.u + j0 + k) : 0u;
-        ev[k] = ok ? __ldca(in.v + j0 + k) : 0u;
-        ew[k] = ok ? __ldca(in.w + j0 + k) : 0u;
-        ei[k] = ok ? (in.id ? __ldca(in.id + j0 + k) : (uint32_t)(j0 + k)) : 0u;
-        valid |= (ok ? 1u : 0u) << k;
-      }
+    for (int k = 0; k < I; ++k) {
+      const uint64_t j = j0 + 32 * k;
+      const bool ok = j < m;
+      eu[k] = ok ? __ldcg(in.u + j) : 0u;
+      ev[k] = ok ? __ldcg(in.v + j) : eu[k];
+      ew[k] = ok ? __ldcg(in.w + j) : 0u;
+      ei[k] = ok && in.id ? __ldcg(in.id + j) : (uint32_t)j;
     }
 #pragma unroll
     for (int k = 0; k < I; ++k) {
-      eu[k] = (valid >> k & 1) ? __ldca(link + eu[k]) & ~ROOT : 0u;
-      ev[k] = (valid >> k & 1) ? __ldca(link + ev[k]) & ~ROOT : 0u;
+      const bool self = eu[k] == ev[k];
+      eu[k] = self ? 0u : __ldca(link + eu[k]) & ~ROOT;
+      ev[k] = self ? 0u : __ldca(link + ev[k]) & ~ROOT;
     }
-    uint32_t keep = 0;
+    uint32_t keep[I], total = 0;
 #pragma unroll
-    for (int k = 0; k < I; ++k) keep |= (eu[k] != ev[k] ? 1u : 0u) << k;
-    uint32_t total;
-    uint32_t p = block_exclusive_scan<RB>((uint32_t)__popc(keep), total, s_warp);
-    if (threadIdx.x == 0) s_base[0] = total ? (uint32_t)atomicAdd(counter, (u64)total) : 0u;
+    for (int k = 0; k < I; ++k) {
+      keep[k] = __ballot_sync(0xffffffffu, eu[k] != ev[k]);
+      total += __popc(keep[k]);
+    }
+    if (lane == 0) s_tot[wid] = total;
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + wid / GROUP), "n"(32 * GROUP) : "memory");
+    uint32_t sum = 0, mine = 0;
 #pragma unroll
-    for (int k = 0; k < I; ++k)
-      if (keep >> k & 1) {
-        sm.out[0][p] = eu[k];
-        sm.out[1][p] = ev[k];
-        sm.out[2][p] = ew[k];
-        sm.out[3][p] = ei[k];
-        ++p;
+    for (int q = 0; q < GROUP; ++q) {
+      const uint32_t t = s_tot[wid / GROUP * GROUP + q];
+      mine += q < wid % GROUP ? t : 0u;
+      sum += t;
+    }
+    if (wid % GROUP == 0 && lane == 0) s_pos[wid / GROUP] = sum ? (uint32_t)atomicAdd(counter, (u64)sum) : 0u;
+    u64 cx[I], cy[I];
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+      const bool has = eu[k] != ev[k];
+      cx[k] = !has ? 0ULL : tab ? sm.tab[eu[k]] : __ldca(a.best + eu[k]);
+      cy[k] = !has ? 0ULL : tab ? sm.tab[ev[k]] : __ldca(a.best + ev[k]);
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + wid / GROUP), "n"(32 * GROUP) : "memory");
+    uint32_t p = s_pos[wid / GROUP] + mine;
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+      const uint32_t o = p + __popc(keep[k] & below);
+      p += __popc(keep[k]);
+      if (eu[k] == ev[k]) continue;
+      out.u[o] = eu[k];
+      out.v[o] = ev[k];
+      out.w[o] = ew[k];
+      out.id[o] = ei[k];
+      const u64 kx = relax_key(kl, ew[k], ei[k], ev[k]), ky = relax_key(kl, ew[k], ei[k], eu[k]);
+      if (tab) {
+        if (kx < cx[k]) atomicMin(&sm.tab[eu[k]], kx);
+        if (ky < cy[k]) atomicMin(&sm.tab[ev[k]], ky);
+      } else {
+        relax(a.best, eu[k], kx, cx[k]);
+        relax(a.best, ev[k], ky, cy[k]);
       }
-    __syncthreads();
-    const uint64_t ob = s_base[0];
-    constexpr int E = I > 2 ? 2 : I;  // survivors in flight per thread
-    for (uint32_t i0 = 0; i0 < total; i0 += E * RB) {
-      uint32_t x[E], y[E], id[E];
-      u64 kx[E], ky[E], cx[E], cy[E];
-#pragma unroll
-      for (int k = 0; k < E; ++k) {
-        const uint32_t i = i0 + k * RB + threadIdx.x;
-        kx[k] = ky[k] = KEY_INF;
-        cx[k] = cy[k] = 0;
-        x[k] = y[k] = id[k] = 0;
-        if (i < total) {
-          x[k] = sm.out[0][i], y[k] = sm.out[1][i], id[k] = sm.out[3][i];
-          const uint32_t w = sm.out[2][i];
-          kx[k] = relax_key(kl, w, id[k], y[k]);
-          ky[k] = relax_key(kl, w, id[k], x[k]);
-          cx[k] = tab ? sm.tab[x[k]] : __ldca(a.best + x[k]);
-          cy[k] = tab ? sm.tab[y[k]] : __ldca(a.best + y[k]);
-          out.u[ob + i] = x[k];
-          out.v[ob + i] = y[k];
-          out.w[ob + i] = w;
-          out.id[ob + i] = id[k];
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < E; ++k) {
-        if (tab) {
-          if (kx[k] < cx[k]) atomicMin(&sm.tab[x[k]], kx[k]);
-          if (ky[k] < cy[k]) atomicMin(&sm.tab[y[k]], ky[k]);
-        } else {
-          relax(a.best, x[k], kx[k], cx[k]);
-          relax(a.best, y[k], ky[k], cy[k]);
-        }
-        if (!kl.packed && kx[k] != KEY_INF) {
-          a.cur_u[id[k]] = x[k];
-          a.cur_v[id[k]] = y[k];
-        }
+      if (!kl.packed) {
+        a.cur_u[ei[k]] = eu[k];
+        a.cur_v[ei[k]] = ev[k];
       }
     }
-    __syncthreads();  // the output stage, s_warp and s_base are reused by the next tile
   }
 }
 
@@ -682,10 +654,11 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
       __syncthreads();
     }
     if (s_m >= (uint64_t)RT * g.nb)
-      relabel_phase<RI>(a, kl, r, s_m, s_off[r], tab, g.nb, g.bid, sm, s_warp, s_base);
+      relabel_phase<RI>(a, kl, r, s_m, s_off[r], tab, g.nb, g.bid, sm);
     else
-      relabel_phase<1>(a, kl, r, s_m, s_off[r], tab, g.nb, g.bid, sm, s_warp, s_base);
+      relabel_phase<1>(a, kl, r, s_m, s_off[r], tab, g.nb, g.bid, sm);
     if (tab) {  // one atomic per component and block at most
+      __syncthreads();
       for (uint32_t i = threadIdx.x; i < (uint32_t)s_nn; i += RB) {
         const u64 k = sm.tab[i];
         if (k != KEY_INF) relax(a.best, i, k, __ldca(a.best + i));
