@@ -415,13 +415,13 @@ __device__ __noinline__ void pair_clear(uint32_t *table_mem, uint32_t np, uint32
 // Relabel of a round that leaves few components (at most PAIR_COMPS): of the
 // edges between two components only the lightest can be in the forest, so the
 // list shrinks to one entry per pair at once, and block 0 finishes the call
-// alone.  Every block collects its pairs' minima in shared memory and then
+// on them.  Every block collects its pairs' minima in shared memory and then
 // sends them to the table; nothing is staged or written per edge, and an edge's
 // id is read only where its weight is not above the pair's minimum.  Bound by
 // reading 12 bytes per edge: RMAT n=2^22 m=2^26, which keeps 64 million edges
 // until its last rounds, passes over them in 227 us (3.4 TB/s; the shared-memory
 // lookups are the rest), where relabel, minEdges and three more rounds took
-// 1260 us; GNM n=2^16 m=2^20 ends in 50 us instead of 75.  The pair functions
+// 1260 us.  The pair functions
 // are calls, with their arguments by value: inlined, their registers cost the
 // long phases spills (RGG2D's first relabel 200 -> 223 us).
 template <int I>
@@ -492,57 +492,79 @@ __device__ __noinline__ void pair_phase(EdgeList in, const uint32_t *link, uint6
   }
 }
 
-// The pairs that have an edge as the next round's list, with its minEdges; one
-// block.  Returns the edges.
-__device__ __noinline__ uint32_t pair_list(EdgeOut out, KeyLayout kl, uint32_t *cur_u, uint32_t *cur_v, u64 *best,
-                                           uint32_t nn, uint32_t *s_warp) {
+// The call's last rounds over the table of pairs, in one block's shared memory:
+// a warp looks through a component's row, and everything else is one thread per
+// component: about 2 us a round, where writing the pairs as a list took 9 and
+// each round over it 7 (GNM n=2^16 m=2^20, 108 components left: 229 -> 204 us).
+// rep: representatives of the nn components, replaced by those of their final
+// ones; or nullptr.
+__device__ __noinline__ void pair_rounds(const uint32_t *table_mem, uint32_t nn, uint32_t *chosen_bits, u64 *wsum,
+                                         uint32_t *rep) {
   extern __shared__ __align__(128) unsigned char smem_dyn[];
-  u64 *pt = reinterpret_cast<u64 *>(smem_dyn);
-  const uint32_t np = nn * (nn - 1) / 2;
-  // the list overlays the table
-  for (uint32_t i = threadIdx.x; i < np; i += RB) pt[i] = __ldcg(reinterpret_cast<u64 *>(out.u) + i);
-  __syncthreads();
-  // warp w writes the pairs [w * per, (w + 1) * per)
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint32_t per = ((np + RW - 1) / RW + 31u) & ~31u, i0 = wid * per, i1 = min(np, i0 + per);
-  uint32_t cnt = 0, total;
-  for (uint32_t b = i0; b < i1; b += 32)
-    cnt += __popc(__ballot_sync(0xffffffffu, b + lane < i1 && pt[b + lane] != KEY_INF));
-  uint32_t o = block_exclusive_scan<RB>(lane == 0 ? cnt : 0u, total, s_warp);
-  o = __shfl_sync(0xffffffffu, o, 0);
-  for (uint32_t b = i0; b < i1; b += 32) {
-    const uint32_t i = b + lane;
-    const u64 k = i < i1 ? pt[i] : KEY_INF;
-    const uint32_t has = __ballot_sync(0xffffffffu, k != KEY_INF);
-    if (k != KEY_INF) {
-      uint32_t hi = (uint32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)i)) * 0.5f);  // hi (hi - 1) / 2 <= i, one off at most
-      if (hi * (hi - 1) / 2 > i) --hi;
-      if (hi * (hi + 1) / 2 <= i) ++hi;
-      const uint32_t lo = i - hi * (hi - 1) / 2, id = (uint32_t)k, p = o + __popc(has & ((1u << lane) - 1u));
-      out.u[p] = hi, out.v[p] = lo, out.w[p] = (uint32_t)(k >> 32), out.id[p] = id;
-      if (!kl.packed) cur_u[id] = hi, cur_v[id] = lo;
-    }
-    o += __popc(has);
-  }
-  // minEdges: a warp per component, over its pairs
-  for (uint32_t c = wid; c < nn; c += RW) {
-    u64 k = KEY_INF;
-    uint32_t other = 0;
-    for (uint32_t d = lane; d < nn; d += 32) {
-      const uint32_t h = max(c, d);
-      const u64 q = c == d ? KEY_INF : pt[h * (h - 1) / 2 + min(c, d)];
-      if (q < k) k = q, other = d;
-    }
+  u64 *pt = reinterpret_cast<u64 *>(smem_dyn), *s_cmin = pt + PAIRS, *s_rmin = s_cmin + PAIR_COMPS;
+  uint32_t *s_lab = reinterpret_cast<uint32_t *>(s_rmin + PAIR_COMPS), *s_far = s_lab + PAIR_COMPS,
+           *s_part = s_far + PAIR_COMPS, *s_next = s_part + PAIR_COMPS;
+  static_assert((PAIRS + 2 * PAIR_COMPS) * sizeof(u64) + 4 * PAIR_COMPS * sizeof(uint32_t) <= sizeof(Smem), "fits");
+  const uint32_t t = threadIdx.x, lane = t & 31, wid = t >> 5, np = nn * (nn - 1) / 2;
+  const bool comp = t < nn;
+  for (uint32_t i = t; i < np; i += RB) pt[i] = __ldcg(reinterpret_cast<const u64 *>(table_mem) + i);
+  if (comp) s_lab[t] = t;
+  u64 wacc = 0;
+  for (uint32_t round = 0; round < nn; ++round) {  // every round but the last merges
+    if (comp) s_cmin[t] = KEY_INF;
+    __syncthreads();
+    for (uint32_t c = wid; c < nn; c += RW) {
+      const uint32_t lc = s_lab[c];
+      u64 k = KEY_INF;
+      uint32_t far = 0;
+      for (uint32_t d = lane; d < nn; d += 32) {
+        if (s_lab[d] == lc) continue;
+        const uint32_t h = max(c, d);
+        const u64 q = pt[h * (h - 1) / 2 + min(c, d)];
+        if (q < k) k = q, far = d;
+      }
 #pragma unroll
-    for (int x = 16; x > 0; x >>= 1) {
-      const u64 q = __shfl_xor_sync(0xffffffffu, k, x);
-      const uint32_t d = __shfl_xor_sync(0xffffffffu, other, x);
-      if (q < k) k = q, other = d;
+      for (int x = 16; x > 0; x >>= 1) {
+        const u64 q = __shfl_xor_sync(0xffffffffu, k, x);
+        const uint32_t d = __shfl_xor_sync(0xffffffffu, far, x);
+        if (q < k) k = q, far = d;
+      }
+      if (lane == 0) {
+        s_rmin[c] = k;
+        s_far[c] = far;
+        if (k != KEY_INF) atomicMin(s_cmin + lc, k);
+      }
     }
-    if (lane == 0 && k != KEY_INF) best[c] = relax_key(kl, (uint32_t)(k >> 32), (uint32_t)k, other);
+    __syncthreads();
+    // (an edge has one end in a component, so one row holds its minimum)
+    if (comp && s_rmin[t] != KEY_INF && s_rmin[t] == s_cmin[s_lab[t]]) s_part[s_lab[t]] = s_lab[s_far[t]];
+    __syncthreads();
+    bool merges = false;
+    if (comp && s_lab[t] == t) {
+      const u64 k = s_cmin[t];
+      merges = k != KEY_INF;
+      const uint32_t y = merges ? s_part[t] : t;
+      const bool root = !merges || (s_cmin[y] == k && t < y);
+      s_next[t] = root ? t : y;
+      if (!root) {
+        atomicOr(chosen_bits + ((uint32_t)k >> 5), 1u << (k & 31));
+        wacc += k >> 32;
+      }
+    }
+    if (!__syncthreads_or(merges)) break;
+    if (comp) {
+      uint32_t q = s_next[s_lab[t]];
+      for (uint32_t s = 0; s < nn && s_next[q] != q; ++s) q = s_next[q];
+      s_lab[t] = q;
+    }
   }
-  __syncthreads();
-  return total;
+  wsum_add(wsum, wacc);
+  if (rep) {
+    __syncthreads();
+    const uint32_t v = comp ? rep[s_lab[t]] : 0u;
+    __syncthreads();
+    if (comp) rep[t] = v;
+  }
 }
 
 // The call's vertices (act) back to representatives in the caller's numbering:
@@ -638,15 +660,9 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
       if (!(ok = g.sync())) break;
       alone = alone || !g.solo;
       if (blockIdx.x != 0) break;
-      const uint32_t left = pair_list(out, kl, a.cur_u, a.cur_v, a.best, (uint32_t)s_nn, s_warp);
-      if (threadIdx.x == 0) {
-        s_m = left;
-        s_nc = s_nn;
-      }
-      __syncthreads();
-      g.solo = true;
-      g.nb = 1;
-      continue;
+      ++r;
+      pair_rounds(out.u, (uint32_t)s_nn, a.chosen_bits, a.wsum, a.want_parent ? a.rep + s_off[r] : nullptr);
+      break;
     }
     const bool tab = s_nn <= STAB;
     if (tab) {
