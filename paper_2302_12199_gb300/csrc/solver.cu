@@ -1240,7 +1240,12 @@ struct Solve {
       caps[K + 1] = light_cap(caps[K]);
       ++K;
     }
-    if (leaf_top != (K == 1)) return MST_OK;  // the light count moved the deepest level: host-driven
+    // The light count may come out on the other side of the sparsity bound than
+    // expected.  A list 1 that was written as the deepest (best[] relaxed) stays
+    // that: it is a few percent longer than the bound.  One that was not gets its
+    // minEdges below.  (Starting over on the host-driven path instead cost GNM
+    // n=2^20 m=2^23, whose light list is as long as the bound, 150 us of 720.)
+    if (leaf_top) K = 1;
     const uint64_t need = plan_round_edges(caps[K]);
     if (need > X.cap) TRY(round_lists(c, need, X, Y, s));  // (not when leaf_top: X already holds list 1)
     planned = true;
@@ -1279,7 +1284,13 @@ struct Solve {
                  ProfTerm{CNT_LVL + k, 16.0, 16.0}, ProfTerm{CNT_LVL + k + 1, 16.0, 16.0});
       E[k + 1] = last ? X.list() : Lb[k + 1].list();
     }
-    TRY(boruvka_planned(X, Y, CNT_LVL + K, cur_u != nullptr, false));
+    if (K == 1 && !leaf_top) {
+      bool ran = false;
+      TRY(boruvka_device(E[1], m1, false, false, false, ran));
+      if (!ran) return MST_ERR_CUDA;
+    } else {
+      TRY(boruvka_planned(X, Y, CNT_LVL + K, cur_u != nullptr, false));
+    }
 
     // levels K-1 .. 0: contract P and mark the giant component, filter the
     // level's heavy edges into X, and solve them
