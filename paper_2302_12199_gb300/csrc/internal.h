@@ -206,6 +206,10 @@ struct InitArgs {
   uint64_t words;
   uint32_t *zero;    // [zero_words] zero: the handle's counters
   uint64_t zero_words;
+  // with w: the largest of its m weights in *max_w (zero before), and *max_next zero
+  const uint32_t *w;
+  uint64_t m;
+  uint32_t *max_w, *max_next;
 };
 void launch_init(const InitArgs &a, int sms, cudaStream_t s);
 // The bitmap's ids in ascending order and their number.

@@ -1146,26 +1146,29 @@ __global__ void hash_insert_kernel(EdgeList in, uint64_t m, HashSlot *table, uin
   }
 }
 
-__global__ void __launch_bounds__(BLOCK) max_weight_kernel(const uint32_t *w, uint64_t m, uint32_t *out) {
+// *out = max(*out, the weights); `t` of `stride` threads, whole warps.
+__device__ __forceinline__ void max_weight(const uint32_t *w, uint64_t m, uint64_t t, uint64_t stride, uint32_t *out) {
   uint32_t mx = 0;
   const uint64_t nv = ((uintptr_t)w & 15u) ? 0 : m / 4;  // 16-byte vectors
   const uint4 *w4 = reinterpret_cast<const uint4 *>(w);
-  const uint64_t stride = (uint64_t)gridDim.x * BLOCK;
-  uint64_t i = (uint64_t)blockIdx.x * BLOCK + threadIdx.x;
+  uint64_t i = t;
   for (; i + 3 * stride < nv; i += 4 * stride) {
-    const uint4 a = __ldcs(w4 + i), b = __ldcs(w4 + i + stride), c = __ldcs(w4 + i + 2 * stride),
-                d = __ldcs(w4 + i + 3 * stride);
+    const uint4 a = __ldg(w4 + i), b = __ldg(w4 + i + stride), c = __ldg(w4 + i + 2 * stride),
+                d = __ldg(w4 + i + 3 * stride);
     mx = max(mx, max(max(max(a.x, a.y), max(a.z, a.w)), max(max(b.x, b.y), max(b.z, b.w))));
     mx = max(mx, max(max(max(c.x, c.y), max(c.z, c.w)), max(max(d.x, d.y), max(d.z, d.w))));
   }
   for (; i < nv; i += stride) {
-    const uint4 a = __ldcs(w4 + i);
+    const uint4 a = __ldg(w4 + i);
     mx = max(mx, max(max(a.x, a.y), max(a.z, a.w)));
   }
-  for (uint64_t j = nv * 4 + (uint64_t)blockIdx.x * BLOCK + threadIdx.x; j < m; j += stride) mx = max(mx, w[j]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0 && mx) atomicMax(out, mx);
+  for (uint64_t j = nv * 4 + t; j < m; j += stride) mx = max(mx, __ldg(w + j));
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0 && mx > __ldcg(out)) atomicMax(out, mx);
+}
+
+__global__ void __launch_bounds__(BLOCK) max_weight_kernel(const uint32_t *w, uint64_t m, uint32_t *out) {
+  max_weight(w, m, (uint64_t)blockIdx.x * BLOCK + threadIdx.x, (uint64_t)gridDim.x * BLOCK, out);
 }
 
 // Sets ERR_VERTEX if some x[i] (i < count) is >= bound.
@@ -2397,7 +2400,9 @@ __global__ void giant_bits_kernel(const uint32_t *P, uint32_t n, const uint32_t 
 // ------------------------------------------------------------ start and end
 
 // The state a solve starts from: best[] at infinity, every vertex its own
-// representative, no edge chosen, counters zero.  One launch of plain stores
+// representative, no edge chosen, counters zero; for plain rounds also the
+// largest weight (a launch of its own took 7 us more: plain solves of the grid
+// 2048 x 2048 595 -> 588 us, of RGG3D n=2^21 609 -> 602).  One launch of plain stores
 // instead of six memsets and a kernel, which took 30 us of a small solve, most of
 // it between launches; n=2^18, m=2^22: 2.3 us, n=2^24, m=2^28: 35 us (6.7 TB/s).
 __global__ void __launch_bounds__(BLOCK) init_kernel(InitArgs a) {
@@ -2408,6 +2413,10 @@ __global__ void __launch_bounds__(BLOCK) init_kernel(InitArgs a) {
   }
   for (uint64_t i = t; i < a.words; i += stride) a.bits[i] = 0;
   for (uint64_t i = t; i < a.zero_words; i += stride) a.zero[i] = 0;
+  if (a.w) {
+    if (t == 0) *a.max_next = 0;
+    max_weight(a.w, a.m, t, stride, a.max_w);
+  }
 }
 
 // Output (Section 2.2; edge ids, Section 6.2): set bits of the chosen-edge
@@ -2760,7 +2769,7 @@ bool launch_pivot_coop(EdgeList in, uint64_t m, u64 state, uint32_t sample, u64 
 }
 
 void launch_init(const InitArgs &a, int sms, cudaStream_t s) {
-  const uint64_t most = std::max(std::max((uint64_t)a.n, a.words), a.zero_words);
+  const uint64_t most = std::max(std::max((uint64_t)a.n, a.words), std::max(a.zero_words, a.w ? a.m / 4 : 0));
   init_kernel<<<grid_for((most + BLOCK - 1) / BLOCK, sms, 8), BLOCK, 0, s>>>(a);
 }
 

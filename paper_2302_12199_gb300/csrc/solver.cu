@@ -39,6 +39,8 @@ struct mst_ctx {
   uint64_t readbacks = 0;
   u64 *hres = nullptr;       // pinned host words for the forest size and weight of the host entry points
   uint32_t *scan_count = nullptr;  // the output scan's counts per block
+  uint32_t *max_slots = nullptr;   // largest weight of a solve whose start finds it: this solve's and the next one's
+  int max_slot = 0;
   u64 *sample_buf = nullptr;
   uint32_t sample_cap = 0;
   void *pivot_scratch = nullptr;  // histograms of the multi-block pivot selection
@@ -470,6 +472,7 @@ struct Solve {
   }
   u64 *best = nullptr;
   uint32_t *parent = nullptr, *act[2] = {nullptr, nullptr}, *bits = nullptr;
+  uint32_t *max_found = nullptr;  // largest weight, found by start()
   int wbits = 32;  // bits of the largest weight (set with the key layout)
   int rounds = 0;
   bool want_parent = true;  // representatives are read after a Borůvka call (the filter contracts them)
@@ -480,7 +483,9 @@ struct Solve {
       : c(c_), s(s_), n(n_), m(m_), shape(shape_index(c_->cfg.block_threads, c_->cfg.items_per_thread)),
         rshape(relabel_shape_index(c_->cfg.relabel_block_threads, c_->cfg.relabel_items_per_thread)) {}
 
-  mst_status init(uint32_t *parent_external = nullptr, uint32_t *bits_external = nullptr) {
+  // max_of: weights whose largest the first rounds will ask for (max_found), or nullptr
+  mst_status init(uint32_t *parent_external = nullptr, uint32_t *bits_external = nullptr,
+                  const uint32_t *max_of = nullptr) {
     TRY(best_b.alloc(c, (size_t)n * 8, s));
     best = best_b.as<u64>();
     if (parent_external) {
@@ -497,12 +502,18 @@ struct Solve {
       TRY(bits_b.alloc(c, (m + 31) / 32 * 4, s));
       bits = bits_b.as<uint32_t>();
     }
-    return start(bits_external == nullptr);
+    return start(bits_external == nullptr, max_of);
   }
   // Everything at its initial value, the handle's counters and flags included
   // (so that a launch that failed earlier leaves nothing behind for this call).
-  mst_status start(bool clear_bits) {
-    launch_init(InitArgs{best, parent, n, bits, clear_bits ? (m + 31) / 32 : 0, (uint32_t *)c->ds, c->zero_words},
+  mst_status start(bool clear_bits, const uint32_t *max_of = nullptr) {
+    max_found = nullptr;
+    if (max_of) {
+      max_found = c->max_slots + c->max_slot;
+      c->max_slot ^= 1;
+    }
+    launch_init(InitArgs{best, parent, n, bits, clear_bits ? (m + 31) / 32 : 0, (uint32_t *)c->ds, c->zero_words,
+                         max_of, m, max_found, c->max_slots + c->max_slot},
                 c->sms, s);
     CK(cudaGetLastError());
     c->rounds_used = 0;
@@ -779,8 +790,11 @@ struct Solve {
     TRY(rounds_alloc());
     const uint32_t *max_w = nullptr;
     if (!layout_set) {  // the kernel picks the key layout from the largest weight
-      launch_max_weight(w_in ? w_in : E.w, m, &c->ds->max_w, c->sms, s);
-      max_w = &c->ds->max_w;
+      max_w = max_found;
+      if (!max_w) {
+        launch_max_weight(w_in ? w_in : E.w, m, &c->ds->max_w, c->sms, s);
+        max_w = &c->ds->max_w;
+      }
       layout_bits();
       if (32 + kl.idbits + kl.vbits > 63) TRY(cur_alloc());  // the keys may not pack
     }
@@ -1404,14 +1418,15 @@ mst_status solve_device(mst_ctx *c, uint32_t n, uint64_t m, const uint32_t *src,
     if (ran) return MST_OK;
   }
   Solve S(c, s, n, m);
-  TRY(S.init(nullptr, bits_out));
+  const bool filt = use_filter(c->cfg, n, m);
+  const bool plain = !filt && c->cfg.tile_contract == 0 && !c->cfg.min_edges_sort && S.device_rounds();
+  TRY(S.init(nullptr, bits_out, plain ? w : nullptr));
   if (!bits_out) ++c->solves;
   S.src = src;
   S.dst = dst;
   S.w_in = w;
   const EdgeList in{src, dst, w, nullptr};
   c->pivot_counter = 0;
-  const bool filt = use_filter(c->cfg, n, m);
   ListBuf local;
   uint64_t m_local = 0;
   bool applied = false;
@@ -1894,7 +1909,7 @@ mst_status mst_create(mst_handle *out, const mst_config *cfg) {
   const size_t b_ds = round_up(sizeof(DevState), 256), b_piv = round_up(pivot_scratch_bytes(), 256),
                b_ws = round_up(WSUM_SLOTS * sizeof(u64), 256),
                b_rs = round_up(ROUNDS_STATES * sizeof(RoundsState), 256),
-               b_sc = round_up(FINISH_BLOCKS * sizeof(uint32_t), 256);
+               b_sc = round_up((FINISH_BLOCKS + 2) * sizeof(uint32_t), 256);
   const size_t b_zero = b_ds + b_ws + b_rs;  // what start() clears
   char *fixed = nullptr;
   ok = ok && cudaMalloc(&fixed, b_zero + b_piv + b_sc + SMALL_BYTES) == cudaSuccess;
@@ -1905,9 +1920,11 @@ mst_status mst_create(mst_handle *out, const mst_config *cfg) {
     c->zero_words = b_zero / 4;
     c->pivot_scratch = fixed + b_zero;
     c->scan_count = (uint32_t *)(fixed + b_zero + b_piv);
+    c->max_slots = c->scan_count + FINISH_BLOCKS;
     c->small_mem = fixed + b_zero + b_piv + b_sc;
   }
-  ok = ok && cudaMemset(fixed, 0, b_zero + b_piv) == cudaSuccess;  // the pivot selection leaves its scratch zero
+  // the pivot selection leaves its scratch zero, a solve's start the next one's slot
+  ok = ok && cudaMemset(fixed, 0, b_zero + b_piv + b_sc) == cudaSuccess;
   ok = ok && cudaHostAlloc(&c->hs, sizeof(DevState), cudaHostAllocMapped) == cudaSuccess;
   ok = ok && cudaHostGetDevicePointer((void **)&c->hs_dev, c->hs, 0) == cudaSuccess;
   ok = ok && cudaHostAlloc(&c->hflag, 64, cudaHostAllocMapped) == cudaSuccess;
