@@ -453,7 +453,7 @@ def gpu_main(args, rank: int, world: int, local_rank: int):
     solver.profile(False)
     stats_all = solver.profile_stats()
     # the dominant class among those whose bytes are counted (the graph
-    # class's are not: its kernels are counted in no class)
+    # class's, the one-launch rounds, are not)
     dom = max((k for k in stats_all if stats_all[k][2] > 0), key=lambda k: stats_all[k][1])
     sampler = ClockSampler(uuid)
     if dist:
@@ -685,8 +685,8 @@ def measure_batched(args, rank: int, world: int, local_rank: int, dev, dist, com
 
     # autotuned configuration (variant, dedupe strategy, tile contraction,
     # then the kernels' tile shape); each candidate keeps one handle across its
-    # runs, so the timed runs see the steady state (pool grown, round graphs
-    # built), not a handle's first solves
+    # runs, so the timed runs see the steady state (pool and round lists
+    # grown), not a handle's first solves
     trial_solver = {}
 
     def trial(cfg):
