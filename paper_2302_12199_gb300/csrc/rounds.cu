@@ -276,6 +276,65 @@ __device__ __forceinline__ void hook_phase(const RoundsArgs &a, const KeyLayout 
   wsum_add(a.wsum, wacc);
 }
 
+// The same for a short pass (rounds of few components, small calls): a lane per
+// vertex, and no block barriers; the GROUP warps of a group claim their roots'
+// ids, and in round 0 places in `act`, together.  A chain of L2 round trips
+// between two grid barriers: 3.4 us per round of GNM n=2^16 m=2^20 where the
+// tiles of the long pass took 4.7; 10.5 instead of 15.6 with 540,969 components.
+// Sparse first rounds need the tiles (RMAT n=2^24: 72 us, a lane per vertex 370).
+__device__ __forceinline__ void hook_short(const RoundsArgs &a, const KeyLayout &kl, int r, uint64_t nc, uint64_t off,
+                                           bool rec, uint32_t nb, uint32_t bid, Smem &sm) {
+  uint32_t *link = r == 0 ? a.parent : a.link + off;
+  const uint32_t *rep = a.rep + off;
+  uint32_t *rep_next = a.rep + (r == 0 ? 0 : off + nc);
+  const uint32_t *eu = rec ? a.cur_u : a.src, *ev = rec ? a.cur_v : a.dst;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t *s_tot = reinterpret_cast<uint32_t *>(sm.tab), *s_pos = s_tot + RW;  // per warp, two per group
+  const uint32_t below = (1u << lane) - 1u;
+  u64 wacc = 0;
+  for (uint64_t tile = (uint64_t)bid * RW + wid; tile / GROUP * GROUP * 32 < nc; tile += (uint64_t)nb * RW) {
+    const uint64_t c64 = tile * 32 + lane;
+    const uint32_t c = (uint32_t)c64;
+    const u64 k = c64 < nc ? a.best[c] : KEY_INF;
+    const bool act = k != KEY_INF;
+    bool root = false;
+    if (act) {
+      const uint32_t e = key_edge_id(kl, k);
+      const uint32_t oth = kl.packed ? (uint32_t)(k & ((1ULL << kl.vbits) - 1)) : __ldca(eu + e) ^ __ldca(ev + e) ^ c;
+      root = same_edge(kl, a.best[oth], k) && c < oth;
+      if (!root) {
+        link[c] = oth;
+        atomicOr(a.chosen_bits + (e >> 5), 1u << (e & 31));
+        wacc += k >> (kl.packed ? kl.idbits + kl.vbits : 32);
+      }
+    } else if (r > 0 && c64 < nc) {
+      link[c] = FIN;
+    }
+    const uint32_t rm = __ballot_sync(0xffffffffu, root), am = __ballot_sync(0xffffffffu, act);
+    if (lane == 0) s_tot[wid] = __popc(rm) | (r == 0 ? __popc(am) << 16 : 0);
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + wid / GROUP), "n"(32 * GROUP) : "memory");
+    uint32_t sum = 0, mine = 0;
+#pragma unroll
+    for (int q = 0; q < GROUP; ++q) {
+      const uint32_t t = s_tot[wid / GROUP * GROUP + q];
+      mine += q < wid % GROUP ? t : 0u;
+      sum += t;
+    }
+    if (wid % GROUP == 0 && lane < 2) {
+      const uint32_t n = lane ? sum >> 16 : sum & 0xffffu;
+      s_pos[wid / GROUP * 2 + lane] = n ? (uint32_t)atomicAdd(lane ? &a.st->ca : &a.st->cv[r], (u64)n) : 0u;
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + wid / GROUP), "n"(32 * GROUP) : "memory");
+    if (root) {
+      const uint32_t d = s_pos[wid / GROUP * 2] + (mine & 0xffffu) + __popc(rm & below);
+      link[c] = ROOT | d;
+      if (a.want_parent) rep_next[d] = r == 0 ? c : rep[c];
+    }
+    if (r == 0 && act) a.act[s_pos[wid / GROUP * 2 + 1] + (mine >> 16) + __popc(am & below)] = c;
+  }
+  wsum_add(a.wsum, wacc);
+}
+
 // Pointer jumping (Section 4.2): every vertex that is not a root follows the
 // links to its root and takes the root's next-round id; best[] goes back to
 // INF.  Other threads' progress may be read on the way (an entry is either a
@@ -620,7 +679,7 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
     if (s_nc >= (uint64_t)4 * RB * g.nb)
       hook_phase<HI>(a, kl, r, s_nc, s_off[r], r > 0 || rec0, g.nb, g.bid, sm, s_warp, s_base);
     else
-      hook_phase<1>(a, kl, r, s_nc, s_off[r], r > 0 || rec0, g.nb, g.bid, sm, s_warp, s_base);
+      hook_short(a, kl, r, s_nc, s_off[r], r > 0 || rec0, g.nb, g.bid, sm);
     if (!(ok = g.sync())) break;
     if (threadIdx.x == 0) {  // components left with a root, vertices to jump
       s_nn = __ldca(&a.st->cv[r]);
