@@ -102,9 +102,10 @@ typedef struct {
                                   component (recursive filtering in local preprocessing, Section 6.2);
                                   0 (default, measured faster on GB300): every edge from the first round */
   uint32_t spin_limit;         /* polls of the barrier in the ordered output scan before the wait
-                                  gives up (>= 1; default 2^21, about a second); a wait that runs out
-                                  makes the call return MST_ERR_INTERNAL.  Small values exist to exercise
-                                  that error path */
+                                  gives up (>= 1; default 2^21, about a second), and an eighth of those of
+                                  a barrier between two passes of the one-launch rounds; a wait that runs
+                                  out makes the call return MST_ERR_INTERNAL.  Small values exist to
+                                  exercise that error path */
   uint32_t block_threads;      /* threads per block of the relabel / partition compactions and the hooking
                                   kernel: 128, 256 or 512 (0 = 256) */
   uint32_t items_per_thread;   /* edges (or vertices) per thread of those kernels: 4, 8 or 16 (0 = 8); a

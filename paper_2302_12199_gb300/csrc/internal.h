@@ -18,7 +18,11 @@ enum : uint32_t {
   ERR_TMA = 16u,      // a bulk copy never completed (bounded mbarrier wait ran out); tiles were skipped
   ERR_TABLE = 32u,    // a batched size table is inconsistent (offsets not starting at 0 or decreasing)
   ERR_OVERFLOW = 64u, // a compaction's survivors exceeded its output capacity (nothing past it was written)
+  ERR_BARRIER = 128u, // a grid barrier of the one-launch rounds was not reached in time (bounded wait ran out)
 };
+// Rounds that ended early: parent[] may hold tagged links instead of vertices,
+// so the passes that follow its entries (jump, filter, further rounds) do nothing.
+constexpr uint32_t ERR_ROUNDS = ERR_JUMP | ERR_BARRIER;
 
 // Small per-handle device state.
 constexpr int LVL_MAX = 32;  // recursion levels of a planned Filter-Borůvka
@@ -179,10 +183,11 @@ void launch_hook(const HookArgs &a, uint64_t max_cand, cudaStream_t s);
 // max_steps: parent steps per thread and launch (0: the default of 64).
 // With act == count_dev == nullptr the launch covers every vertex
 // 0..count_host-1 and, given gbits, sets bit v of that bitmap iff v's walk
-// reached the root *groot in this launch (gbits is ignored for lists).
+// reached the root *groot in this launch (gbits is ignored for lists); it does
+// nothing when *err holds ERR_ROUNDS.
 void launch_jump(const uint32_t *act, const u64 *count_dev, uint64_t count_host, uint64_t max_count,
-                 uint32_t *parent, u64 *best, int reset_best, uint32_t *flag, int sms, cudaStream_t s,
-                 uint32_t max_steps = 0, const uint32_t *groot = nullptr, uint32_t *gbits = nullptr);
+                 uint32_t *parent, u64 *best, int reset_best, uint32_t *flag, const uint32_t *err, int sms,
+                 cudaStream_t s, uint32_t max_steps = 0, const uint32_t *groot = nullptr, uint32_t *gbits = nullptr);
 // Sets ERR_VERTEX in *err if some x[i] (i < count) is >= bound.
 void launch_range_check(const uint32_t *x, uint64_t count, uint32_t bound, uint32_t *err, int sms, cudaStream_t s);
 void launch_hash_insert(EdgeList in, uint64_t m, HashSlot *table, uint64_t tmask, uint32_t *err, int sms,
@@ -298,6 +303,7 @@ struct RoundsArgs {
   uint32_t n, max_rounds;
   RoundsState *st;
   uint32_t *err;
+  uint32_t spin_limit;  // polls of a grid barrier before the wait gives up (ERR_BARRIER)
 };
 // States that a solve's start clears; its later launches clear the last again.
 constexpr int ROUNDS_STATES = 8;

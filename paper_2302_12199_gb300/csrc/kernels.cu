@@ -323,6 +323,7 @@ struct Shape {
 // block; the staging buffer (16 bytes per item) is dynamic shared memory.
 template <int MODE, bool VEC, int B, int I>
 __global__ void __launch_bounds__(B, Shape<B, I>::minb(Shape<B, I>::compact_regs)) compact_kernel(CompactArgs a) {
+  if (MODE == CM_FILTER && (__ldcg(a.st.err) & ERR_ROUNDS)) return;  // the labels may be no vertices
   constexpr int T = Shape<B, I>::T;
   extern __shared__ __align__(16) uint32_t s_stage[];  // u, v, w, id: T each
   __shared__ uint32_t s_warp[B / 32 + 1];
@@ -462,6 +463,7 @@ constexpr size_t tma_smem_bytes() { return sizeof(EdgeStage<B * I>) * (TMA_STAGE
 
 template <int MODE, int B, int I>
 __global__ void __launch_bounds__(B, Shape<B, I>::minb(Shape<B, I>::tma_regs)) compact_tma_kernel(CompactArgs a) {
+  if (MODE == CM_FILTER && (__ldcg(a.st.err) & ERR_ROUNDS)) return;  // the labels may be no vertices
   constexpr int T = Shape<B, I>::T;
   extern __shared__ __align__(128) unsigned char smem_dyn[];
   EdgeStage<T> *stage = reinterpret_cast<EdgeStage<T> *>(smem_dyn);  // TMA_STAGES input stages + 1 output stage
@@ -675,6 +677,7 @@ __device__ __forceinline__ void warp_flush(const CompactArgs &a, const typename 
 
 template <int MODE, class WS>
 __global__ void __launch_bounds__(WS::threads, WS::minb) stream_warp_kernel(CompactArgs a) {
+  if (MODE == CM_FILTER && (__ldcg(a.st.err) & ERR_ROUNDS)) return;  // the labels may be no vertices
   static_assert(MODE == CM_FILTER || MODE == CM_HEAVY || MODE == CM_PARTITION,
                 "the warp-streamed pass serves the filter modes and the partition");
   constexpr int I = WS::items, S = WS::stages, O = WS::out, T = WS::tile;
@@ -1066,8 +1069,9 @@ __global__ void __launch_bounds__(BLOCK) jump_kernel(const uint32_t *act, const 
 // roots).  Warps stride over warp-aligned bases and stay converged; with
 // gbits, eight lanes' four marks form one 32-vertex bitmap word.
 __global__ void __launch_bounds__(BLOCK) jump_all_kernel(uint32_t *parent, u64 *best, int reset_best, uint64_t n,
-                                                         uint32_t *flag, uint32_t max_steps, const uint32_t *groot,
-                                                         uint32_t *gbits) {
+                                                         uint32_t *flag, const uint32_t *err, uint32_t max_steps,
+                                                         const uint32_t *groot, uint32_t *gbits) {
+  if (__ldcg(err) & ERR_ROUNDS) return;  // parent may hold entries past n
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t nq = (n + 3) / 4;
   const uint64_t stride = (uint64_t)gridDim.x * BLOCK;
@@ -2720,13 +2724,13 @@ void launch_hook(const HookArgs &a, uint64_t max_cand, cudaStream_t s) {
 }
 
 void launch_jump(const uint32_t *act, const u64 *count_dev, uint64_t count_host, uint64_t max_count,
-                 uint32_t *parent, u64 *best, int reset_best, uint32_t *flag, int sms, cudaStream_t s,
-                 uint32_t max_steps, const uint32_t *groot, uint32_t *gbits) {
+                 uint32_t *parent, u64 *best, int reset_best, uint32_t *flag, const uint32_t *err, int sms,
+                 cudaStream_t s, uint32_t max_steps, const uint32_t *groot, uint32_t *gbits) {
   if (max_count == 0) return;
   if (!act && !count_dev) {  // every vertex 0..count_host-1
     const unsigned g = grid_for(((count_host + 3) / 4 + BLOCK - 1) / BLOCK, sms, 8);
-    jump_all_kernel<<<g, BLOCK, 0, s>>>(parent, best, reset_best, count_host, flag, max_steps ? max_steps : JUMP_STEPS,
-                                        groot, gbits);
+    jump_all_kernel<<<g, BLOCK, 0, s>>>(parent, best, reset_best, count_host, flag, err,
+                                        max_steps ? max_steps : JUMP_STEPS, groot, gbits);
     return;
   }
   const unsigned grid = grid_for((max_count + JUMP_TILE - 1) / JUMP_TILE, sms, 8);

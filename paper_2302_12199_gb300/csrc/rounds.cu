@@ -50,7 +50,6 @@ constexpr uint32_t NO_PAIRS = 0xffffffffu;
 constexpr uint32_t LABS = 4096;
 // A call's last rounds run in one block from this size on.
 constexpr uint64_t SOLO_EDGES = 4096, SOLO_VERTS = 4096;
-constexpr uint32_t BAR_SPINS = 1u << 24;  // polls of the grid barrier before giving up
 
 struct Smem {
   uint32_t out[4][RT];  // a hooking tile's vertices; the relabel's claims
@@ -59,10 +58,15 @@ struct Smem {
 static_assert(PAIRS * sizeof(u64) + LABS <= sizeof(Smem), "pairs and labels fit");
 
 // All blocks of the launch are resident (cooperative launch), so a wait for
-// the others ends; it is bounded all the same.
+// the others ends; it is bounded all the same.  A block that gives up has
+// arrived at that barrier but arrives at no later one, so the others, whose
+// phases only read what was complete at the last barrier they passed, give up
+// at the next.  Whatever of parent[] is unfinished then stays so: the passes
+// queued behind the launch look at the error first (ERR_ROUNDS).
 struct GridSync {
   uint32_t nb, bid;  // blocks that take part, this block's number
   uint32_t *bar, *err;
+  uint32_t limit;    // polls
   uint32_t target;
   bool solo;
   // False when the wait ran out (the error is latched; the kernel ends).
@@ -82,8 +86,8 @@ struct GridSync {
         uint32_t v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
         if ((int32_t)(v - target) >= 0) break;
-        if (++spins >= BAR_SPINS) {
-          atomicOr(err, ERR_JUMP);
+        if (++spins >= limit) {
+          atomicOr(err, ERR_BARRIER);
           bad = 1;
           break;
         }
@@ -650,7 +654,7 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
   // the round's edges, vertices, next round's vertices, vertices to jump, and each round's part of link and rep
   __shared__ uint64_t s_m, s_nc, s_nn, s_cnt, s_off[ROUNDS_MAX + 2];
   __shared__ uint32_t s_np;  // pairs of the next round's components, if the round ends by pairs
-  GridSync g{gridDim.x, blockIdx.x, &a.st->bar, a.err, 0, gridDim.x == 1};
+  GridSync g{gridDim.x, blockIdx.x, &a.st->bar, a.err, a.spin_limit, 0, gridDim.x == 1};
 
   const uint64_t m0 = a.m_dev ? min((uint64_t)*a.m_dev, a.m) : a.m;
   const KeyLayout kl = resolve_layout(a.kl, a.max_w);
@@ -658,7 +662,8 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
     min_edges_phase(a, kl, m0, g.nb, g.bid);
     if (!g.sync()) return;
   }
-  if (*(volatile uint32_t *)a.err & (ERR_VERTEX | ERR_OVERFLOW)) return;  // the same in every block: set before the barrier
+  // an error set before the barrier, or by another block that gave up at it: one answer per block
+  if (__syncthreads_or((int)(*(volatile uint32_t *)a.err & (ERR_VERTEX | ERR_OVERFLOW | ERR_ROUNDS)))) return;
 
   const bool rec0 = a.ends_rec || a.record_first;
   if (threadIdx.x == 0) {

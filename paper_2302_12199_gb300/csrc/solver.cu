@@ -556,7 +556,7 @@ struct Solve {
     const double fixed = count_dev ? 0.0 : (8.0 + (gbits ? 0.125 : 0.0)) * (double)count_host;
     PROF(MST_K_JUMP, fixed, slot, reset_best ? 20.0 : 12.0, -1, 0.0,
          launch_jump(act_list, count_dev, count_host, max_count, parent, best, reset_best, &c->ds->jump_flag,
-                     c->sms, s, c->cfg.jump_steps, groot, gbits));
+                     &c->ds->err, c->sms, s, c->cfg.jump_steps, groot, gbits));
     return MST_OK;
   }
 
@@ -777,6 +777,7 @@ struct Solve {
     ra.max_rounds = (uint32_t)std::min(ROUNDS_MAX, 2 * (ceil_log2(n) + 2));
     ra.st = c->rstate + std::min(c->rounds_used, ROUNDS_STATES - 1);
     ra.err = &c->ds->err;
+    ra.spin_limit = (uint32_t)std::min<uint64_t>(8ULL * c->cfg.spin_limit, 0xffffffffu);
     return ra;
   }
   // boruvka() as one launch; nothing is read back (an error it sets stays
@@ -1314,8 +1315,8 @@ struct Solve {
       launch_giant_root(E[k], caps[k], host_mix64(state[k]), parent, n, &c->ds->giant_root, s, mk,
                         &c->ds->giant_count);
       PROF(MST_K_JUMP, 8.125 * (double)n, -1, 0.0, -1, 0.0,
-           launch_jump(nullptr, nullptr, n, n, parent, best, 0, &c->ds->jump_flag, c->sms, s, 4096,
-                       &c->ds->giant_root, gbits));
+           launch_jump(nullptr, nullptr, n, n, parent, best, 0, &c->ds->jump_flag, &c->ds->err, c->sms, s,
+                       4096, &c->ds->giant_root, gbits));
       CompactArgs cf{};
       cf.shape = shape;
       cf.in = E[k];
