@@ -598,13 +598,14 @@ constexpr int SINGLE_T = 1024;
 
 bool launch_block_single(const BlockArgs &args, uint32_t n, uint32_t m, uint32_t *out_ids, uint32_t *out_count,
                          cudaStream_t s) {
-  static const bool ok = [] {  // set once per process
-    const bool set = cudaFuncSetAttribute(block_single_kernel<SINGLE_T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)BIG_SMEM) == cudaSuccess;
+  static PerDevice set_of;
+  const int set = set_of.get(current_device(), []() -> int {
+    const bool ok = cudaFuncSetAttribute(block_single_kernel<SINGLE_T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)BIG_SMEM) == cudaSuccess;
     cudaGetLastError();
-    return set;
-  }();
-  if (!ok) return false;
+    return ok;
+  });
+  if (!set) return false;
   BlockArgs a = args;
   // room for the vertices' minima in either key size and for labels with minima behind them
   a.smem = (uint32_t)std::min<size_t>(BIG_SMEM, std::max<size_t>((size_t)n * 10 + 64, 16384));
@@ -613,13 +614,16 @@ bool launch_block_single(const BlockArgs &args, uint32_t n, uint32_t m, uint32_t
 }
 
 bool launch_block_batch(const BlockArgs &args, int kind, cudaStream_t s) {
-  static const int blocks[3] = {resident_blocks<1024, 1>(BIG_SMEM), resident_blocks<512, 2>(MID_SMEM),
-                                resident_blocks<256, 4>(SMALL_SMEM)};
+  static PerDevice blocks_of[3];
   constexpr size_t smem[3] = {BIG_SMEM, MID_SMEM, SMALL_SMEM};
-  if (blocks[kind] <= 0) return false;
+  const int blocks = blocks_of[kind].get(current_device(), [&] {
+    return kind == 0 ? resident_blocks<1024, 1>(smem[0])
+                     : kind == 1 ? resident_blocks<512, 2>(smem[1]) : resident_blocks<256, 4>(smem[2]);
+  });
+  if (blocks <= 0) return false;
   BlockArgs a = args;
   a.smem = (uint32_t)smem[kind];
-  const unsigned grid = std::min<unsigned>(a.num, (unsigned)blocks[kind]);
+  const unsigned grid = std::min<unsigned>(a.num, (unsigned)blocks);
   if (grid == 0) return true;
   if (kind == 0)
     block_batch_kernel<1024, 1><<<grid, 1024, smem[0], s>>>(a);

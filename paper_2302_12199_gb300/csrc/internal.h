@@ -4,6 +4,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "per_device.h"
+
 namespace mstgpu {
 
 typedef unsigned long long u64;
@@ -172,6 +174,12 @@ inline uint32_t shape_tile(int shape) {
 // Counters the kernels that choose MSF edges add the chosen weights into, so
 // that the forest's total needs no gather of w at the end.
 constexpr int WSUM_SLOTS = 256;
+
+inline int current_device() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return dev;
+}
 
 // ---- launchers (kernels.cu); all asynchronous on `s` ----
 void launch_compact(CompactMode mode, const CompactArgs &a, uint64_t max_count, cudaStream_t s);

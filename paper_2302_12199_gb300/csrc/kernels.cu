@@ -2570,10 +2570,9 @@ static void launch_compact_shaped(const CompactArgs &a, uint64_t max_count, bool
   constexpr int T = B * I;
   constexpr size_t stage_bytes = 16 * (size_t)T;  // compact_kernel's staging buffer
   constexpr bool tma_fits = tma_smem_bytes<B, I>() <= 200 * 1024;
-  // Set once per process (a function-local static is initialised exactly once,
-  // even when several host threads launch at the same time): prefer shared
-  // memory over L1, allow the staging buffer, size the persistent grid.
-  static const int tma_blocks = []() -> int {
+  // Once per device: prefer shared memory over L1, allow the staging buffer, size the persistent grid.
+  static PerDevice tma_blocks_of;
+  const int tma_blocks = tma_blocks_of.get(current_device(), []() -> int {
     cudaFuncSetAttribute(compact_kernel<MODE, true, B, I>, cudaFuncAttributePreferredSharedMemoryCarveout,
                          cudaSharedmemCarveoutMaxShared);
     cudaFuncSetAttribute(compact_kernel<MODE, true, B, I>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2591,7 +2590,7 @@ static void launch_compact_shaped(const CompactArgs &a, uint64_t max_count, bool
     }
     cudaGetLastError();
     return blocks;
-  }();
+  });
   const uint64_t tiles = (max_count + T - 1) / T;
   if (tiles == 0) return;
   if constexpr (tma_fits) {
@@ -2603,13 +2602,13 @@ static void launch_compact_shaped(const CompactArgs &a, uint64_t max_count, bool
   if (aligned) {
     compact_kernel<MODE, true, B, I><<<(unsigned)tiles, B, stage_bytes, s>>>(a);
   } else {  // unaligned lists: scalar loads in the default shape
-    static const bool carveout_set = [] {  // once per process, as above
+    static PerDevice carveout_of;
+    carveout_of.get(current_device(), []() -> int {
       cudaFuncSetAttribute(compact_kernel<MODE, false, BLOCK, ITEMS>, cudaFuncAttributePreferredSharedMemoryCarveout,
                            cudaSharedmemCarveoutMaxShared);
       cudaGetLastError();
-      return true;
-    }();
-    (void)carveout_set;
+      return 1;
+    });
     compact_kernel<MODE, false, BLOCK, ITEMS><<<(unsigned)((max_count + TILE - 1) / TILE), BLOCK, 16 * TILE, s>>>(a);
   }
 }
@@ -2618,8 +2617,8 @@ static void launch_compact_shaped(const CompactArgs &a, uint64_t max_count, bool
 // launched, the caller uses the block kernels).
 template <int MODE, class WS>
 static bool launch_warp_stream(const CompactArgs &a, uint64_t max_count, cudaStream_t s) {
-  // resident blocks of the pass (0: not available); set once per process
-  static const int blocks = []() -> int {
+  static PerDevice blocks_of;  // resident blocks of the pass (0: not available)
+  const int blocks = blocks_of.get(current_device(), []() -> int {
     int dev = 0, sms = 0, per_sm = 0, b = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -2630,7 +2629,7 @@ static bool launch_warp_stream(const CompactArgs &a, uint64_t max_count, cudaStr
       b = sms * per_sm;
     cudaGetLastError();
     return b;
-  }();
+  });
   if (blocks <= 0) return false;
   const uint64_t wtiles = (max_count + WS::tile - 1) / WS::tile;
   const uint64_t want = (wtiles + WS::warps - 1) / WS::warps;
@@ -2826,9 +2825,10 @@ bool launch_tile_contract(uint32_t n, uint32_t B, uint64_t nlocal, const u64 *cu
                           const uint32_t *b_ends, const uint32_t *b_w, const uint32_t *b_id, uint32_t *parent,
                           uint32_t *bits, EdgeOut rest, u64 *rest_fill, uint32_t *err, cudaStream_t s,
                           int filter_heavy, u64 *wsum) {
-  // set once per process, and only published once the attribute is in place
-  // (another host thread must not launch with the larger size before it is)
-  static const int smem_full = []() -> int {
+  // only published once the attribute is in place (another host thread must
+  // not launch with the larger size before it is)
+  static PerDevice smem_full_of;
+  const int smem_full = smem_full_of.get(current_device(), []() -> int {
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -2836,7 +2836,7 @@ bool launch_tile_contract(uint32_t n, uint32_t B, uint64_t nlocal, const u64 *cu
     cudaFuncSetAttribute(tile_contract_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaGetLastError();
     return bytes;
-  }();
+  });
   const size_t vbytes = (size_t)B * (8 + 8 + 4 + 4 + 4);
   if ((size_t)smem_full <= vbytes) return false;
   const uint32_t ntiles = (uint32_t)(((uint64_t)n + B - 1) / B);

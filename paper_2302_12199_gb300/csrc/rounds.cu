@@ -779,8 +779,8 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
 }  // namespace
 
 bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, bool clear, int sms, cudaStream_t s) {
-  // resident blocks per SM (0: not available); set once per process
-  static const int per_sm = []() -> int {
+  static PerDevice per_sm_of;  // resident blocks per SM (0: not available)
+  const int per_sm = per_sm_of.get(current_device(), []() -> int {
     int b = 0;
     if (cudaFuncSetAttribute(rounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)) !=
             cudaSuccess ||
@@ -788,7 +788,7 @@ bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, bool clear, int sms,
       b = 0;
     cudaGetLastError();
     return b < 2 ? b : 2;
-  }();
+  });
   if (per_sm <= 0 || a.n >= ROOT) return false;
   if (clear && cudaMemsetAsync(a.st, 0, sizeof(RoundsState), s) != cudaSuccess) {
     cudaGetLastError();
