@@ -594,6 +594,16 @@ int resident_blocks(size_t smem) {
 
 constexpr int SINGLE_T = 1024;
 
+// False when the launch was refused (nothing runs; the error is the caller's to act on, not left pending).
+template <class... Args>
+bool launch(void (*kernel)(Args...), unsigned grid, int threads, size_t smem, cudaStream_t s, Args... args) {
+  void *p[] = {&args...};
+  if (cudaLaunchKernel((const void *)kernel, dim3(grid), dim3((unsigned)threads), p, smem, s) == cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
+}
+
 }  // namespace
 
 bool launch_block_single(const BlockArgs &args, uint32_t n, uint32_t m, uint32_t *out_ids, uint32_t *out_count,
@@ -609,11 +619,11 @@ bool launch_block_single(const BlockArgs &args, uint32_t n, uint32_t m, uint32_t
   BlockArgs a = args;
   // room for the vertices' minima in either key size and for labels with minima behind them
   a.smem = (uint32_t)std::min<size_t>(BIG_SMEM, std::max<size_t>((size_t)n * 10 + 64, 16384));
-  block_single_kernel<SINGLE_T><<<1, SINGLE_T, a.smem, s>>>(a, n, m, out_ids, out_count);
-  return true;
+  return launch<BlockArgs>(block_single_kernel<SINGLE_T>, 1, SINGLE_T, a.smem, s, a, n, m, out_ids, out_count);
 }
 
 bool launch_block_batch(const BlockArgs &args, int kind, cudaStream_t s) {
+  if (args.num == 0) return true;
   static PerDevice blocks_of[3];
   constexpr size_t smem[3] = {BIG_SMEM, MID_SMEM, SMALL_SMEM};
   const int blocks = blocks_of[kind].get(current_device(), [&] {
@@ -624,14 +634,9 @@ bool launch_block_batch(const BlockArgs &args, int kind, cudaStream_t s) {
   BlockArgs a = args;
   a.smem = (uint32_t)smem[kind];
   const unsigned grid = std::min<unsigned>(a.num, (unsigned)blocks);
-  if (grid == 0) return true;
-  if (kind == 0)
-    block_batch_kernel<1024, 1><<<grid, 1024, smem[0], s>>>(a);
-  else if (kind == 1)
-    block_batch_kernel<512, 2><<<grid, 512, smem[1], s>>>(a);
-  else
-    block_batch_kernel<256, 4><<<grid, 256, smem[2], s>>>(a);
-  return true;
+  if (kind == 0) return launch<BlockArgs>(block_batch_kernel<1024, 1>, grid, 1024, smem[0], s, a);
+  if (kind == 1) return launch<BlockArgs>(block_batch_kernel<512, 2>, grid, 512, smem[1], s, a);
+  return launch<BlockArgs>(block_batch_kernel<256, 4>, grid, 256, smem[2], s, a);
 }
 
 }  // namespace mstgpu

@@ -344,9 +344,11 @@ struct BlockArgs {
   uint32_t smem;               // set by the launchers
   Readback rb;                 // at the end of launch_block_single
 };
-// kind: 0 the large graphs, 1 the middle ones, 2 the small ones.
+// kind: 0 the large graphs, 1 the middle ones, 2 the small ones.  False if the
+// launch was refused (nothing ran).
 bool launch_block_batch(const BlockArgs &a, int kind, cudaStream_t s);
 // The one graph (n, m) of the arrays; clears *err, bits and writes the forest.
+// False as above.
 bool launch_block_single(const BlockArgs &a, uint32_t n, uint32_t m, uint32_t *out_ids, uint32_t *out_count,
                          cudaStream_t s);
 

@@ -2273,9 +2273,10 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
     a.solved = solved;
     a.err = &h->ds->err;
     mst_ctx *c = h;
-    bool ok = true;
+    bool ok = true, ran = true;
     // The three kinds run side by side: a kind's last blocks leave SMs idle
-    // that the next kind's fill.
+    // that the next kind's fill.  The graphs of a kind whose launch is refused
+    // stay unsolved and go to the union below.
     const bool fork = kinds[0] + kinds[1] + kinds[2] >= (uint64_t)h->sms;
     if (fork && !h->kind_ev[2]) {
       for (int k = 0; k < 2; ++k)
@@ -2293,7 +2294,7 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
       const bool own = fork && kind > 0 && a.num > 0;
       cudaStream_t ks = own ? h->kind_stream[kind - 1] : s;
       if (own) ok = ok && cudaStreamWaitEvent(ks, h->kind_ev[2], 0) == cudaSuccess;
-      ok = ok && launch_block_batch(a, kind, ks);
+      if (ok) ran = launch_block_batch(a, kind, ks) && ran;
       if (own)  // s goes on after every kind, also after an error
         ok = cudaEventRecord(h->kind_ev[kind - 1], ks) == cudaSuccess &&
              cudaStreamWaitEvent(s, h->kind_ev[kind - 1], 0) == cudaSuccess && ok;
@@ -2301,7 +2302,7 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
     }
     prof_end(c, s, p, MST_K_BASE, 12.0 * (double)mblk);
     if (!ok) return record_cuda(h, __LINE__);
-    if (mblk == m) {  // every graph: straight to the output
+    if (ran && mblk == m) {  // every graph: straight to the output
       ++h->solves;
       batch_msf_off_kernel<<<1, TAB_THREADS, 0, s>>>(sizes, num_graphs, d_msf_off);
       batch_emit_kernel<<<(unsigned)std::min<uint64_t>(num_graphs, (uint64_t)h->sms * 4), EMIT_THREADS, 0, s>>>(
