@@ -601,6 +601,7 @@ struct Solve {
       bool ran = false;
       TRY(boruvka_device(E, mE, validate, best_ready, ends_rec, ran));
       if (ran) return MST_OK;
+      refuse_rounds();
     }
     if (!act[1]) {
       TRY(act_b[1].alloc(c, (size_t)n * 4, s));
@@ -754,8 +755,14 @@ struct Solve {
   // The rounds of a call run in one cooperative launch (rounds.cu) unless an
   // option needs the host between them.
   static constexpr uint64_t MIN_EDGES_KERNEL = 1ULL << 20;
+  bool rounds_refused = false;  // the launch was refused: the host drives this solve's rounds
+  void refuse_rounds() {
+    rounds_refused = true;
+    link_b.release();
+    link = reps = nullptr;
+  }
   bool device_rounds() const {
-    return c->cfg.graph_rounds && c->cfg.dedupe != MST_DEDUPE_HASH && c->cfg.dedupe != MST_DEDUPE_SORT;
+    return !rounds_refused && c->cfg.graph_rounds && c->cfg.dedupe != MST_DEDUPE_HASH && c->cfg.dedupe != MST_DEDUPE_SORT;
   }
   RoundsArgs rounds_args(RoundList &X, RoundList &Y) {
     RoundsArgs ra{};
@@ -1177,8 +1184,8 @@ struct Solve {
   // Borůvka rounds on the list in round list X whose length is count[slot]
   // (best[] holds its minEdges; ends_rec: its ends were recorded by id as it
   // was written), in one launch.  last: nothing reads the representatives
-  // afterwards.
-  mst_status boruvka_planned(RoundList &X, RoundList &Y, int slot, bool ends_rec, bool last) {
+  // afterwards.  ran: false when it was not launched.
+  mst_status boruvka_planned(RoundList &X, RoundList &Y, int slot, bool ends_rec, bool last, bool &ran) {
     RoundsArgs ra = rounds_args(X, Y);
     ra.in = X.list();
     ra.m = std::min(X.cap, Y.cap);
@@ -1187,10 +1194,8 @@ struct Solve {
     ra.best_ready = 1;
     ra.want_parent = last ? 0 : 1;
     ra.ends_rec = (ends_rec && cur_u) ? 1 : 0;
-    bool ran = false;
     PROF(MST_K_GRAPH, 0.0, -1, 0.0, -1, 0.0, ran = launch_rounds(ra, ra.m, c->rounds_used++ >= ROUNDS_STATES, c->sms, s));
-    if (!ran) return MST_ERR_CUDA;
-    ++rounds;
+    if (ran) ++rounds;
     return MST_OK;
   }
 
@@ -1299,13 +1304,18 @@ struct Solve {
                  ProfTerm{CNT_LVL + k, 16.0, 16.0}, ProfTerm{CNT_LVL + k + 1, 16.0, 16.0});
       E[k + 1] = last ? X.list() : Lb[k + 1].list();
     }
-    if (K == 1 && !leaf_top) {
-      bool ran = false;
+    // a refused launch ends the plan: the caller starts over, with the host driving the rounds
+    const auto refused = [&] {
+      refuse_rounds();
+      planned = false;
+      return MST_OK;
+    };
+    bool ran = false;
+    if (K == 1 && !leaf_top)
       TRY(boruvka_device(E[1], m1, false, false, false, ran));
-      if (!ran) return MST_ERR_CUDA;
-    } else {
-      TRY(boruvka_planned(X, Y, CNT_LVL + K, cur_u != nullptr, false));
-    }
+    else
+      TRY(boruvka_planned(X, Y, CNT_LVL + K, cur_u != nullptr, false, ran));
+    if (!ran) return refused();
 
     // levels K-1 .. 0: contract P and mark the giant component, filter the
     // level's heavy edges into X, and solve them
@@ -1340,7 +1350,8 @@ struct Solve {
       PROF_TERMS(MST_K_FILTER, fixed, fixed, launch_compact(CM_FILTER, cf, caps[k], s),
                  ProfTerm{k == 0 ? -1 : CNT_LVL + k, per, per}, ProfTerm{CNT_LVL + k + 1, 0.0, -per},
                  ProfTerm{CNT_LVL + LVL_MAX + k, 16.0, 16.0});
-      TRY(boruvka_planned(X, Y, CNT_LVL + LVL_MAX + k, cur_u != nullptr, k == 0));
+      TRY(boruvka_planned(X, Y, CNT_LVL + LVL_MAX + k, cur_u != nullptr, k == 0, ran));
+      if (!ran) return refused();
     }
     return MST_OK;
   }

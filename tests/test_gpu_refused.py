@@ -108,3 +108,26 @@ def test_refused_block_launch_in_a_batch(lib, monkeypatch, name, copies):
     finally:
         lib.refuse(None)
         s.close()
+
+
+# plain rounds, and Filter-Borůvka planned with light lists on either side of the sparsity bound, several levels deep,
+# with packed and unpacked keys
+@pytest.mark.parametrize("cfg", [dict(), dict(variant="filter"), dict(variant="filter", filter_max_avg_degree=4.0),
+                                 dict(variant="filter", pivot_quantile=0.5), dict(variant="filter", filter_plan=0)])
+@pytest.mark.parametrize("wmax", [255, 0xFFFFFFFF])
+def test_refused_rounds(lib, monkeypatch, cfg, wmax):
+    monkeypatch.setattr(mst, "_lib", lib)
+    g = W.gnm(1 << 14, 1 << 18, 9)
+    w = np.random.default_rng(4).integers(1, wmax, g.m, endpoint=True).astype(np.uint32)
+    kid, ktot = oracle.kruskal(g.n, g.src, g.dst, w)
+    t = to_dev(W.Graph(g.n, g.src, g.dst, w))
+    s = mst.Solver(0, filter_min_edges=1 << 10, pivot_sample=1 << 12, **cfg)
+    try:
+        for name in (b"rounds_kernel", None, b"rounds_kernel"):
+            lib.refuse(name)
+            ids, tot = s.solve(g.n, *t).to_host()
+            assert np.array_equal(ids, kid) and tot == ktot
+            assert (lib.refused() > 0) == (name is not None)
+    finally:
+        lib.refuse(None)
+        s.close()
