@@ -50,6 +50,7 @@ constexpr uint32_t NO_PAIRS = 0xffffffffu;
 constexpr uint32_t LABS = 4096;
 // A call's last rounds run in one block from this size on.
 constexpr uint64_t SOLO_EDGES = 4096, SOLO_VERTS = 4096;
+constexpr uint32_t BAR_SPINS = 1u << 24;  // polls of the grid barrier before giving up, by default
 
 struct Smem {
   uint32_t out[4][RT];  // a hooking tile's vertices; the relabel's claims
@@ -63,6 +64,10 @@ static_assert(PAIRS * sizeof(u64) + LABS <= sizeof(Smem), "pairs and labels fit"
 // phases only read what was complete at the last barrier they passed, give up
 // at the next.  Whatever of parent[] is unfinished then stays so: the passes
 // queued behind the launch look at the error first (ERR_ROUNDS).
+// FIXED: the limit is BAR_SPINS.  A limit read at run time changes the long
+// phases' registers (RMAT n=2^22 m=2^26, plain: 2719 -> 2737 us; RGG2D n=2^22
+// 903 -> 910), so it has an instance of its own.
+template <bool FIXED>
 struct GridSync {
   uint32_t nb, bid;  // blocks that take part, this block's number
   uint32_t *bar, *err;
@@ -86,7 +91,7 @@ struct GridSync {
         uint32_t v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
         if ((int32_t)(v - target) >= 0) break;
-        if (++spins >= limit) {
+        if (++spins >= (FIXED ? BAR_SPINS : limit)) {
           atomicOr(err, ERR_BARRIER);
           bad = 1;
           break;
@@ -647,6 +652,7 @@ __device__ __forceinline__ void compose_phase(const RoundsArgs &a, const uint64_
   }
 }
 
+template <bool FIXED>
 __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ RoundsArgs a) {
   extern __shared__ __align__(128) unsigned char smem_dyn[];
   Smem &sm = *reinterpret_cast<Smem *>(smem_dyn);
@@ -654,7 +660,7 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
   // the round's edges, vertices, next round's vertices, vertices to jump, and each round's part of link and rep
   __shared__ uint64_t s_m, s_nc, s_nn, s_cnt, s_off[ROUNDS_MAX + 2];
   __shared__ uint32_t s_np;  // pairs of the next round's components, if the round ends by pairs
-  GridSync g{gridDim.x, blockIdx.x, &a.st->bar, a.err, a.spin_limit, 0, gridDim.x == 1};
+  GridSync<FIXED> g{gridDim.x, blockIdx.x, &a.st->bar, a.err, a.spin_limit, 0, gridDim.x == 1};
 
   const uint64_t m0 = a.m_dev ? min((uint64_t)*a.m_dev, a.m) : a.m;
   const KeyLayout kl = resolve_layout(a.kl, a.max_w);
@@ -776,15 +782,14 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
   compose_phase(a, s_off, r);
 }
 
-}  // namespace
-
-bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, bool clear, int sms, cudaStream_t s) {
+template <bool FIXED>
+bool launch(const RoundsArgs &a, uint64_t max_edges, bool clear, int sms, cudaStream_t s) {
   static PerDevice per_sm_of;  // resident blocks per SM (0: not available)
   const int per_sm = per_sm_of.get(current_device(), []() -> int {
     int b = 0;
-    if (cudaFuncSetAttribute(rounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)) !=
+    if (cudaFuncSetAttribute(rounds_kernel<FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)) !=
             cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, rounds_kernel, RB, sizeof(Smem)) != cudaSuccess)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, rounds_kernel<FIXED>, RB, sizeof(Smem)) != cudaSuccess)
       b = 0;
     cudaGetLastError();
     return b < 2 ? b : 2;
@@ -801,11 +806,18 @@ bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, bool clear, int sms,
   if (max_edges <= SOLO_EDGES && a.n <= SOLO_VERTS) grid = 1;
   RoundsArgs arg = a;
   void *args[] = {&arg};
-  if (cudaLaunchCooperativeKernel((const void *)rounds_kernel, dim3(grid), dim3(RB), args, sizeof(Smem), s) ==
+  if (cudaLaunchCooperativeKernel((const void *)rounds_kernel<FIXED>, dim3(grid), dim3(RB), args, sizeof(Smem), s) ==
       cudaSuccess)
     return true;
   cudaGetLastError();
   return false;
+}
+
+}  // namespace
+
+bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, bool clear, int sms, cudaStream_t s) {
+  return a.spin_limit == BAR_SPINS ? launch<true>(a, max_edges, clear, sms, s)
+                                   : launch<false>(a, max_edges, clear, sms, s);
 }
 
 }  // namespace mstgpu
