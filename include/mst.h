@@ -82,7 +82,7 @@ typedef struct {
                                   that the device ends (no host round trip per round; not with hash or
                                   sort dedupe, nor for n >= 2^31); 0: one host readback per round */
   int graph_jump_launches;     /* 1..8 (default 2); kept for callers that set it, without effect: the
-                                  one-launch rounds repeat their jump passes of 256 parent steps on the
+                                  one-launch rounds repeat their jump passes of 32 parent steps on the
                                   device until every vertex has its root */
   int filter_carry;            /* Filter-Borůvka: 1 hands a level's filtered heavy edges, when at most
                                   n/8, back to the level above instead of solving them there (Section
