@@ -296,7 +296,7 @@ struct RoundsArgs {
   int validate;         // check u, v < n in the first pass (without best_ready)
   KeyLayout kl;         // with max_w only its bit widths count
   const uint32_t *max_w;  // largest weight in device memory: packs the keys when they fit; or nullptr
-  u64 *best;            // [n] all KEY_INF but for a ready first round; all KEY_INF again afterwards
+  u64 *best;            // [n] all KEY_INF but for a ready first round; with want_parent all KEY_INF again afterwards
   uint32_t *parent;     // [n] representatives; the call's vertices are updated if want_parent
   uint32_t *link;       // [n] links of the rounds after the first
   uint32_t *rep;        // [n] representatives of their components (want_parent)

@@ -708,7 +708,10 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
       s_np = s_nn <= PAIR_COMPS && s_m > SOLO_EDGES && s_m >= (uint64_t)4 * np ? np : NO_PAIRS;
     }
     __syncthreads();
-    if (s_nn == 0) {  // no vertex had an edge
+    // no vertex had an edge; or all are in one component, so no edge between
+    // components is left (a star of 2^20 vertices and 2^23 edges read its edges
+    // once more for nothing: 574 -> 532 us)
+    if (s_nn == 0 || (s_nn == 1 && !a.want_parent)) {
       ++r;
       break;
     }
@@ -726,6 +729,10 @@ __global__ void __launch_bounds__(RB, 2) rounds_kernel(const __grid_constant__ R
     }
     ++pass;
     if (!ok) break;
+    if (s_nn == 1) {
+      ++r;
+      break;
+    }
     if (s_np != NO_PAIRS) {
       const EdgeOut out = a.list[(a.first_slot + r) & 1], prev = a.list[(a.first_slot + r + 1) & 1];
       const EdgeList in = r == 0 ? a.in : EdgeList{prev.u, prev.v, prev.w, prev.id};
