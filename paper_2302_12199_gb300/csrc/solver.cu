@@ -2237,6 +2237,8 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
   const uint64_t n_total = h->hs->count[CNT_AUX], m = h->hs->count[CNT_AUX + 1];
   if (n_total >= (1ULL << 32) || m >= (1ULL << 32)) return record(h, MST_ERR_TOO_LARGE);
   if (m > 0 && (!d_src || !d_dst || !d_w || !d_msf_ids)) return record(h, MST_ERR_INVALID_ARG);
+  if (!aligned4(d_w) || (m > 0 && (!aligned4(d_src) || !aligned4(d_dst) || !aligned4(d_msf_ids))))
+    return record(h, MST_ERR_INVALID_ARG);
   const uint32_t n = (uint32_t)n_total;
   const uint64_t cap = m < (uint64_t)n ? m : (uint64_t)n, words = (m + 31) / 32;
   // the forest's union ids, then (256-byte aligned) its size, then 256 bytes on, its weight
