@@ -503,8 +503,7 @@ __device__ __forceinline__ void solve_graph(const BlockArgs &a, Work g, Shared<T
   g.wlo = min(end, (threadIdx.x >> 5) * part);
   g.whi = min(end, g.wlo + part);
   g.base = g.wlo > g.skip ? g.wlo - g.skip : 0u;
-  const uint32_t pb = g.m > 1 ? 32 - __clz(g.m - 1) : 1;
-  const uint32_t wlim = (1u << (31 - pb)) - 1u;  // larger weights need 64-bit keys
+  const uint32_t pb = block_pos_bits(g.m), wlim = block_weight_limit(g.m);
   // the pivot: about 1.5 n light edges, from one sampled weight per thread
   const uint64_t j = g.off + __umul64hi(splitmix64_at(0x5eedULL + g.off, threadIdx.x), (u64)g.m);
   const uint32_t sw = __ldg(a.w + j);
@@ -577,7 +576,7 @@ __global__ void __launch_bounds__(T, 1) block_single_kernel(const __grid_constan
   publish_state(a.rb);
 }
 
-constexpr size_t BIG_SMEM = 224 * 1024, MID_SMEM = BLOCK_MID_N * 4, SMALL_SMEM = BLOCK_SMALL_N * 4;
+constexpr size_t BIG_SMEM = BLOCK_BIG_N * 4, MID_SMEM = BLOCK_MID_N * 4, SMALL_SMEM = BLOCK_SMALL_N * 4;
 
 template <int T, int MINB>
 int resident_blocks(size_t smem) {

@@ -27,6 +27,11 @@ __device__ __forceinline__ bool same_edge(const KeyLayout &kl, u64 a, u64 b) {
   return kl.packed ? (a >> kl.vbits) == (b >> kl.vbits) : a == b;
 }
 
+// Block solves: bits of a position among a graph's m edges (m > 0), and the
+// weights from which on its keys take 64 bits.
+__device__ __forceinline__ uint32_t block_pos_bits(uint32_t m) { return m > 1 ? 32 - __clz(m - 1) : 1; }
+__device__ __forceinline__ uint32_t block_weight_limit(uint32_t m) { return (1u << (31 - block_pos_bits(m))) - 1u; }
+
 __device__ __forceinline__ u64 mix64(u64 z) {  // splitmix64 finaliser
   z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
   z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;

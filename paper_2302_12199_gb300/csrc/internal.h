@@ -323,8 +323,9 @@ bool launch_rounds(const RoundsArgs &a, uint64_t max_edges, bool clear, int sms,
 constexpr uint32_t BLOCK_MAX_N = 65536;   // 16-bit labels
 constexpr uint64_t BLOCK_MAX_M = 1ULL << 22;
 // Vertices up to which a graph runs in a block of 256 threads (four per SM),
-// and of 512 (two per SM): their minima fill the blocks' shared memory.
-constexpr uint32_t BLOCK_SMALL_N = 12288, BLOCK_MID_N = 28416;
+// and of 512 (two per SM): their minima fill the blocks' shared memory, as those
+// of BLOCK_BIG_N vertices fill a whole SM's.
+constexpr uint32_t BLOCK_SMALL_N = 12288, BLOCK_MID_N = 28416, BLOCK_BIG_N = 57344;
 struct BlockArgs {
   const uint32_t *gn;          // vertices per graph
   const uint64_t *edge_off, *vert_off;

@@ -1548,7 +1548,7 @@ __device__ __forceinline__ uint32_t batch_graph_of(const uint64_t *off, uint32_t
 // totals[1] = edge_off[G] (all edges); ERR_TABLE if edge_off[0] != 0 or the
 // offsets decrease somewhere.
 constexpr int TAB_THREADS = 1024;
-// A block solves a graph of this many edges whatever the batch: about 0.2 ms.
+// Edges of a graph that a block may solve however many graphs there are.
 constexpr uint64_t BLOCK_MIN_LIMIT = 1ULL << 17;
 __global__ void __launch_bounds__(TAB_THREADS) batch_tables_kernel(const uint32_t *gn, const uint64_t *edge_off,
                                                                   uint32_t G, uint64_t *vert_off, u64 *totals,
@@ -1599,40 +1599,96 @@ __global__ void __launch_bounds__(TAB_THREADS) batch_tables_kernel(const uint32_
   }
 }
 
+// What a block's time grows with, about 2 ns a unit (n vertices, m edges):
+// measured alone, 58 us with n=2048 m=8192, 167 with 8192/32768, 269 with
+// 12288/65536; the larger kinds have two and four times the threads (176 us with
+// 16384/32768, 302 with 32768/131072), up to the vertices whose 32-bit minima no
+// longer fit (915 us with 65536/131072).  Wide weights take 64-bit minima, which
+// fit half as many vertices and then go over the edges in ranges (299, 372 and
+// 584 us in place of 167, 176 and 302).
+__device__ __forceinline__ u64 block_cost(uint32_t n, uint64_t m, int kind, bool wide) {
+  const u64 c = 6ULL * n + m;
+  const uint32_t room = kind == 2 ? BLOCK_SMALL_N : kind == 1 ? BLOCK_MID_N : BLOCK_BIG_N;
+  const u64 t = n > room ? c : kind == 2 ? c : kind == 1 ? c - c / 4 : c / 2;
+  return wide && n > room / 2 ? 2 * t : t;
+}
+// The same units for the union of M edges and N vertices, beyond what it takes
+// with few (UNION_BASE).  The constants lose least over 138 measured batches of 1
+// to 608 graphs of 512 to 65536 vertices, with weights of 8 and of 32 bits: none
+// is slower than the union alone was before there were blocks, five take more
+// than 10% longer than the other choice would (28% at most).
+__host__ __device__ inline u64 union_cost(uint64_t M, uint64_t N) { return M / 32 + N / 24; }
+constexpr u64 UNION_BASE = 1ULL << 15;
+
 // Which graphs of a batch one block each solves, and in which order: those
 // with at most BLOCK_MAX_N vertices and at most mlim edges (no block should
-// run much longer than the batch's share per SM), the large ones first, then
+// run much longer than the batch's share per SM) that a block solves no later
+// than the union of the whole batch would be, the large ones first, then
 // the middle and the small ones, each kind by falling size (half powers of
-// two).  counts: their three numbers and their edges.
+// two).  One graph of 65536 vertices and 131072 edges takes a block 1086 us and
+// the union 259, 152 of them 1682 and 2055; one of 8192 and 32768 takes 288 and
+// 206, 64 of them 301 and 448.  totals: the batch's vertices and edges.  Weights
+// (w, if the arrays are known to be what the tables say) are sampled for their
+// width only; `bucket_of` is scratch.  counts: the numbers of the three kinds,
+// their edges, their vertices and the largest block_cost among them.
 __global__ void __launch_bounds__(TAB_THREADS) batch_order_kernel(const uint32_t *gn, const uint64_t *edge_off,
                                                                   uint32_t G, uint64_t mlim, int sms,
+                                                                  const uint32_t *w, const u64 *totals,
+                                                                  const uint32_t *err, uint32_t *bucket_of,
                                                                   uint32_t *order, u64 *counts) {
   constexpr int BUCKETS = 64;
+  constexpr uint32_t NONE = 0xffffffffu;
   __shared__ uint32_t s_n[3 * BUCKETS];
-  __shared__ u64 s_edges;
-  const uint64_t lim = max(mlim, (uint64_t)edge_off[G] / (uint64_t)sms);
+  __shared__ u64 s_edges, s_verts, s_cost;
+  const uint64_t M = totals[1], N = totals[0];
+  const uint64_t lim = max(mlim, M / (uint64_t)sms);
+  const u64 cost_lim = UNION_BASE + union_cost(M, N);
+  if ((*err & ERR_TABLE) || M >= (1ULL << 32) || N >= (1ULL << 32)) w = nullptr;  // the call ends with an error
   if (threadIdx.x < 3 * BUCKETS) s_n[threadIdx.x] = 0;
-  if (threadIdx.x == 0) s_edges = 0;
+  if (threadIdx.x == 0) s_edges = s_verts = s_cost = 0;
   __syncthreads();
-  auto bucket = [&](uint32_t g) -> int {
-    const uint64_t m = edge_off[g + 1] - edge_off[g];
+  u64 edges = 0, verts = 0, cost = 0;
+  for (uint32_t g = threadIdx.x; g < G; g += TAB_THREADS) {
+    const uint64_t off = edge_off[g], m = edge_off[g + 1] - off;
     const uint32_t n = gn[g];
-    if (m > 0 && (n > BLOCK_MAX_N || m > lim || m > BLOCK_MAX_M)) return -1;
+    const int kind = m == 0 || n <= BLOCK_SMALL_N ? 2 : n <= BLOCK_MID_N ? 1 : 0;
+    u64 c = 0;
+    bool fits = m == 0 || (n <= BLOCK_MAX_N && m <= lim && m <= BLOCK_MAX_M);
+    if (fits && m) {
+      bool wide = false;
+      if (w) {
+        const uint32_t wlim = block_weight_limit((uint32_t)m);
+        uint32_t x[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = __ldg(w + off + __umul64hi(splitmix64_at(off, k), m));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) wide |= x[k] >= wlim;
+      }
+      c = block_cost(n, m, kind, wide);
+      fits = c <= cost_lim;
+    }
+    bucket_of[g] = NONE;
+    if (!fits) continue;
     const int lg = 63 - __clzll((long long)(m | 1));
     const int half = lg > 0 ? (int)(m >> (lg - 1) & 1) : 0;
-    const int kind = m == 0 || n <= BLOCK_SMALL_N ? 2 : n <= BLOCK_MID_N ? 1 : 0;
-    return kind * BUCKETS + BUCKETS - 1 - (2 * lg + half);
-  };
-  u64 edges = 0;
-  for (uint32_t g = threadIdx.x; g < G; g += TAB_THREADS) {
-    const int b = bucket(g);
-    if (b < 0) continue;
+    const uint32_t b = (uint32_t)(kind * BUCKETS + BUCKETS - 1 - (2 * lg + half));
+    bucket_of[g] = b;
     atomicAdd(&s_n[b], 1u);
-    edges += edge_off[g + 1] - edge_off[g];
+    edges += m;
+    verts += n;
+    cost = max(cost, c);
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) edges += __shfl_xor_sync(0xffffffffu, edges, o);
-  if ((threadIdx.x & 31) == 0 && edges) atomicAdd(&s_edges, edges);
+  for (int o = 16; o > 0; o >>= 1) {
+    edges += __shfl_xor_sync(0xffffffffu, edges, o);
+    verts += __shfl_xor_sync(0xffffffffu, verts, o);
+    cost = max(cost, __shfl_xor_sync(0xffffffffu, cost, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&s_edges, edges);
+    atomicAdd(&s_verts, verts);
+    atomicMax(&s_cost, cost);
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     uint32_t sum = 0;
@@ -1646,11 +1702,13 @@ __global__ void __launch_bounds__(TAB_THREADS) batch_order_kernel(const uint32_t
       counts[kind] = sum - before;
     }
     counts[3] = s_edges;
+    counts[4] = s_verts;
+    counts[5] = s_cost;
   }
   __syncthreads();
   for (uint32_t g = threadIdx.x; g < G; g += TAB_THREADS) {
-    const int b = bucket(g);
-    if (b >= 0) order[atomicAdd(&s_n[b], 1u)] = g;
+    const uint32_t b = bucket_of[g];
+    if (b != NONE) order[atomicAdd(&s_n[b], 1u)] = g;
   }
 }
 
@@ -2229,8 +2287,10 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
     solved = sizes + num_graphs;
     queue = solved + num_graphs;
     if (cudaMemsetAsync(solved, 0, ((size_t)num_graphs + 4) * 4, s) != cudaSuccess) return record_cuda(h, __LINE__);
-    batch_order_kernel<<<1, TAB_THREADS, 0, s>>>(d_n, d_edge_off, num_graphs, BLOCK_MIN_LIMIT, h->sms, order,
-                                                          &h->ds->count[CNT_LVL]);
+    batch_order_kernel<<<1, TAB_THREADS, 0, s>>>(
+        d_n, d_edge_off, num_graphs, BLOCK_MIN_LIMIT, h->sms,
+        d_src && d_dst && d_msf_ids && aligned4(d_w) ? d_w : nullptr, &h->ds->count[CNT_AUX], &h->ds->err, sizes, order,
+        &h->ds->count[CNT_LVL]);
   }
   st = readback(h, s);
   if (st != MST_OK) return record(h, st);
@@ -2256,10 +2316,12 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
 
   // Graphs that fit a block each, when they hold at least half of the edges
   // (below that the union passes below dominate, and a block per graph only
-  // adds its own time in front of them).
+  // adds its own time in front of them) and, where others are left for the
+  // union, save it more than the longest of them takes.
   const u64 *kinds = &h->hs->count[CNT_LVL];
   const uint64_t mblk = h->hs->count[CNT_LVL + 3];
-  const bool use_blocks = blocks && m > 0 && 2 * mblk >= m;
+  const bool use_blocks = blocks && m > 0 && 2 * mblk >= m &&
+                          (mblk == m || kinds[5] <= union_cost(mblk, kinds[4]));
   if (use_blocks) {
     Buf scr_b;
     const uint64_t ent_bytes = round_up(m * sizeof(uint4), 256), live_bytes = round_up(m * sizeof(uint2), 256);
