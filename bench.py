@@ -689,17 +689,25 @@ def measure_batched(args, rank: int, world: int, local_rank: int, dev, dist, com
     # grown), not a handle's first solves
     trial_solver = {}
 
+    ran = {}  # kernel classes that a configuration's first trial launched
+
     def trial(cfg):
         key = label(cfg)
         if key not in trial_solver:
             for k in list(trial_solver):
                 trial_solver.pop(k).close()
-            trial_solver[key] = Solver(local_rank, **cfg)
+            s = trial_solver[key] = Solver(local_rank, **cfg)
+            s.profile(True, classes=[])
+            t = timed_batch(s)[0]
+            s.profile(False)
+            ran[key] = {k for k, v in s.profile_stats().items() if v[0]}
+            return t
         return timed_batch(trial_solver[key])[0]
     if args.no_autotune:
         best, tuning = dict(variant="boruvka", dedupe="none", tile_contract=0), []
     else:
-        best, tuning = autotune(trial, reps=3, relabel_shapes=RELABEL_SHAPE_CANDIDATES)
+        best, tuning = autotune(trial, reps=3, relabel_shapes=RELABEL_SHAPE_CANDIDATES,
+                                launched=lambda cfg: ran[label(cfg)])
     for k in list(trial_solver):
         trial_solver.pop(k).close()
     if args.base_case is not None:

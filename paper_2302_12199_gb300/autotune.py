@@ -13,7 +13,7 @@ Host logic only: each trial is one call into the CUDA library.
 """
 from __future__ import annotations
 
-from typing import Callable, Dict, Iterable, List, Tuple
+from typing import Callable, Container, Dict, Iterable, List, Tuple
 
 # Candidate configurations (keyword arguments of mst.Solver).
 DEFAULT_CANDIDATES: Tuple[dict, ...] = (
@@ -45,6 +45,13 @@ RELABEL_SHAPE_CANDIDATES: Tuple[dict, ...] = tuple(dict(relabel_block_threads=b,
 _DEFAULTS = dict(block_threads=256, items_per_thread=8, relabel_block_threads=128, relabel_items_per_thread=4,
                  pivot_quantile=0.125)
 
+# Kernel classes (mst.KERNEL_CLASSES) whose launches read an option of the
+# later stages.  One-launch rounds and one-block solves read none of them.
+READ_BY: Dict[str, Tuple[str, ...]] = dict(
+    pivot_quantile=("pivot",), block_threads=("partition", "hook", "dedupe"),
+    items_per_thread=("partition", "hook", "dedupe"), relabel_block_threads=("relabel_min", "dedupe"),
+    relabel_items_per_thread=("relabel_min", "dedupe"))
+
 _cache: Dict[str, dict] = {}
 
 
@@ -56,7 +63,8 @@ def autotune(trial: Callable[[dict], float], candidates: Iterable[dict] = DEFAUL
              key: str | None = None,
              shapes: Iterable[dict] | None = SHAPE_CANDIDATES,
              relabel_shapes: Iterable[dict] | None = None,
-             quantiles: Iterable[dict] | None = QUANTILE_CANDIDATES) -> Tuple[dict, List[Tuple[str, float]]]:
+             quantiles: Iterable[dict] | None = QUANTILE_CANDIDATES,
+             launched: Callable[[dict], Container[str]] | None = None) -> Tuple[dict, List[Tuple[str, float]]]:
     """Returns (best configuration, [(label, best seconds)] for every trial).
 
     trial(cfg) runs one solve of the workload with configuration cfg and
@@ -67,7 +75,9 @@ def autotune(trial: Callable[[dict], float], candidates: Iterable[dict] = DEFAUL
     empty: none) on top of it; then each of `shapes` (kernel tile shapes) on
     top of the best so far; then each of `relabel_shapes` (e.g.
     RELABEL_SHAPE_CANDIDATES).  Settings equal to what the configuration
-    already runs are skipped.  With `key`, the choice is remembered for the
+    already runs are skipped, and so are those that it does not read, where
+    `launched` says which kernel classes (mst.KERNEL_CLASSES) a trial of a
+    configuration launched: their trials would only differ by noise.  With `key`, the choice is remembered for the
     process and later calls with the same key return it without trials."""
     if key is not None and key in _cache:
         return dict(_cache[key]), []
@@ -93,6 +103,8 @@ def autotune(trial: Callable[[dict], float], candidates: Iterable[dict] = DEFAUL
         for shape in stage or ():
             if all(base.get(k, _DEFAULTS.get(k)) == v for k, v in shape.items()):
                 continue  # already timed
+            if launched is not None and not any(c in launched(base) for k in shape for c in READ_BY.get(k, ())):
+                continue  # nothing that runs reads it
             run({**base, **shape})
     if key is not None:
         _cache[key] = dict(best)
