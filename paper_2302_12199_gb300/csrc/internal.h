@@ -135,7 +135,6 @@ struct CompactArgs {
 struct HookArgs {
   const uint32_t *cand;    // candidate vertices; nullptr = 0..ncand-1
   uint64_t ncand;
-  const u64 *ncand_dev;    // candidate count in device memory, or nullptr
   u64 *best;               // keys (see KeyLayout) of the round's minimum edges
   KeyLayout kl;
   const uint32_t *src, *dst;  // ends of each edge by id (unpacked keys): the input arrays,
@@ -166,10 +165,6 @@ inline int shape_index(uint32_t block_threads, uint32_t items_per_thread) {
 inline int relabel_shape_index(uint32_t block_threads, uint32_t items_per_thread) {
   return (block_threads == 0 && items_per_thread == 0) ? 1 : shape_index(block_threads, items_per_thread);
 }
-inline uint32_t shape_tile(int shape) {
-  static const uint32_t b[3] = {128, 256, 512}, i[3] = {4, 8, 16};
-  return shape <= 0 ? 2048u : b[(shape - 1) / 3] * i[(shape - 1) % 3];
-}
 
 // Counters the kernels that choose MSF edges add the chosen weights into, so
 // that the forest's total needs no gather of w at the end.
@@ -187,7 +182,7 @@ void launch_compact(CompactMode mode, const CompactArgs &a, uint64_t max_count, 
 void launch_min_edges(EdgeList in, uint64_t m, uint32_t n, int validate, KeyLayout kl, u64 *best, uint32_t *err,
                       int sms, cudaStream_t s, const uint32_t *max_w = nullptr);
 void launch_max_weight(const uint32_t *w, uint64_t m, uint32_t *out, int sms, cudaStream_t s);
-void launch_hook(const HookArgs &a, uint64_t max_cand, cudaStream_t s);
+void launch_hook(const HookArgs &a, cudaStream_t s);
 // max_steps: parent steps per thread and launch (0: the default of 64).
 // With act == count_dev == nullptr the launch covers every vertex
 // 0..count_host-1 and, given gbits, sets bit v of that bitmap iff v's walk

@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(B, Shape<B, I>::minb(PACKED ? Shape<B, I>::hoo
   __shared__ uint32_t s_warp[B / 32 + 1];
   __shared__ uint32_t s_base[1];
 
-  const uint64_t nc = a.ncand_dev ? *a.ncand_dev : a.ncand;
+  const uint64_t nc = a.ncand;
   const int wshift = PACKED ? a.kl.idbits + a.kl.vbits : 32;  // the weight's place in a key
   u64 wacc = 0;  // weights of the edges this thread chose
   for (uint64_t tile = blockIdx.x; tile * T < nc; tile += gridDim.x) {  // uniform per block
@@ -2691,12 +2691,9 @@ void launch_max_weight(const uint32_t *w, uint64_t m, uint32_t *out, int sms, cu
 }
 
 template <int B, int I>
-static void launch_hook_shaped(const HookArgs &a, uint64_t max_cand, cudaStream_t s) {
+static void launch_hook_shaped(const HookArgs &a, cudaStream_t s) {
   constexpr int T = B * I;
-  // a count known on the host gets one block per tile; a count in device
-  // memory (up to max_cand) gets a bounded grid that strides over the tiles
-  const uint64_t tiles = (max_cand + T - 1) / T;
-  const unsigned grid = (unsigned)(a.ncand_dev ? std::min<uint64_t>(tiles, 152u * 8u * 256u / B) : tiles);
+  const unsigned grid = (unsigned)((a.ncand + T - 1) / T);  // a block per tile
   // the packed layout needs no parent-chain walks: its own instantiation
   // keeps far fewer registers live (higher occupancy)
   if (a.cand)
@@ -2707,18 +2704,18 @@ static void launch_hook_shaped(const HookArgs &a, uint64_t max_cand, cudaStream_
                 : hook_kernel<true, false, B, I><<<grid, B, 0, s>>>(a);
 }
 
-void launch_hook(const HookArgs &a, uint64_t max_cand, cudaStream_t s) {
-  if (max_cand == 0) return;
+void launch_hook(const HookArgs &a, cudaStream_t s) {
+  if (a.ncand == 0) return;
   switch (a.shape) {  // the shapes of shape_index
-    case 1: launch_hook_shaped<128, 4>(a, max_cand, s); return;
-    case 2: launch_hook_shaped<128, 8>(a, max_cand, s); return;
-    case 3: launch_hook_shaped<128, 16>(a, max_cand, s); return;
-    case 4: launch_hook_shaped<256, 4>(a, max_cand, s); return;
-    case 6: launch_hook_shaped<256, 16>(a, max_cand, s); return;
-    case 7: launch_hook_shaped<512, 4>(a, max_cand, s); return;
-    case 8: launch_hook_shaped<512, 8>(a, max_cand, s); return;
-    case 9: launch_hook_shaped<512, 16>(a, max_cand, s); return;
-    default: launch_hook_shaped<BLOCK, ITEMS>(a, max_cand, s); return;  // 0 and 5: 256 x 8
+    case 1: launch_hook_shaped<128, 4>(a, s); return;
+    case 2: launch_hook_shaped<128, 8>(a, s); return;
+    case 3: launch_hook_shaped<128, 16>(a, s); return;
+    case 4: launch_hook_shaped<256, 4>(a, s); return;
+    case 6: launch_hook_shaped<256, 16>(a, s); return;
+    case 7: launch_hook_shaped<512, 4>(a, s); return;
+    case 8: launch_hook_shaped<512, 8>(a, s); return;
+    case 9: launch_hook_shaped<512, 16>(a, s); return;
+    default: launch_hook_shaped<BLOCK, ITEMS>(a, s); return;  // 0 and 5: 256 x 8
   }
 }
 

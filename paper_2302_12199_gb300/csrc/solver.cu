@@ -640,7 +640,7 @@ struct Solve {
     ha.counter = &c->ds->count[CNT_ACTIVE];
     ha.err = &c->ds->err;
     ha.wsum = c->wsum;
-    PROF(MST_K_HOOK, 8.0 * (double)n, CNT_ACTIVE, 8.0, -1, 0.0, launch_hook(ha, n, s));
+    PROF(MST_K_HOOK, 8.0 * (double)n, CNT_ACTIVE, 8.0, -1, 0.0, launch_hook(ha, s));
     TRY(jump_until_stars(act[0], &c->ds->count[CNT_ACTIVE], 0, n, 1, nullptr, nullptr, true));
     uint64_t n_act = c->hs->count[CNT_ACTIVE];
     ++rounds;
@@ -739,7 +739,7 @@ struct Solve {
       hb.counter = &c->ds->count[CNT_ACTIVE];
       hb.err = &c->ds->err;
       hb.wsum = c->wsum;
-      PROF(MST_K_HOOK, 12.0 * (double)n_act, CNT_ACTIVE, 8.0, -1, 0.0, launch_hook(hb, n_act, s));
+      PROF(MST_K_HOOK, 12.0 * (double)n_act, CNT_ACTIVE, 8.0, -1, 0.0, launch_hook(hb, s));
       TRY(jump_until_stars(act[1 - a], &c->ds->count[CNT_ACTIVE], 0, n_act, 1, nullptr, nullptr, true));
       table_b.release();
       a = 1 - a;
@@ -2463,7 +2463,7 @@ mst_status mst_step_contract(mst_handle h, uint32_t n, uint64_t m, const uint32_
   ha.counter = &h->ds->count[CNT_ACTIVE];
   ha.err = &h->ds->err;
   ha.wsum = h->wsum;
-  launch_hook(ha, n, s);
+  launch_hook(ha, s);
   return record(h, S.jump_until_stars(S.act[0], &h->ds->count[CNT_ACTIVE], 0, n, 1));
 }
 
