@@ -72,10 +72,10 @@ WORKLOADS = {
 TRAFFIC = {
     "class": "filter",
     "kernel": "stream_warp_kernel<CM_FILTER>",
-    "dram_per_algorithmic_byte": 1.352,
+    "dram_per_algorithmic_byte": 1.351,
     "measured_on": "RMAT n=2^22 m=2^26, both filter launches of one timed solve (pivot quantile 1/8)",
     "pivot_quantile": 0.125,
-    "source_sha256": "a90ad8de4d5004aeb0ae6e62c8b2c6004d9762fb0085350b95469a5fbad917b5",
+    "source_sha256": "0b0bca98017819e433be723510190736b0992e94a78759ff6e8a8e55b2a029de",
 }
 TRAFFIC_SOURCE = (
     ("paper_2302_12199_gb300/csrc/kernels.cu", "__device__ __forceinline__ uint32_t keep_flags",

@@ -18,16 +18,19 @@
  * aligned; 16-byte alignment enables vector loads.  The library allocates its
  * own scratch memory (stream-ordered) and frees it when the handle is destroyed.
  *
- * Streams: `stream` is a cudaStream_t (NULL = the legacy default stream).  All
- * of a call's device work is issued on that stream, after the work the caller
- * queued on it before the call.  A call returns once its results are written:
+ * Streams: `stream` is a cudaStream_t (NULL = the legacy default stream).  A
+ * call's device work runs after the work the caller queued on that stream before
+ * the call, and the stream waits for all of it: a batch runs parts of its work on
+ * two streams of the handle, and mst_solve_host_many its copies on another, which
+ * are joined before the call returns.  A call returns once its results are written:
  * the Filter-Borůvka recursion is planned from a count that the host reads
  * back on that stream, and the final status is read back, so a solve is
  * stream-ordered but not asynchronous to the host.  A
  * handle must not be used by two host threads at once; different handles may
  * solve at the same time from different threads (each on its own stream): a
  * solve grows its buffers in stream order and never waits for the whole
- * device.  mst_create and mst_destroy do wait for the device, so create and
+ * device (some of its kernels need all of their blocks resident, so solves on
+ * several streams take turns at those).  mst_create and mst_destroy do wait for the device, so create and
  * destroy handles while no other thread is capturing a CUDA graph.
  *
  * Errors: every call returns an mst_status.  Errors detected on the device
@@ -72,12 +75,19 @@ typedef struct {
   uint64_t seed;               /* seed of the pivot sampling stream */
   uint64_t filter_min_edges;   /* isSparse: lists shorter than this are not partitioned */
   float filter_max_avg_degree; /* isSparse: stop partitioning at average degree 2m/n <= this (the paper's
-                                  Section 6.3 uses 4; the default 1.25 is measured on GB300, where the range
-                                  0.75-2.5 is flat with the default pivot quantile) */
-  int base_case;               /* 1 (default): once a Borůvka call's live components (<= 4096) and
-                                  edges (<= 6144) fit one block's shared memory, finish its rounds in
-                                  one launch (the role of the paper's base case, Section 4.4); 0: run
-                                  every round globally */
+                                  Section 6.3 uses 4; the default 1.25 is measured on GB300 with median
+                                  pivots.  With the default pivot quantile the lists of RMAT n=2^24 m=2^28
+                                  have average degrees 32, 4 and 0.5, so every bound from 0.5 to 4 gives
+                                  the same recursion there) */
+  int base_case;               /* 1 (default): one block solves a small graph (the role of the paper's
+                                  base case, Section 4.4): a graph of at most 12288 vertices and 32768
+                                  edges alone; in a batch, graphs of at most 65536 vertices that a block
+                                  solves no later than the batch's union would be.  The variant, pivot,
+                                  filter, jump and tile-shape options have no effect there (the forest is
+                                  the same).  Not with graph_rounds = 0, local contraction, sorted
+                                  minEdges, or hash or sort dedupe.  With graph_rounds = 0: once a Borůvka
+                                  call's live components (<= 4096) and edges (<= 6144) fit one block's
+                                  shared memory, its rounds finish in one launch.  0: neither */
   int graph_rounds;            /* 1 (default): the rounds of a Borůvka call run in one cooperative launch
                                   that the device ends (no host round trip per round; not with hash or
                                   sort dedupe, nor for n >= 2^31); 0: one host readback per round */
@@ -212,8 +222,10 @@ mst_status mst_solve_host_many(mst_handle h, uint32_t count, mst_host_graph *gra
 /* Minimum spanning forests of G independent graphs in one solve (each graph
  * the Section 2.2 problem).  Graph g has d_n[g] vertices (graph-local ids
  * 0..d_n[g]-1) and the edges d_edge_off[g] .. d_edge_off[g+1]-1 of
- * d_src/d_dst/d_w.  The graphs are solved together as one disjoint union, so
- * their rounds share launches.
+ * d_src/d_dst/d_w.  Graphs that fit one are solved by a block each
+ * (mst_config.base_case), when they hold at least half of the edges and a block
+ * takes no longer than the union would; the others are solved together as one
+ * disjoint union, so that their rounds share launches.
  *   d_n         [G] uint32 vertex counts, device memory
  *   d_edge_off  [G+1] uint64 edge offsets, device memory; d_edge_off[0] == 0,
  *               non-decreasing (else MST_ERR_INVALID_ARG); d_edge_off[G] = m
@@ -224,7 +236,8 @@ mst_status mst_solve_host_many(mst_handle h, uint32_t count, mst_host_graph *gra
  *   d_total_weight [out] [G] uint64 MSF weight of each graph
  * The totals (all vertices, all edges) are read back from the device tables
  * before the solve is sized.  MST_ERR_TOO_LARGE if either reaches 2^32.
- * Errors as mst_solve; a vertex id out of range in any graph fails the call. */
+ * Errors as mst_solve; a vertex id out of range in any graph fails the call, and
+ * arrays that are not 4-byte aligned are MST_ERR_INVALID_ARG. */
 mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *d_n, const uint64_t *d_edge_off,
                              const uint32_t *d_src, const uint32_t *d_dst, const uint32_t *d_w, uint32_t *d_msf_ids,
                              uint64_t *d_msf_off, uint64_t *d_total_weight, void *stream);
@@ -236,16 +249,18 @@ mst_status mst_solve_batched(mst_handle h, uint32_t num_graphs, const uint32_t *
  * probes are not counted) are accumulated per class until reset. */
 enum {
   MST_K_MIN_EDGES = 0,  /* minEdges from a stored list (first round of a Borůvka call) */
-  MST_K_RELABEL_MIN,    /* relabel + self-loop removal + compaction, fused with the next minEdges */
-  MST_K_HOOK,           /* hooking + active-vertex compaction */
-  MST_K_JUMP,           /* pointer doubling */
+  MST_K_RELABEL_MIN,    /* relabel + self-loop removal + compaction, fused with the next minEdges (the same,
+                           and after local contraction) */
+  MST_K_HOOK,           /* hooking + active-vertex compaction (rounds the host drives) */
+  MST_K_JUMP,           /* pointer doubling (the same, and over all vertices before a filter) */
   MST_K_DEDUPE,         /* hash parallel-edge removal (insert and keep passes) */
   MST_K_PIVOT,          /* pivot sampling and selection */
   MST_K_PARTITION,      /* light/heavy partition */
   MST_K_FILTER,         /* filtering of heavy edges */
   MST_K_FINALIZE,       /* bitmap -> ascending ids + weight */
   MST_K_TILE,           /* tile-local contraction (count, bucket, contract) */
-  MST_K_BASE,           /* single-block base case (the last rounds of a Borůvka call) */
+  MST_K_BASE,           /* graphs solved by one block each, and the single-block base case of rounds the
+                           host drives (the last rounds of a Borůvka call) */
   MST_K_GRAPH,          /* Borůvka rounds run as one launch (time only; bytes not counted) */
   MST_K_COUNT
 };

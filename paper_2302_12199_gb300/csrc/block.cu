@@ -18,7 +18,8 @@
 // where the graph's weights allow (w <= 255 and up to 2^22 edges), else 64.
 //
 // GB300, 4096 graphs of 2^8 to 2^16 vertices (337 M edges): 12.1 ms as a union,
-// 5.5 ms here, of which 0.14 ms for the ids.  What bounds it is latency between
+// 5.1 to 5.7 ms here (runs of the same code differ by that much), of which 0.14
+// ms for the ids.  What bounds it is latency between
 // barriers with one or two graphs per SM: half of the issue slots and half of
 // L1's throughput are used (ncu, 224 KB blocks).  An edge's record is one
 // 16-byte store and a live edge 8 bytes (three arrays: 5.63 ms); separate warps'

@@ -288,9 +288,11 @@ __device__ __forceinline__ void hook_phase(const RoundsArgs &a, const KeyLayout 
 // The same for a short pass (rounds of few components, small calls): a lane per
 // vertex, and no block barriers; the GROUP warps of a group claim their roots'
 // ids, and in round 0 places in `act`, together.  A chain of L2 round trips
-// between two grid barriers: 3.4 us per round of GNM n=2^16 m=2^20 where the
-// tiles of the long pass took 4.7; 10.5 instead of 15.6 with 540,969 components.
-// Sparse first rounds need the tiles (RMAT n=2^24: 72 us, a lane per vertex 370).
+// between two grid barriers: 3.1 to 5.2 us a pass in GNM n=2^16 m=2^20, 21 with
+// 541,226 components.  Against the tiles of the long pass, whole solves: that GNM
+// 208 -> 204 us, RGG3D n=2^21 596 -> 586, grid 2048 x 2048 582 -> 572.  Sparse
+// first rounds need the tiles (RMAT n=2^24: about 95 us, a lane per vertex four
+// to five times that).
 __device__ __forceinline__ void hook_short(const RoundsArgs &a, const KeyLayout &kl, int r, uint64_t nc, uint64_t off,
                                            bool rec, uint32_t nb, uint32_t bid, Smem &sm) {
   uint32_t *link = r == 0 ? a.parent : a.link + off;
@@ -397,12 +399,13 @@ __device__ __forceinline__ void jump_phase(const RoundsArgs &a, int r, uint64_t 
 // atomic, and write them from registers (a store's lanes are dense).  `tab`:
 // collect the minima in shared memory first.  Bound by the label and best[]
 // gathers, four per edge, which warps that wait for no more than their group
-// keep coming: with whole blocks passing from load to gather to a staged store
-// behind barriers, RMAT n=2^22 m=2^26 took 1180 and 840 us for its first two
-// relabels (905 and 610 now, 296 G gathers/s), RGG2D n=2^22 200 and 112 (155 and
-// 92), GNM n=2^16 m=2^20 14.0 (7.5).  A claim per warp queues at the counter
-// and scatters neighbours over the next list (1040, 707; 169, 119); groups of
-// eight wait longer (942, 639; 165, 104).
+// keep coming.  Its first two passes take 1040 and 673 us in RMAT n=2^22 m=2^26
+// (254 and 383 G gathers/s), 207 and 128 in RGG2D n=2^22, 33 and 16 in GNM n=2^16
+// m=2^20.  Whole solves, with whole blocks passing from load to gather to a staged
+// store behind barriers: that RMAT 3.23 ms (now 2.88), that RGG2D 997 us (936),
+// that GNM 233 (229).  A claim per warp queues at the counter and scatters
+// neighbours over the next list (the RMAT's first two passes a seventh longer);
+// groups of eight wait longer (a twentieth).
 template <int I>
 __device__ __forceinline__ void relabel_phase(const RoundsArgs &a, KeyLayout kl, int r, uint64_t m, uint64_t off,
                                                bool tab, uint32_t nb, uint32_t bid, Smem &sm) {
@@ -494,9 +497,9 @@ __device__ __noinline__ void pair_clear(uint32_t *table_mem, uint32_t np, uint32
 // sends them to the table; nothing is staged or written per edge, and an edge's
 // id is read only where its weight is not above the pair's minimum.  Bound by
 // reading 12 bytes per edge: RMAT n=2^22 m=2^26, which keeps 64 million edges
-// until its last rounds, passes over them in 227 us (3.4 TB/s; the shared-memory
-// lookups are the rest), where relabel, minEdges and three more rounds took
-// 1260 us.  The pair functions
+// until its last rounds, passes over them in 241 us (3.2 TB/s; the shared-memory
+// lookups are the rest); relabel, minEdges and three more rounds in its place made
+// the solve 4.1 ms instead of 3.4.  The pair functions
 // are calls, with their arguments by value: inlined, their registers cost the
 // long phases spills (RGG2D's first relabel 200 -> 223 us).
 template <int I>
@@ -569,8 +572,9 @@ __device__ __noinline__ void pair_phase(EdgeList in, const uint32_t *link, uint6
 
 // The call's last rounds over the table of pairs, in one block's shared memory:
 // a warp looks through a component's row, and everything else is one thread per
-// component: about 2 us a round, where writing the pairs as a list took 9 and
-// each round over it 7 (GNM n=2^16 m=2^20, 108 components left: 229 -> 204 us).
+// component: 17 us for all of them in GNM n=2^16 m=2^20 (108 components left); with
+// the pairs written as a list, and rounds over that, the solve took 229 us instead
+// of 204.
 // rep: representatives of the nn components, replaced by those of their final
 // ones; or nullptr.
 __device__ __noinline__ void pair_rounds(const uint32_t *table_mem, uint32_t nn, uint32_t *chosen_bits, u64 *wsum,

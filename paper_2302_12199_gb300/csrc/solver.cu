@@ -1,6 +1,7 @@
 // Host side of libmstgpu: the C ABI declared in include/mst.h, the Borůvka
 // round loop (Section 2.3, Alg. 1), the Filter-Borůvka recursion (Alg. 2), the
-// batched disjoint-union solve and the step entry points.
+// batched solve (a block per graph, the rest as a disjoint union) and the step
+// entry points.
 //
 // Device memory: each handle owns a CUDA memory pool; every solve allocates its
 // scratch from it in stream order and returns it at the end, so repeated solves
@@ -71,7 +72,7 @@ struct mst_ctx {
   // kept by the handle and grown on demand
   void *rl_mem = nullptr;
   uint64_t rl_cap = 0;  // edges per list
-  void *small_mem = nullptr;      // scratch of graphs that one block solves (SmallScratch)
+  void *small_mem = nullptr;      // scratch of a graph that one block solves (SMALL_BYTES)
   cudaStream_t kind_stream[2] = {nullptr, nullptr};  // block solves of the middle and the small graphs of a batch
   cudaEvent_t kind_ev[3] = {nullptr, nullptr, nullptr};
   RoundsState *rstate = nullptr;  // device states of the one-launch rounds, one per launch of a solve

@@ -4,10 +4,10 @@ Requests (independent graphs of different sizes) arrive over time.  The loop
 batches them as they arrive: whenever a solver slot is free it takes the
 waiting requests, oldest first, up to a device-memory budget per slot
 (admission by footprint, from mst_workspace_bytes plus the batch's own
-arrays), and solves them with one mst_solve_batched call, in which all graphs
-of the batch share every round's launches (the disjoint union of the graphs;
-its MSF is the union of their MSFs, each the unique one under the graphs' own
-(w, id) order).  Several slots, each with its own solver handle, CUDA stream
+arrays), and solves them with one mst_solve_batched call: a block per graph
+where that is no slower, the other graphs sharing every round's launches as a
+disjoint union (its MSF is the union of their MSFs, each the unique one under
+the graphs' own (w, id) order).  Several slots, each with its own solver handle, CUDA stream
 and host thread, keep batches in flight at once, so requests that arrive while
 others run on the GPU start as soon as a slot and memory free up, and their
 work overlaps on the device.
