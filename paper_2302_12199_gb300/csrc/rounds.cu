@@ -353,10 +353,9 @@ __device__ __forceinline__ void hook_short(const RoundsArgs &a, const KeyLayout 
 // multiplies every vertex's reach by at least RSTEPS + 1, so long chains want
 // several short passes, and the trees of other graphs are less deep.  `flag` is
 // raised once per warp at most, and not where it is up already: raised by every
-// thread, its atomics queued at one word for most of a pass.  Plain solves of a
-// path with ascending weights, n=2^20 and 2^24: 432 and 3920 us with 256 steps
-// and a flag per thread, 345 and 3780 with 256 steps, 257 and 2040 with 64, 211
-// and 2020 with 32.
+// thread, its atomics queued at one word for most of a pass.  Plain solve of 16
+// paths of 2^16 vertices with ascending weights, joined end to end: 388 us with
+// 256 steps and a flag per thread, 319 with 256 steps, 226 with 64, 192 with 32.
 __device__ __forceinline__ void jump_phase(const RoundsArgs &a, int r, uint64_t cnt, uint64_t off, bool reset,
                                         uint32_t *flag, uint32_t nb, uint32_t bid) {
   uint32_t *link = r == 0 ? a.parent : a.link + off;
